@@ -210,22 +210,19 @@ struct IluEll {
     void *lval = nullptr, *uval = nullptr, *udinv = nullptr;
 };
 
-// ILU(0) factors in the line-block order (see ilu_lines.cu): positions by
-// colour, block, line, x; per colour the parallel parts of L and U as ELL
-// blocks (columns as positions), per position the line recurrence
-// coefficients and 1 / u_pp.
+// ILU(0) factors in the line-block order: positions by colour, block, line,
+// x; the coefficients by neighbour line and x offset (see ilu_lines.cu).
+// Index 0: L (earlier in the order), 1: U.
 struct IluLines {
     int nx = 0, ncol = 0;
     int cptr[5] = {0};  // first position of each colour (+ end)
     int bptr[5] = {0};  // first block of each colour (+ end)
-    int wl[4] = {0}, wu[4] = {0};    // off-block entries per point, per colour
-    int wli[4] = {0}, wui[4] = {0};  // in-block entries (the block's other lines) per point
-    long lbase[4] = {0}, ubase[4] = {0}, libase[4] = {0}, uibase[4] = {0};
-    int32_t *rows = nullptr, *blk_start = nullptr, *blk_nsub = nullptr;
-    int32_t *lcol = nullptr, *ucol = nullptr;  // off-block columns (positions)
-    int16_t *lidx = nullptr, *uidx = nullptr;  // in-block entries: index inside the block
-    void *lval = nullptr, *uval = nullptr, *lvin = nullptr, *uvin = nullptr;
-    void *lrec = nullptr, *urec = nullptr, *udinv = nullptr;
+    int noff[2][4] = {{0}};    // neighbour lines in other blocks, per colour
+    long obase[2][4] = {{0}};  // first off-block coefficient of each colour
+    int32_t *rows = nullptr, *blk_line = nullptr, *blk_nsub = nullptr;
+    int32_t *nbr = nullptr;                    // first positions of the neighbour lines
+    void *off[2] = {nullptr, nullptr};  // off-block coefficients
+    void *in[2] = {nullptr, nullptr};   // line recurrence, 1 / u_pp, the block's other lines
 };
 
 // ---- device helpers -------------------------------------------------------

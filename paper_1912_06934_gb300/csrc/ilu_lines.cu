@@ -19,7 +19,10 @@
 // per block, one warp per line, on a wavefront: line q trails line q-1 by two
 // points, since (x, q) needs (x+1, q-1).
 #include "common.cuh"
+#include "lines.cuh"
 #include <climits>
+#include <cstring>
+#include <type_traits>
 #include <vector>
 #include <cub/device/device_radix_sort.cuh>
 
@@ -287,404 +290,106 @@ __global__ void __launch_bounds__(128) lines_factor_ring_kernel(
 
 // ---- factors for the sweeps -------------------------------------------------------------
 //
-// Per position p (the order above) the earlier entries split three ways: the
-// line predecessor (x-1, same line): lrec[p]; entries of the block's earlier
-// lines: an in-block ELL block of its colour (index of the column inside the
-// block, value); all others (earlier colours): an off-block ELL block
-// (columns as positions). The later entries likewise (urec towards
-// (x+1, same line)); udinv[p] = 1 / u_pp.
-
-// first position of the block of row i and whether row k is in that block
-__device__ __forceinline__ bool same_block(int i, int k, int nx, int ny) {
-    const int yi = (i / nx) % ny, zi = i / (nx * ny), yk = (k / nx) % ny, zk = k / (nx * ny);
-    return (yi >> 1) == (yk >> 1) && (zi >> 1) == (zk >> 1);
-}
-__device__ __forceinline__ int block_first_row(int i, int nx, int ny) {
-    const int y = (i / nx) % ny, z = i / (nx * ny);
-    return nx * ((y & ~1) + ny * (z & ~1));
-}
-
-// Per colour, the widest row of each of the four parts (off-block / in-block,
-// lower / upper): a maximum in shared memory per CTA, then one global atomic
-// per part and colour.
-__global__ void __launch_bounds__(256) lines_width_kernel(int n, int nx, int ny, const int32_t *__restrict__ rowptr,
-                                                          const int32_t *__restrict__ colidx,
-                                                          const int32_t *__restrict__ pos,
-                                                          const int32_t *__restrict__ ccol, int *__restrict__ w) {
-    __shared__ int s_w[16];
-    if (threadIdx.x < 16) s_w[threadIdx.x] = 0;
-    __syncthreads();
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) {
-        const int p = pos[i], x = i % nx;
-        int nl = 0, nu = 0, nli = 0, nui = 0;
-        for (int e = rowptr[i]; e < rowptr[i + 1]; ++e) {
-            const int k = colidx[e], pk = pos[k];
-            if (pk < p && !(k == i - 1 && x > 0)) {
-                if (same_block(i, k, nx, ny)) ++nli;
-                else ++nl;
-            }
-            if (pk > p && !(k == i + 1 && x < nx - 1)) {
-                if (same_block(i, k, nx, ny)) ++nui;
-                else ++nu;
-            }
+// A's pattern lies in the 3^dim neighbourhood, so a point's entries fall on at
+// most 8 neighbour lines of 3 points each and on its own line, and the line
+// (the same for every point of a line) says which block it belongs to. The
+// factors are therefore stored by neighbour line and x offset, zeros where the
+// pattern has no entry, without column indices: half the bytes of column and
+// value pairs, read as 16-byte vectors.
+//  - off-block: up to 5 neighbour lines lie in other blocks (per axis one of
+//    the two neighbours); by the colours' order, colour c has noff[0][c]
+//    lines of earlier and noff[1][c] of later colours. nbr[dir][line][5] holds
+//    the first position of each (ascending in z, then y); off[dir] their
+//    coefficients.
+//  - in-block: the block's other lines; in[0] of a point of line q holds
+//    (l to x-1 on its own line, then 3 per earlier line of the block), in[1]
+//    (u to x+1, 1 / u_pp, then 3 per later line).
+// Group g (kLineGroup<T> values, 16 bytes) of point x of a line sits at
+// (line * groups + g) * nx + x, so a warp reads consecutive vectors. Every
+// line keeps room for its widest in-block record; groups past a line's own
+// count are never read.
+// nbr[dir][line][5] (dir 0: lines of earlier colours, 1: of later ones), the
+// line's own first position where there is no such line
+__global__ void lines_nbr_kernel(int nlines, int dim, int nx, int ny, int nz, const int32_t *__restrict__ rows,
+                                 const int32_t *__restrict__ pos, int32_t *__restrict__ nbr) {
+    const int l = blockIdx.x * blockDim.x + threadIdx.x;
+    if (l >= nlines) return;
+    const int i = rows[l * nx], y = (i / nx) % ny, z = dim == 3 ? i / (nx * ny) : 0;
+    const int c = ((y >> 1) & 1) | (dim == 3 ? ((z >> 1) & 1) << 1 : 0);
+    int cnt[2] = {0, 0};
+    for (int dz = dim == 3 ? -1 : 0; dz <= (dim == 3 ? 1 : 0); ++dz)
+        for (int dy = -1; dy <= 1; ++dy) {
+            const int yk = y + dy, zk = z + dz;
+            if (yk < 0 || yk >= ny || zk < 0 || zk >= nz) continue;
+            if ((yk >> 1) == (y >> 1) && (zk >> 1) == (z >> 1)) continue;
+            const int ck = ((yk >> 1) & 1) | (dim == 3 ? ((zk >> 1) & 1) << 1 : 0);
+            const int d = ck < c ? 0 : 1;  // blocks of one colour are not neighbours
+            nbr[((long)d * nlines + l) * kLineNbr + cnt[d]++] = pos[nx * (yk + (long)ny * zk)];
         }
-        const int c = ccol[i];
-        atomicMax(s_w + c, nl);
-        atomicMax(s_w + 4 + c, nu);
-        atomicMax(s_w + 8 + c, nli);
-        atomicMax(s_w + 12 + c, nui);
-    }
-    __syncthreads();
-    if (threadIdx.x < 16 && s_w[threadIdx.x] > 0) atomicMax(w + threadIdx.x, s_w[threadIdx.x]);
+    for (int d = 0; d < 2; ++d)
+        for (int k = cnt[d]; k < kLineNbr; ++k) nbr[((long)d * nlines + l) * kLineNbr + k] = l * nx;
 }
 
 template <typename T>
-__global__ void lines_fill_kernel(int n, int nx, int ny, const int32_t *__restrict__ rowptr,
-                                  const int32_t *__restrict__ colidx, const T *__restrict__ lu,
-                                  const int32_t *__restrict__ dpos, const int32_t *__restrict__ pos,
-                                  const int32_t *__restrict__ ccol, const IluLines L, T *__restrict__ lval,
-                                  T *__restrict__ uval, T *__restrict__ lvin, T *__restrict__ uvin,
-                                  T *__restrict__ lrec, T *__restrict__ urec, T *__restrict__ udinv) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const int c = ccol[i], p = pos[i], x = i % nx;
-    const int r = p - L.cptr[c], m = L.cptr[c + 1] - L.cptr[c];
-    const int bst = pos[block_first_row(i, nx, ny)];
-    const long lb = L.lbase[c], ub = L.ubase[c], lib = L.libase[c], uib = L.uibase[c];
-    int nl = 0, nu = 0, nli = 0, nui = 0;
-    T lr = T(0), ur = T(0);
-    for (int e = rowptr[i]; e < rowptr[i + 1]; ++e) {
-        const int k = colidx[e], pk = pos[k];
-        const bool inb = same_block(i, k, nx, ny);
-        if (pk < p) {
-            if (k == i - 1 && x > 0) {
-                lr = lu[e];
-            } else if (inb) {
-                L.lidx[lib + (long)nli * m + r] = (int16_t)(pk - bst);
-                lvin[lib + (long)nli * m + r] = lu[e];
-                ++nli;
-            } else {
-                L.lcol[lb + (long)nl * m + r] = pk;
-                lval[lb + (long)nl * m + r] = lu[e];
-                ++nl;
-            }
-        } else if (pk > p) {
-            if (k == i + 1 && x < nx - 1) {
-                ur = lu[e];
-            } else if (inb) {
-                L.uidx[uib + (long)nui * m + r] = (int16_t)(pk - bst);
-                uvin[uib + (long)nui * m + r] = lu[e];
-                ++nui;
-            } else {
-                L.ucol[ub + (long)nu * m + r] = pk;
-                uval[ub + (long)nu * m + r] = lu[e];
-                ++nu;
-            }
-        }
-    }
-    // padding: value 0 at the point itself (read, multiplied by 0)
-    for (; nl < L.wl[c]; ++nl) {
-        L.lcol[lb + (long)nl * m + r] = p;
-        lval[lb + (long)nl * m + r] = T(0);
-    }
-    for (; nu < L.wu[c]; ++nu) {
-        L.ucol[ub + (long)nu * m + r] = p;
-        uval[ub + (long)nu * m + r] = T(0);
-    }
-    for (; nli < L.wli[c]; ++nli) {
-        L.lidx[lib + (long)nli * m + r] = (int16_t)(p - bst);
-        lvin[lib + (long)nli * m + r] = T(0);
-    }
-    for (; nui < L.wui[c]; ++nui) {
-        L.uidx[uib + (long)nui * m + r] = (int16_t)(p - bst);
-        uvin[uib + (long)nui * m + r] = T(0);
-    }
-    lrec[p] = lr;
-    urec[p] = ur;
-    udinv[p] = T(1) / lu[dpos[i]];
-}
-
-__global__ void lines_colour_of_kernel(int n, const int32_t *__restrict__ rows, const IluLines L,
-                                       int32_t *__restrict__ ccol) {
+__global__ void __launch_bounds__(128) lines_fill_kernel(int n, int dim, int nx, int ny, int nz,
+                                                         const int32_t *__restrict__ rowptr,
+                                                         const uint32_t *__restrict__ rmask,
+                                                         const T *__restrict__ lu, const int32_t *__restrict__ rows,
+                                                         const IluLines L, T *__restrict__ offl, T *__restrict__ offu,
+                                                         T *__restrict__ inl, T *__restrict__ inu) {
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= n) return;
-    int c = 0;
-    while (c + 1 < L.ncol && p >= L.cptr[c + 1]) ++c;
-    ccol[rows[p]] = c;
-}
-
-// ---- sweeps ---------------------------------------------------------------------------------
-
-// one step of an affine warp scan: (A, B) represents y_out = A + B y_in; the
-// inclusive scan composes lane 0's map first
-template <typename T>
-__device__ __forceinline__ void affine_scan(T &A, T &B, int lane) {
+    const int i = rows[p], x = i % nx, y = (i / nx) % ny, z = dim == 3 ? i / (nx * ny) : 0;
+    const int c = ((y >> 1) & 1) | (dim == 3 ? ((z >> 1) & 1) << 1 : 0);
+    const int sy = min(2, ny - (y & ~1)), q = (y & 1) + (z & 1) * sy;
+    T off[2][kLineOff], in[2][kLineIn];
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const T Ap = __shfl_up_sync(0xffffffffu, A, o), Bp = __shfl_up_sync(0xffffffffu, B, o);
-        if (lane >= o) {
-            A = fma(B, Ap, A);
-            B = B * Bp;
+    for (int k = 0; k < kLineOff; ++k) off[0][k] = off[1][k] = T(0);
+#pragma unroll
+    for (int k = 0; k < kLineIn; ++k) in[0][k] = in[1][k] = T(0);
+    const uint32_t mask = rmask[i];
+    int e = rowptr[i], cnt[2] = {0, 0};
+    for (int o = 0; o < (dim == 3 ? 27 : 18); o += 3) {  // entries in column order, three x offsets at a time
+        const int dy = (o / 3) % 3 - 1, dz = dim == 3 ? o / 9 - 1 : 0;
+        if (dim != 3 && o < 9) continue;  // 2D rows use the bits of dz = 0
+        const uint32_t m3 = (mask >> o) & 7u;
+        const int yk = y + dy, zk = z + dz;
+        if (yk < 0 || yk >= ny || zk < 0 || zk >= nz) continue;
+        T v[3];
+#pragma unroll
+        for (int d = 0; d < 3; ++d) v[d] = (m3 >> d) & 1u ? lu[e + __popc(m3 & ((1u << d) - 1u))] : T(0);
+        e += __popc(m3);
+        if (dy == 0 && dz == 0) {
+            in[0][0] = v[0];
+            in[1][0] = v[2];
+            in[1][1] = T(1) / v[1];
+        } else if ((yk >> 1) == (y >> 1) && (zk >> 1) == (z >> 1)) {
+            const int qk = (yk & 1) + (zk & 1) * sy;
+            T *dst = qk < q ? in[0] + 1 + 3 * qk : in[1] + 2 + 3 * (qk - q - 1);
+#pragma unroll
+            for (int d = 0; d < 3; ++d) dst[d] = v[d];
+        } else {
+            const int ck = ((yk >> 1) & 1) | (dim == 3 ? ((zk >> 1) & 1) << 1 : 0);
+            const int dir = ck < c ? 0 : 1;
+            T *dst = off[dir] + 3 * cnt[dir]++;
+#pragma unroll
+            for (int d = 0; d < 3; ++d) dst[d] = v[d];
         }
     }
-}
-
-// The recurrence v_k = a_k + b_k v_{k-1}, v_-1 = 0, along one line (k in
-// processing order, the lanes of the line's warps in k order), two-level: an
-// affine warp scan, then the composed maps of the line's earlier warps (wl
-// of them, through wA / wB in shared memory) applied as the carry. Every
-// thread of the CTA calls it (threads off the line pass the identity map
-// a = 0, b = 1), so the barrier inside is reached by all. Returns v_k.
-template <typename T>
-__device__ __forceinline__ T cta_line_scan(T a, T b, int lane, int wl, T *wA, T *wB) {
-    T A = a, B = b;
-    affine_scan(A, B, lane);  // now v_k = A + B v_{-1 of this warp}
-    if (lane == 31) {
-        wA[threadIdx.x >> 5] = A;
-        wB[threadIdx.x >> 5] = B;
-    }
-    __syncthreads();
-    T carry = T(0);  // v just before this warp
-    const int w = threadIdx.x >> 5;
-    for (int u = w - wl; u < w; ++u) carry = fma(wB[u], carry, wA[u]);
-    return fma(B, carry, A);
-}
-
-// In-block coefficients a thread keeps in registers (9 per direction for a
-// 27-point pattern); wider patterns read the rest from global memory.
-constexpr int kLinesInReg = 9;
-
-template <typename T>
-struct LineCoef {
-    T v[kLinesInReg];
-    int16_t ix[kLinesInReg];
-    T rec, d;
-};
-
-// The in-block coefficients of point li of the block (set-up data, so they
-// may be read before the wait on the preceding kernel).
-template <typename T>
-__device__ __forceinline__ void line_coef_load(LineCoef<T> &cf, bool on, int li, int st, int c0, int m, int w,
-                                               const int16_t *__restrict__ ix, const T *__restrict__ v,
-                                               const T *__restrict__ rec, const T *__restrict__ dinv) {
-    const int r = st + li - c0;
-#pragma unroll
-    for (int j = 0; j < kLinesInReg; ++j) {
-        const bool has = on && j < w;
-        cf.v[j] = has ? v[(long)j * m + r] : T(0);
-        cf.ix[j] = has ? ix[(long)j * m + r] : int16_t(0);
-    }
-    cf.rec = on ? rec[st + li] : T(0);
-    cf.d = on && dinv ? dinv[st + li] : T(1);
-}
-
-// sm[li] - sum_in coef * sm[idx] for the point of cf
-template <typename T>
-__device__ __forceinline__ T line_in_sum(const LineCoef<T> &cf, const T *sm, int li, int st, int c0, int m, int w,
-                                         const int16_t *__restrict__ ix, const T *__restrict__ v) {
-    T acc = sm[li];
-#pragma unroll
-    for (int j = 0; j < kLinesInReg; ++j) acc = fma(-cf.v[j], sm[cf.ix[j]], acc);
-    const int r = st + li - c0;
-    for (int j = kLinesInReg; j < w; ++j) acc = fma(-v[(long)j * m + r], sm[ix[(long)j * m + r]], acc);
-    return acc;
-}
-
-// mode 0: forward over the block's lines; 1: backward; 2: forward then
-// backward (the last colour). One CTA per block, one thread per point: line q
-// is held by threads q * nxp ... q * nxp + nx - 1 (nxp = nx rounded up to a
-// whole warp), the block's values in shared memory. The contributions from
-// other blocks are gathered by every point at once; the lines then follow in
-// turn, each a scan over its threads, with each thread's in-block
-// coefficients already in registers.
-template <typename T, typename TZ>
-__global__ void __launch_bounds__(1024) lines_sweep_kernel(
-    int mode, int b0, const int32_t *__restrict__ blk_start, const int32_t *__restrict__ blk_nsub, int nx, int nxp,
-    int c0, int m, int wl, const int32_t *__restrict__ lcol, const T *__restrict__ lval, int wli,
-    const int16_t *__restrict__ lidx, const T *__restrict__ lvin, const T *__restrict__ lrec, int wu,
-    const int32_t *__restrict__ ucol, const T *__restrict__ uval, int wui, const int16_t *__restrict__ uidx,
-    const T *__restrict__ uvin, const T *__restrict__ urec, const T *__restrict__ udinv,
-    const int32_t *__restrict__ rows, T *__restrict__ y, TZ *__restrict__ z) {
-    extern __shared__ unsigned char s_raw[];
-    T *sm = reinterpret_cast<T *>(s_raw);  // [4 * nx]
-    T *wA = sm + 4 * nx, *wB = wA + 32;    // composed maps of the warps
-    const int b = b0 + blockIdx.x;
-    const int st = blk_start[b], nsub = blk_nsub[b];
-    const int q = threadIdx.x / nxp, xx = threadIdx.x - q * nxp, lane = threadIdx.x & 31;
-    const int wline = xx >> 5;  // this warp's place in its line
-    const bool on = q < nsub && xx < nx;
-    const int lf = q * nx + xx;           // the point of the forward sweep
-    const int lb = q * nx + (nx - 1 - xx);  // the point of the backward sweep (from the line's end)
-    LineCoef<T> cf;
-    if (mode != 1)
-        line_coef_load(cf, on, lf, st, c0, m, wli, lidx, lvin, lrec, (const T *)nullptr);
-    else
-        line_coef_load(cf, on, lb, st, c0, m, wui, uidx, uvin, urec, udinv);
-    pdl_prologue();
-    if (mode != 1) {
-        if (on) {  // s = r - sum_off L y
-            const int r = st + lf - c0;
-            T acc = T(0);
-            for (int j = 0; j < wl; ++j) acc = fma(lval[(long)j * m + r], y[lcol[(long)j * m + r]], acc);
-            sm[lf] = y[st + lf] - acc;
-        }
-        __syncthreads();
-        for (int qq = 0; qq < nsub; ++qq) {
-            const bool act = q == qq && xx < nx;
-            T a = T(0), bb = T(1);
-            if (act) {
-                a = line_in_sum(cf, sm, lf, st, c0, m, wli, lidx, lvin);
-                bb = -cf.rec;
-            }
-            const T v = cta_line_scan<T>(a, bb, lane, wline, wA, wB);
-            if (act) {
-                sm[lf] = v;
-                y[st + lf] = v;
-            }
-            __syncthreads();
-        }
-        if (mode == 0) return;
-        line_coef_load(cf, on, lb, st, c0, m, wui, uidx, uvin, urec, udinv);
-    } else {
-        if (on) sm[lf] = y[st + lf];
-        __syncthreads();
-    }
-    // backward: t = y - sum_off U e in place; then the lines from the last, each
-    // from its end: e_x = udinv_x ((t_x - sum_in U e) - urec_x e_{x+1})
-    if (on) {
-        const int r = st + lf - c0;
-        T acc = T(0);
-        for (int j = 0; j < wu; ++j) acc = fma(uval[(long)j * m + r], y[ucol[(long)j * m + r]], acc);
-        sm[lf] -= acc;
-    }
-    __syncthreads();
-    for (int qq = nsub - 1; qq >= 0; --qq) {
-        const bool act = q == qq && xx < nx;
-        T a = T(0), bb = T(1);
-        if (act) {
-            const T acc = line_in_sum(cf, sm, lb, st, c0, m, wui, uidx, uvin);
-            a = cf.d * acc;
-            bb = -cf.d * cf.rec;
-        }
-        const T v = cta_line_scan<T>(a, bb, lane, wline, wA, wB);
-        if (act) {
-            sm[lb] = v;
-            y[st + lb] = v;
-            const int row = rows[st + lb];
-            z[row] = TZ(z[row] + TZ(v));
-        }
-        __syncthreads();
-    }
-}
-
-// The same sweep for k right-hand sides (k <= kMaxRhs): each loaded factor
-// entry serves every vector; per vector the arithmetic and its order are
-// those of lines_sweep_kernel. Shared memory: per vector its block values
-// (4 nx) and the warp maps of its scans (64). At most 512 threads a CTA.
-constexpr int kLinesMultiThreads = 512;
-
-template <typename T, typename TZ>
-__global__ void __launch_bounds__(kLinesMultiThreads) lines_sweep_multi_kernel(
-    int mode, int k, int b0, const int32_t *__restrict__ blk_start, const int32_t *__restrict__ blk_nsub, int nx,
-    int nxp, int c0, int m, int wl, const int32_t *__restrict__ lcol, const T *__restrict__ lval, int wli,
-    const int16_t *__restrict__ lidx, const T *__restrict__ lvin, const T *__restrict__ lrec, int wu,
-    const int32_t *__restrict__ ucol, const T *__restrict__ uval, int wui, const int16_t *__restrict__ uidx,
-    const T *__restrict__ uvin, const T *__restrict__ urec, const T *__restrict__ udinv,
-    const int32_t *__restrict__ rows, Cols<T> y, Cols<TZ> z) {
-    extern __shared__ unsigned char s_raw[];
-    T *smb = reinterpret_cast<T *>(s_raw);  // [k][4 nx] block values, then [k][64] warp maps
-    T *wmb = smb + (long)k * 4 * nx;
-    const int b = b0 + blockIdx.x;
-    const int st = blk_start[b], nsub = blk_nsub[b];
-    const int q = threadIdx.x / nxp, xx = threadIdx.x - q * nxp, lane = threadIdx.x & 31;
-    const int wline = xx >> 5;
-    const bool on = q < nsub && xx < nx;
-    const int lf = q * nx + xx;
-    const int lb = q * nx + (nx - 1 - xx);
-    LineCoef<T> cf;
-    if (mode != 1)
-        line_coef_load(cf, on, lf, st, c0, m, wli, lidx, lvin, lrec, (const T *)nullptr);
-    else
-        line_coef_load(cf, on, lb, st, c0, m, wui, uidx, uvin, urec, udinv);
-    pdl_prologue();
-    T acc[kMaxRhs];
-    if (mode != 1) {
-        if (on) {  // s = r - sum_off L y
-            const int r = st + lf - c0;
-#pragma unroll
-            for (int c = 0; c < kMaxRhs; ++c) acc[c] = T(0);
-            for (int j = 0; j < wl; ++j) {
-                const T lv = lval[(long)j * m + r];
-                const int col = lcol[(long)j * m + r];
-#pragma unroll
-                for (int c = 0; c < kMaxRhs; ++c)
-                    if (c < k) acc[c] = fma(lv, y.p[c][col], acc[c]);
-            }
-#pragma unroll
-            for (int c = 0; c < kMaxRhs; ++c)
-                if (c < k) smb[(long)c * 4 * nx + lf] = y.p[c][st + lf] - acc[c];
-        }
-        __syncthreads();
-        for (int qq = 0; qq < nsub; ++qq) {
-            const bool act = q == qq && xx < nx;
-            for (int c = 0; c < k; ++c) {
-                T *sm = smb + (long)c * 4 * nx;
-                T a = T(0), bb = T(1);
-                if (act) {
-                    a = line_in_sum(cf, sm, lf, st, c0, m, wli, lidx, lvin);
-                    bb = -cf.rec;
-                }
-                const T v = cta_line_scan<T>(a, bb, lane, wline, wmb + 64 * c, wmb + 64 * c + 32);
-                if (act) {
-                    sm[lf] = v;
-                    y.p[c][st + lf] = v;
-                }
-            }
-            __syncthreads();
-        }
-        if (mode == 0) return;
-        line_coef_load(cf, on, lb, st, c0, m, wui, uidx, uvin, urec, udinv);
-    } else {
-        if (on)
-            for (int c = 0; c < k; ++c) smb[(long)c * 4 * nx + lf] = y.p[c][st + lf];
-        __syncthreads();
-    }
-    if (on) {  // backward: t = y - sum_off U e
-        const int r = st + lf - c0;
-#pragma unroll
-        for (int c = 0; c < kMaxRhs; ++c) acc[c] = T(0);
-        for (int j = 0; j < wu; ++j) {
-            const T uv = uval[(long)j * m + r];
-            const int col = ucol[(long)j * m + r];
-#pragma unroll
-            for (int c = 0; c < kMaxRhs; ++c)
-                if (c < k) acc[c] = fma(uv, y.p[c][col], acc[c]);
-        }
-#pragma unroll
-        for (int c = 0; c < kMaxRhs; ++c)
-            if (c < k) smb[(long)c * 4 * nx + lf] -= acc[c];
-    }
-    __syncthreads();
-    for (int qq = nsub - 1; qq >= 0; --qq) {
-        const bool act = q == qq && xx < nx;
-        for (int c = 0; c < k; ++c) {
-            T *sm = smb + (long)c * 4 * nx;
-            T a = T(0), bb = T(1);
-            if (act) {
-                const T t = line_in_sum(cf, sm, lb, st, c0, m, wui, uidx, uvin);
-                a = cf.d * t;
-                bb = -cf.d * cf.rec;
-            }
-            const T v = cta_line_scan<T>(a, bb, lane, wline, wmb + 64 * c, wmb + 64 * c + 32);
-            if (act) {
-                sm[lb] = v;
-                y.p[c][st + lb] = v;
-                const int row = rows[st + lb];
-                z.p[c][row] = TZ(z.p[c][row] + TZ(v));
-            }
-        }
-        __syncthreads();
+    constexpr int G = kLineGroup<T>;
+    const long line = p / nx, lc = line - L.cptr[c] / nx;  // the line, and its place in the colour
+    using V = typename std::conditional<sizeof(T) == 4, float4, double2>::type;
+    auto put = [&](T *dst, long at, const T *src) {
+        V v;
+        memcpy(&v, src, 16);
+        reinterpret_cast<V *>(dst)[at] = v;
+    };
+    for (int d = 0; d < 2; ++d) {
+        const int ng = line_groups<T>(3 * L.noff[d][c]);
+        T *o = (d == 0 ? offl : offu) + L.obase[d][c];
+        for (int g = 0; g < ng; ++g) put(o, (lc * ng + g) * nx + x, off[d] + g * G);
+        constexpr int NI = line_groups<T>(kLineIn);
+        for (int g = 0; g < NI; ++g) put(d == 0 ? inl : inu, (line * NI + g) * nx + x, in[d] + g * G);
     }
 }
 
@@ -730,7 +435,7 @@ msrsb_status lines_setup(msrsb_handle *h, TF *lu, cudaStream_t s) {
     MSRSB_LAUNCHED("lines_pos_kernel");
     // ---- block table (host): blocks of each colour in block order ----
     const int nby = (ny + 1) / 2, nbz = dim == 3 ? (nz + 1) / 2 : 1;
-    std::vector<int32_t> bstart, bnsub;
+    std::vector<int32_t> bline, bstart, bnsub;
     int run = 0;
     for (int c = 0; c < L.ncol; ++c) {
         L.cptr[c] = run;
@@ -740,6 +445,7 @@ msrsb_status lines_setup(msrsb_handle *h, TF *lu, cudaStream_t s) {
                 const int cc = (by & 1) | (dim == 3 ? ((bz & 1) << 1) : 0);
                 if (cc != c) continue;
                 const int sy = ny - 2 * by < 2 ? 1 : 2, sz = dim == 3 ? (nz - 2 * bz < 2 ? 1 : 2) : 1;
+                bline.push_back(run / nx);
                 bstart.push_back(run);
                 bnsub.push_back(sy * sz);
                 run += sy * sz * nx;
@@ -749,18 +455,20 @@ msrsb_status lines_setup(msrsb_handle *h, TF *lu, cudaStream_t s) {
     L.bptr[L.ncol] = (int)bstart.size();
     if (run != n) return fail(MSRSB_ESHAPE, "line blocks cover %d of %d rows", run, n);
     const int nblk = (int)bstart.size();
-    MSRSB_TRY(dalloc(&L.blk_start, nblk, s));
+    int32_t *blk_start = nullptr;
+    MSRSB_TRY(dalloc(&blk_start, nblk, s));
+    MSRSB_TRY(dalloc(&L.blk_line, nblk, s));
     MSRSB_TRY(dalloc(&L.blk_nsub, nblk, s));
-    MSRSB_TRY(upload(L.blk_start, bstart.data(), nblk * sizeof(int32_t), s));
+    MSRSB_TRY(upload(L.blk_line, bline.data(), nblk * sizeof(int32_t), s));
+    MSRSB_TRY(upload(blk_start, bstart.data(), nblk * sizeof(int32_t), s));
     MSRSB_TRY(upload(L.blk_nsub, bnsub.data(), nblk * sizeof(int32_t), s));
     // ---- factorisation, colour by colour ----
     int *status = nullptr;
     TF *rdiag = nullptr;
-    int32_t *dpos = nullptr, *ccol = nullptr;
+    int32_t *dpos = nullptr;
     MSRSB_TRY(dalloc(&status, 1, s));
     MSRSB_TRY(dalloc(&rdiag, n, s));
     MSRSB_TRY(dalloc(&dpos, n, s));
-    MSRSB_TRY(dalloc(&ccol, n, s));
     MSRSB_CUDA(cudaMemsetAsync(status, 0, sizeof(int), s));
     diag_pos_launch(n, A.rowptr, A.colidx, dpos, status, s);
     MSRSB_LAUNCHED("diag_pos_kernel");
@@ -773,158 +481,60 @@ msrsb_status lines_setup(msrsb_handle *h, TF *lu, cudaStream_t s) {
                 L.cptr[c], cnt, dim, nx, ny, L.rows, A.rowptr, A.colidx, h->pos_of, rmask, lu, rdiag);
             MSRSB_LAUNCHED("lines_factor_off_kernel");
         }
-        lines_factor_ring_kernel<TF><<<nb, 128, 0, s>>>(c, L.bptr[c], L.blk_start, L.blk_nsub, dim, nx, ny, L.rows,
+        lines_factor_ring_kernel<TF><<<nb, 128, 0, s>>>(c, L.bptr[c], blk_start, L.blk_nsub, dim, nx, ny, L.rows,
                                                         A.rowptr, A.colidx, lu, rdiag, status);
         MSRSB_LAUNCHED("lines_factor_ring_kernel");
     }
+    // ---- the sweeps' coefficients by neighbour line, and the lines' neighbours ----
+    const int nlines = n / nx;
+    long ot[2] = {0, 0};
+    for (int c = 0; c < L.ncol; ++c) {
+        const int flips = dim == 3 ? 3 : 1;  // neighbour blocks' colours: c with y's and z's parity flipped
+        L.noff[0][c] = L.noff[1][c] = 0;
+        for (int f = 1; f <= flips; ++f) L.noff[(c ^ f) < c ? 0 : 1][c] += f == 3 || dim == 2 ? 1 : 2;
+        for (int d = 0; d < 2; ++d) {
+            L.obase[d][c] = ot[d];
+            ot[d] += (long)(L.cptr[c + 1] - L.cptr[c]) * line_groups<TF>(3 * L.noff[d][c]) * kLineGroup<TF>;
+        }
+    }
+    TF *offl = nullptr, *offu = nullptr, *inl = nullptr, *inu = nullptr;
+    MSRSB_TRY(dalloc(&offl, ot[0], s));
+    L.off[0] = offl;
+    MSRSB_TRY(dalloc(&offu, ot[1], s));
+    L.off[1] = offu;
+    MSRSB_TRY(dalloc(&inl, (size_t)n * kLineIn, s));
+    L.in[0] = inl;
+    MSRSB_TRY(dalloc(&inu, (size_t)n * kLineIn, s));
+    L.in[1] = inu;
+    MSRSB_TRY(dalloc(&L.nbr, (size_t)2 * nlines * kLineNbr, s));
+    lines_nbr_kernel<<<ceil_div(nlines, 128), 128, 0, s>>>(nlines, dim, nx, ny, nz, L.rows, h->pos_of, L.nbr);
+    MSRSB_LAUNCHED("lines_nbr_kernel");
+    lines_fill_kernel<TF><<<ceil_div(n, 128), 128, 0, s>>>(n, dim, nx, ny, nz, A.rowptr, rmask, lu, L.rows, L, offl,
+                                                           offu, inl, inu);
+    MSRSB_LAUNCHED("lines_fill_kernel");
     int hs = 0;
     MSRSB_TRY(read_back(&hs, status, sizeof(int), s));
     dfree(rdiag, s);
     dfree(rmask, s);
-    if (hs) {
-        dfree(status, s);
-        dfree(dpos, s);
-        dfree(ccol, s);
-        if (hs < 0) return fail(MSRSB_EINVAL, "ILU(0): row %d has more than 32 entries", -hs - 1);
-        return fail(MSRSB_EBREAKDOWN, "ILU(0): zero pivot at row %d", hs - 1);
-    }
-    // ---- per-colour ELL blocks of the parallel parts, line coefficients ----
-    lines_colour_of_kernel<<<ceil_div(n, 256), 256, 0, s>>>(n, L.rows, L, ccol);
-    MSRSB_LAUNCHED("lines_colour_of_kernel");
-    int *w = nullptr;
-    MSRSB_TRY(dalloc(&w, 16, s));
-    MSRSB_CUDA(cudaMemsetAsync(w, 0, 16 * sizeof(int), s));
-    lines_width_kernel<<<ceil_div(n, 256), 256, 0, s>>>(n, nx, ny, A.rowptr, A.colidx, h->pos_of, ccol, w);
-    MSRSB_LAUNCHED("lines_width_kernel");
-    int hw[16];
-    MSRSB_TRY(read_back(hw, w, 16 * sizeof(int), s));
-    dfree(w, s);
-    long lt = 0, ut = 0, lit = 0, uit = 0;
-    for (int c = 0; c < L.ncol; ++c) {
-        L.wl[c] = hw[c];
-        L.wu[c] = hw[4 + c];
-        L.wli[c] = hw[8 + c];
-        L.wui[c] = hw[12 + c];
-        L.lbase[c] = lt;
-        L.ubase[c] = ut;
-        L.libase[c] = lit;
-        L.uibase[c] = uit;
-        const long m = L.cptr[c + 1] - L.cptr[c];
-        lt += m * L.wl[c];
-        ut += m * L.wu[c];
-        lit += m * L.wli[c];
-        uit += m * L.wui[c];
-    }
-    TF *lval = nullptr, *uval = nullptr, *lvin = nullptr, *uvin = nullptr, *lrec = nullptr, *urec = nullptr,
-       *udinv = nullptr;
-    MSRSB_TRY(dalloc(&L.lcol, lt, s));
-    MSRSB_TRY(dalloc(&L.ucol, ut, s));
-    MSRSB_TRY(dalloc(&L.lidx, lit, s));
-    MSRSB_TRY(dalloc(&L.uidx, uit, s));
-    MSRSB_TRY(dalloc(&lval, lt, s));
-    MSRSB_TRY(dalloc(&uval, ut, s));
-    MSRSB_TRY(dalloc(&lvin, lit, s));
-    MSRSB_TRY(dalloc(&uvin, uit, s));
-    MSRSB_TRY(dalloc(&lrec, n, s));
-    MSRSB_TRY(dalloc(&urec, n, s));
-    MSRSB_TRY(dalloc(&udinv, n, s));
-    L.lval = lval;
-    L.uval = uval;
-    L.lvin = lvin;
-    L.uvin = uvin;
-    L.lrec = lrec;
-    L.urec = urec;
-    L.udinv = udinv;
-    lines_fill_kernel<TF><<<ceil_div(n, 256), 256, 0, s>>>(n, nx, ny, A.rowptr, A.colidx, lu, dpos, h->pos_of, ccol, L,
-                                                           lval, uval, lvin, uvin, lrec, urec, udinv);
-    MSRSB_LAUNCHED("lines_fill_kernel");
     dfree(status, s);
     dfree(dpos, s);
-    dfree(ccol, s);
+    dfree(blk_start, s);
+    if (hs < 0) return fail(MSRSB_EINVAL, "ILU(0): row %d has more than 32 entries", -hs - 1);
+    if (hs) return fail(MSRSB_EBREAKDOWN, "ILU(0): zero pivot at row %d", hs - 1);
     return MSRSB_OK;
 }
 template msrsb_status lines_setup<double>(msrsb_handle *, double *, cudaStream_t);
 template msrsb_status lines_setup<float>(msrsb_handle *, float *, cudaStream_t);
 
-// z += U^-1 L^-1 r with r given in the line-block order in ry (overwritten):
-// 2 C - 1 launches for C colours, one CTA per line block
-template <typename T, typename TZ>
-msrsb_status lines_apply(const msrsb_handle *h, T *ry, TZ *z, cudaStream_t s) {
-    const IluLines &L = h->lines;
-    const int last = L.ncol - 1, nxp = ((L.nx + 31) / 32) * 32;
-    const int nsub_max = L.ncol == 4 ? 4 : 2;
-    const size_t smem = (4 * (size_t)L.nx + 64) * sizeof(T);
-    auto launch = [&](int mode, int c) -> msrsb_status {
-        const int nb = L.bptr[c + 1] - L.bptr[c];
-        if (!nb) return MSRSB_OK;
-        const int m = L.cptr[c + 1] - L.cptr[c];
-        MSRSB_PDL((lines_sweep_kernel<T, TZ>), nb, nsub_max * nxp, smem, s, mode, L.bptr[c], L.blk_start,
-                  L.blk_nsub, L.nx, nxp, L.cptr[c], m, L.wl[c], L.lcol + L.lbase[c], (const T *)L.lval + L.lbase[c],
-                  L.wli[c], L.lidx + L.libase[c], (const T *)L.lvin + L.libase[c], (const T *)L.lrec, L.wu[c],
-                  L.ucol + L.ubase[c], (const T *)L.uval + L.ubase[c], L.wui[c], L.uidx + L.uibase[c],
-                  (const T *)L.uvin + L.uibase[c], (const T *)L.urec, (const T *)L.udinv, L.rows, ry, z);
-        return MSRSB_OK;
-    };
-    for (int c = 0; c < last; ++c) MSRSB_TRY(launch(0, c));
-    MSRSB_TRY(launch(2, last));
-    for (int c = last - 1; c >= 0; --c) MSRSB_TRY(launch(1, c));
-    return MSRSB_OK;
-}
-template msrsb_status lines_apply<double, double>(const msrsb_handle *, double *, double *, cudaStream_t);
-template msrsb_status lines_apply<float, double>(const msrsb_handle *, float *, double *, cudaStream_t);
-template msrsb_status lines_apply<float, float>(const msrsb_handle *, float *, float *, cudaStream_t);
-
-// lines_apply for k right-hand sides (one launch per colour and direction,
-// as lines_apply); false in *ok when the blocks exceed the multi kernel's CTA
-bool lines_multi_fit(const msrsb_handle *h) {
-    const IluLines &L = h->lines;
-    const int nxp = ((L.nx + 31) / 32) * 32;
-    return (L.ncol == 4 ? 4 : 2) * nxp <= kLinesMultiThreads;
-}
-
-template <typename T, typename TZ>
-msrsb_status lines_apply_multi(const msrsb_handle *h, int k, Cols<T> ry, Cols<TZ> z, cudaStream_t s) {
-    const IluLines &L = h->lines;
-    const int last = L.ncol - 1, nxp = ((L.nx + 31) / 32) * 32;
-    const int threads = (L.ncol == 4 ? 4 : 2) * nxp;
-    if (threads > kLinesMultiThreads || k < 1 || k > kMaxRhs) return fail(MSRSB_EINVAL, "multi-vector sweep shape");
-    const size_t smem = (size_t)k * (4 * (size_t)L.nx + 64) * sizeof(T);
-    auto launch = [&](int mode, int c) -> msrsb_status {
-        const int nb = L.bptr[c + 1] - L.bptr[c];
-        if (!nb) return MSRSB_OK;
-        const int m = L.cptr[c + 1] - L.cptr[c];
-        MSRSB_PDL((lines_sweep_multi_kernel<T, TZ>), nb, threads, smem, s, mode, k, L.bptr[c], L.blk_start,
-                  L.blk_nsub, L.nx, nxp, L.cptr[c], m, L.wl[c], L.lcol + L.lbase[c], (const T *)L.lval + L.lbase[c],
-                  L.wli[c], L.lidx + L.libase[c], (const T *)L.lvin + L.libase[c], (const T *)L.lrec, L.wu[c],
-                  L.ucol + L.ubase[c], (const T *)L.uval + L.ubase[c], L.wui[c], L.uidx + L.uibase[c],
-                  (const T *)L.uvin + L.uibase[c], (const T *)L.urec, (const T *)L.udinv, L.rows, ry, z);
-        return MSRSB_OK;
-    };
-    for (int c = 0; c < last; ++c) MSRSB_TRY(launch(0, c));
-    MSRSB_TRY(launch(2, last));
-    for (int c = last - 1; c >= 0; --c) MSRSB_TRY(launch(1, c));
-    return MSRSB_OK;
-}
-template msrsb_status lines_apply_multi<double, double>(const msrsb_handle *, int, Cols<double>, Cols<double>,
-                                                        cudaStream_t);
-template msrsb_status lines_apply_multi<float, double>(const msrsb_handle *, int, Cols<float>, Cols<double>,
-                                                       cudaStream_t);
-
 void lines_free(IluLines *L, cudaStream_t s) {
-    dfree(L->lidx, s);
-    dfree(L->uidx, s);
-    dfree(L->lvin, s);
-    dfree(L->uvin, s);
     dfree(L->rows, s);
-    dfree(L->blk_start, s);
+    dfree(L->blk_line, s);
     dfree(L->blk_nsub, s);
-    dfree(L->lcol, s);
-    dfree(L->ucol, s);
-    dfree(L->lval, s);
-    dfree(L->uval, s);
-    dfree(L->lrec, s);
-    dfree(L->urec, s);
-    dfree(L->udinv, s);
+    dfree(L->nbr, s);
+    for (int d = 0; d < 2; ++d) {
+        dfree(L->off[d], s);
+        dfree(L->in[d], s);
+    }
 }
 
 }  // namespace msrsb
