@@ -23,11 +23,13 @@
 // inside the plane (ties to the lowest row; magnitudes compared through the
 // integer order of their FP64 bit patterns). Both the factorisation and the
 // application run as thread-block clusters (up to 16 CTAs on 16 SMs) whose
-// CTAs own contiguous columns (factorisation) or rows (application) and
-// exchange pivot columns and partial vectors through distributed shared
-// memory, with hardware cluster barriers between steps (no spin waits).
+// CTAs own columns (factorisation, dealt out in turn) or contiguous rows
+// (application) and exchange pivot columns and partial vectors through
+// distributed shared memory, with hardware cluster barriers between steps (no
+// spin waits).
 #include "common.cuh"
 #include <cooperative_groups.h>
+#include <initializer_list>
 #include <mutex>
 
 namespace cg = cooperative_groups;
@@ -92,17 +94,93 @@ __device__ __forceinline__ double sub_coupling(double v, const PlaneGeom &G, con
 
 constexpr int kPlaneThreads = 256;
 constexpr int kPlaneMaxCols = 128;  // columns of a plane one CTA of the factorisation owns
+constexpr int kPlaneMaxRows = 768;  // rows of a plane the factorisation takes
+constexpr int kPlaneMaxCluster = 16;
+constexpr int kFactorThreads = kPlaneThreads + 32;  // a warp of its own for the pivot's reciprocal
+
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_arrive_relaxed() {
+    asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+// shared-memory address of p in CTA `rank` of the cluster
+__device__ __forceinline__ unsigned map_rank(const void *p, int rank) {
+    unsigned a;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((unsigned)__cvta_generic_to_shared(p)), "r"(rank));
+    return a;
+}
+__device__ __forceinline__ void st_rank(unsigned a, double v) {
+    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
+}
+__device__ __forceinline__ void st_rank(unsigned a, int v) {
+    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
+}
+__device__ __forceinline__ double ld_rank(unsigned a) {
+    double v;
+    asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(a) : "memory");
+    return v;
+}
+
+// The lane (as a mask of one bit) with the largest key, ties to the lowest row;
+// 0 when every key is negative. Keys are magnitudes as 63-bit integers: the
+// high words decide unless they tie.
+__device__ __forceinline__ unsigned plane_top(long long key, int row) {
+    const unsigned hi = key < 0 ? 0u : (unsigned)(key >> 32) + 1u, mh = __reduce_max_sync(0xffffffffu, hi);
+    if (!mh) return 0u;
+    unsigned who = __ballot_sync(0xffffffffu, hi == mh);
+    if (who & (who - 1u)) {
+        const unsigned ml = __reduce_max_sync(0xffffffffu, hi == mh ? (unsigned)key : 0u);
+        const bool top = hi == mh && (unsigned)key == ml;
+        const unsigned r = __reduce_min_sync(0xffffffffu, top ? (unsigned)row : 0xffffffffu);
+        who = __ballot_sync(0xffffffffu, top && (unsigned)row == r);
+    }
+    return who;
+}
 
 // Factorisation. With middle = 0 the grid holds one cluster per side (side 0:
 // planes 0 .. h-1 upwards, side 1: planes np-1 .. h+1 downwards); with
 // middle = 1 one cluster takes plane h. Outputs (row-major m x m per plane):
 // X_k with S_k^-1 = X_k Pi_k (Pi_k the row interchanges of the elimination,
 // kept as the gather pi_k: (Pi_k v)[i] = v[pi_k[i]]), and G_k for k != h.
-// status[0] = 1 + (global row) on a zero pivot.
-__global__ void __launch_bounds__(kPlaneThreads, 1) plane_factor_kernel(PlaneGeom G, int h, int middle,
-                                                                     const double *__restrict__ Acs,
-                                                                     double *__restrict__ X, double *__restrict__ Gm,
-                                                                     int *__restrict__ pi, int *__restrict__ status) {
+// status[0] = 1 + (global row) on a zero pivot. keep: a CTA's columns of the
+// last G_k stay in shared memory, where its columns of the next S_k need them.
+//
+// The elimination is a chain of m pivot steps per plane. A step's update (m^2
+// FMAs over the cluster) keeps the FP64 pipes of 16 SMs busy for 1.4 us at m =
+// 256 (measured: an SM starts a warp's FP64 FMA every 19 cycles); the pivot
+// search, the exchange of the pivot column and the cluster barrier are latency,
+// and took 3 us when they followed it. They now run beside it, and are short:
+//  - columns are dealt out in turn (column j to CTA j mod nct), so the owner of
+//    the next pivot column changes at every step;
+//  - at step kk the owner of column kk + 1 brings that column up to date first,
+//    finds its pivot, and stores the column into every CTA's shared memory
+//    before it arrives at the barrier; the others arrive at once. All then
+//    update their own columns, and wait for the barrier only at the start of
+//    step kk + 1;
+//  - the pivot's reciprocal (a chain of FP64 operations as long as the column's
+//    exchange) is taken by a warp of its own beside that exchange;
+//  - a warp updates whole columns, the pivot column's rows of a lane in RPL
+//    registers, so that row interchange, pivot-row entry and update need no
+//    CTA barrier and read no pivot column twice;
+//  - a thread's row of S_k takes its couplings from registers, and the columns of
+//    X_k that G_k combines are listed once per plane, so that their loads from
+//    other CTAs are independent of one another.
+// Three pivot-column buffers: a CTA arrives for column kk + 1 when it has done
+// with step kk - 1, so the column that a passed barrier lets the next owner
+// overwrite is two steps old. The arithmetic and its order are those of the
+// plain elimination. Measured, both factorisation launches: 128^3 (9 dependent
+// planes of 256) 11.2 -> 4.9 ms, 48^3 elasticity (5 of 243) 5.6 -> 2.7 ms, 64^3 (5
+// of 64, with the explicit inverse) 0.79 -> 0.61 ms; of a step's 4,200 cycles at
+// m = 256 the update takes 2,790, the owner's column, search, exchange and
+// release 4,000 beside it.
+template <int RPL>
+__global__ void __launch_bounds__(kFactorThreads, 1) plane_factor_kernel(PlaneGeom G, int h, int middle, int keep,
+                                                                      const double *__restrict__ Acs,
+                                                                      double *__restrict__ X,
+                                                                      double *__restrict__ Gm, int *__restrict__ pi,
+                                                                      int *__restrict__ status) {
+    constexpr int RPT = (32 * RPL + kPlaneThreads - 1) / kPlaneThreads;  // rows per thread
+    constexpr int kWarps = kPlaneThreads / 32;
     cg::cluster_group cluster = cg::this_cluster();
     const int rank = (int)cluster.block_rank(), nct = (int)cluster.num_blocks();
     // side 0: planes 0 .. h-1 upwards; side 1: planes np-1 .. h+1 downwards;
@@ -111,19 +189,94 @@ __global__ void __launch_bounds__(kPlaneThreads, 1) plane_factor_kernel(PlaneGeo
     const int nplanes = middle ? 1 : (side == 0 ? h : G.np - 1 - h);
     const int m = G.m, bd = G.bd, NI = G.NI;
     const int cw = (m + nct - 1) / nct;
-    const int c0 = rank * cw, c1 = min(m, c0 + cw), ncol = max(0, c1 - c0);
-    const int tid = threadIdx.x;
+    const int ncol = rank < m ? (m - rank + nct - 1) / nct : 0;  // own columns: rank, rank + nct, ...
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const bool worker = tid < kPlaneThreads;
     extern __shared__ double sm[];
-    double *Sown = sm;                       // own columns of S_k, column-major [cw][m]
-    double *fbuf = Sown + (long)cw * m;      // published pivot column, double buffered [2][m]
-    double *floc = fbuf + 2 * m;             // local copy of the pivot column [m]
-    int *piv_hist = (int *)(floc + m);       // pivot row of every step [m]
-    int *pil = piv_hist + m;                 // gather pi [m]
-    int *pinv = pil + m;                     // inverse of pi [m]
-    __shared__ double s_inv[2], s_xk[kPlaneMaxCols];
-    __shared__ int s_p[2], s_bad[2];
-    __shared__ double s_best[8];
-    __shared__ int s_idx[8];
+    double *Sown = sm;                     // own columns of S_k, column-major [cw][m]
+    double *pcol = Sown + (long)cw * m;    // pivot columns [3][m], written by their owners
+    int *pil = (int *)(pcol + 3 * m);      // gather pi [m]
+    int *pinv = pil + m;                   // inverse of pi [m]
+    double *Gown = (double *)(pinv + m);   // own columns of the last G_k [cw][m] (keep)
+    __shared__ double s_inv[3], s_best[kWarps], s_top;
+    __shared__ int s_p[3], s_bad[3], s_idx[kWarps];
+    __shared__ double s_gval[kWarps][27];    // one column's list of a warp: value, address of X's column
+    __shared__ unsigned s_gcol[kWarps][27];
+    unsigned rcol[kPlaneMaxCluster];  // the pivot buffers of every CTA
+#pragma unroll
+    for (int r = 0; r < kPlaneMaxCluster; ++r) rcol[r] = map_rank(pcol, r < nct ? r : 0);
+
+    // Column kk (local index jl) is up to date through step kk - 1 and its rows
+    // v[] (row tid + 256 t) are in this CTA's registers: find the pivot among
+    // rows kk .. m-1 (largest magnitude, ties to the lowest row), store the
+    // column with rows kk and pivot interchanged here and in every CTA's pivot
+    // buffer, with 1 / pivot.
+    auto publish = [&](int kk, int jl, const double (&v)[RPT]) {
+        if (worker) {
+            long long best = -1;
+            int bi = m;
+            double bv = 0.0;
+#pragma unroll
+            for (int t = 0; t < RPT; ++t) {
+                const int i = tid + t * kPlaneThreads;
+                if (i >= kk && i < m) {
+                    const long long a = __double_as_longlong(v[t]) & 0x7fffffffffffffffLL;
+                    if (a > best) {
+                        best = a;
+                        bi = i;
+                        bv = v[t];
+                    }
+                }
+                if (i == kk) s_top = v[t];
+            }
+            const unsigned who = plane_top(best, bi);
+            if (who ? who >> lane & 1u : lane == 0) {
+                s_idx[warp] = who ? bi : m;
+                s_best[warp] = who ? bv : 0.0;
+            }
+        }
+        __syncthreads();
+        int bi;
+        double pv;
+        {  // the warps' candidates, one per lane
+            const int w = lane & (kWarps - 1);
+            const int i2 = s_idx[w];
+            const double v2 = s_best[w];
+            const long long best = __double_as_longlong(v2) & 0x7fffffffffffffffLL;
+            const unsigned who = plane_top(i2 < m && lane < kWarps ? best : -1, i2);
+            const int src = who ? __ffs(who) - 1 : 0;
+            bi = who ? __shfl_sync(0xffffffffu, i2, src) : m;
+            pv = __shfl_sync(0xffffffffu, v2, src);
+        }
+        // zero, infinite or NaN, by the bits
+        const long long pb = __double_as_longlong(pv) & 0x7fffffffffffffffLL;
+        const bool bad = bi >= m || pb == 0 || pb >= 0x7ff0000000000000LL;
+        const int p = bi < m ? bi : kk, buf = kk % 3;
+        if (!worker) {  // the pivot's row and reciprocal, one destination a lane
+            if (lane < nct) {
+                st_rank(map_rank(s_p + buf, lane), p);
+                st_rank(map_rank(s_bad + buf, lane), bad ? 1 : 0);
+                st_rank(map_rank(s_inv + buf, lane), bad ? 0.0 : 1.0 / pv);
+            }
+            return;
+        }
+        const double vt = s_top;
+        double *col = Sown + (long)jl * m;
+#pragma unroll
+        for (int t = 0; t < RPT; ++t) {
+            const int i = tid + t * kPlaneThreads;
+            if (i < m) {
+                const double x = bad ? v[t] : (i == kk ? pv : (i == p ? vt : v[t]));
+                const unsigned at = (unsigned)(buf * m + i) * 8u;
+                col[i] = x;
+#pragma unroll
+                for (int r = 0; r < kPlaneMaxCluster; ++r)
+                    if (r < nct) st_rank(rcol[r] + at, x);
+            }
+        }
+    };
+
+    cluster.sync();  // every CTA runs before another stores into its shared memory
     for (int st = 0; st < nplanes; ++st) {
         const int k = middle ? h : (side == 0 ? st : G.np - 1 - st);
         // ---- S_k = D_k - C_{k,p} G_p over the planes p finished before it, own columns ----
@@ -138,157 +291,193 @@ __global__ void __launch_bounds__(kPlaneThreads, 1) plane_factor_kernel(PlaneGeo
             pa = side == 0 ? k - 1 : k + 1;
             ba = side == 0 ? 0 : 2 * NI;
         }
-        for (int idx = tid; idx < ncol * m; idx += kPlaneThreads) {
-            const int jl = idx / m, i = idx - jl * m;
-            const int j = c0 + jl;
-            const int ui = i / bd, l = i - ui * bd, uj = j / bd, mj = j - uj * bd;
-            const int a = plane_offset(G, ui, uj);
-            double v = a >= 0 ? st_val(Acs, G, Jbase + ui, a + NI, l, mj) : 0.0;
-            if (pa >= 0) v = sub_coupling(v, G, Acs, Jbase + ui, ui, l, ba, Gm + (long)pa * m * m + j, m);
-            if (pb >= 0) v = sub_coupling(v, G, Acs, Jbase + ui, ui, l, bb, Gm + (long)pb * m * m + j, m);
-            Sown[(long)jl * m + i] = v;
-        }
+        if (worker)
+            for (int i = tid; i < m; i += kPlaneThreads) {  // a thread's row, all own columns
+                const int ui = i / bd, l = i - ui * bd;
+                int nbr[9];  // dof 0 of the row's in-plane neighbours, -1 off the grid
+#pragma unroll
+                for (int a = 0; a < 9; ++a) {
+                    nbr[a] = a < NI ? plane_nbr(G, ui, a) : -1;
+                    if (nbr[a] >= 0) nbr[a] *= bd;
+                }
+                for (int jl = 0; jl < ncol; ++jl) {
+                    const int j = rank + jl * nct, uj = j / bd, a = plane_offset(G, ui, uj);
+                    Sown[(long)jl * m + i] = a >= 0 ? st_val(Acs, G, Jbase + ui, a + NI, l, j - uj * bd) : 0.0;
+                }
+                for (int side2 = 0; side2 < 2; ++side2) {
+                    const int pl = side2 ? pb : pa, base = side2 ? bb : ba;
+                    if (pl < 0) continue;
+                    const bool own = keep && !middle;
+#pragma unroll
+                    for (int a0 = 0; a0 < 9; a0 += 3) {  // three neighbours at a time, in order
+                        double cf[9];
+#pragma unroll
+                        for (int a = 0; a < 3; ++a)
+#pragma unroll
+                            for (int c = 0; c < 3; ++c)
+                                cf[a * 3 + c] = nbr[a0 + a] >= 0 && c < bd
+                                                    ? -st_val(Acs, G, Jbase + ui, a0 + a + base, l, c) : 0.0;
+#pragma unroll 2
+                        for (int jl = 0; jl < ncol; ++jl) {
+                            const double *vec = own ? Gown + (long)jl * m : Gm + (long)pl * m * m + rank + jl * nct;
+                            const long sd = own ? 1 : m;
+                            double v = Sown[(long)jl * m + i];
+#pragma unroll
+                            for (int a = 0; a < 3; ++a)
+#pragma unroll
+                                for (int c = 0; c < 3; ++c)
+                                    if (nbr[a0 + a] >= 0 && c < bd)
+                                        v = fma(cf[a * 3 + c], vec[(nbr[a0 + a] + c) * sd], v);
+                            Sown[(long)jl * m + i] = v;
+                        }
+                    }
+                }
+                pil[i] = i;
+            }
         __syncthreads();
         // ---- Gauss-Jordan with partial pivoting, one pivot per step ----
-        for (int kk = 0; kk < m; ++kk) {
-            const int owner = kk / cw, buf = kk & 1;
-            if (rank == owner) {
-                double *col = Sown + (long)(kk - c0) * m;
-                // largest |col[i]|, kk <= i < m, ties to the lowest index
-                long long best = -1;
-                int bi = m;
-                for (int i = kk + tid; i < m; i += kPlaneThreads) {
-                    const long long v = __double_as_longlong(col[i]) & 0x7fffffffffffffffLL;
-                    if (v > best) {
-                        best = v;
-                        bi = i;
-                    }
-                }
+        if (rank == 0) {
+            double v[RPT];
 #pragma unroll
-                for (int o = 16; o > 0; o >>= 1) {
-                    const long long b2 = __shfl_xor_sync(0xffffffffu, best, o);
-                    const int i2 = __shfl_xor_sync(0xffffffffu, bi, o);
-                    if (b2 > best || (b2 == best && i2 < bi)) {
-                        best = b2;
-                        bi = i2;
-                    }
-                }
-                long long *sb = reinterpret_cast<long long *>(s_best);
-                if ((tid & 31) == 0) {
-                    sb[tid >> 5] = best;
-                    s_idx[tid >> 5] = bi;
-                }
-                __syncthreads();
-                if (tid == 0) {
-                    long long bb = sb[0];
-                    int bj = s_idx[0];
-                    for (int w = 1; w < kPlaneThreads / 32; ++w)
-                        if (sb[w] > bb || (sb[w] == bb && s_idx[w] < bj)) {
-                            bb = sb[w];
-                            bj = s_idx[w];
-                        }
-                    const double pv = bj < m ? col[bj] : 0.0;
-                    const int bad = (bj >= m || pv == 0.0 || !isfinite(pv)) ? 1 : 0;
-                    if (!bad && bj != kk) {
-                        const double t = col[kk];
-                        col[kk] = col[bj];
-                        col[bj] = t;
-                    }
-                    s_p[buf] = bj < m ? bj : kk;
-                    s_bad[buf] = bad;
-                    s_inv[buf] = bad ? 0.0 : 1.0 / pv;
-                }
-                __syncthreads();
-                for (int i = tid; i < m; i += kPlaneThreads) fbuf[buf * m + i] = col[i];
+            for (int t = 0; t < RPT; ++t) {
+                const int i = tid + t * kPlaneThreads;
+                v[t] = worker && i < m ? Sown[i] : 0.0;
             }
-            cluster.sync();  // the owner's pivot column is published
-            const int *op = cluster.map_shared_rank(s_p, owner);
-            const int *ob = cluster.map_shared_rank(s_bad, owner);
-            const double *oi = cluster.map_shared_rank(s_inv, owner);
-            const double *of = cluster.map_shared_rank(fbuf, owner) + buf * m;
-            const int p = op[buf], bad = ob[buf];
-            const double inv = oi[buf];
-            if (bad) {
+            publish(0, 0, v);
+        }
+        cluster_arrive();
+        for (int kk = 0; kk < m; ++kk) {
+            cluster_wait();  // pivot column kk is in every CTA's buffer
+            const int buf = kk % 3, p = s_p[buf];
+            const double inv = s_inv[buf];
+            const double *f = pcol + buf * m;
+            if (s_bad[buf]) {  // uniform over the cluster
                 if (rank == 0 && tid == 0) *status = 1 + k * m + kk;
-                cluster.sync();  // no CTA leaves while another may still read its shared memory
+                cluster.sync();  // no CTA leaves while another may still write its shared memory
                 return;
             }
-            for (int i = tid; i < m; i += kPlaneThreads) floc[i] = of[i];
-            if (tid == 0) piv_hist[kk] = p;
-            if (tid < ncol) {  // row interchange and scaled pivot-row entry of every own column but kk
-                const int j = c0 + tid;
-                if (j != kk) {
-                    double *cj = Sown + (long)tid * m;
-                    double x = cj[kk];
-                    if (p != kk) {
-                        const double y = cj[p];
-                        cj[p] = x;
-                        x = y;
-                    }
-                    x *= inv;
-                    cj[kk] = x;
-                    s_xk[tid] = x;
+            const bool next = kk + 1 < m && rank == (kk + 1) % nct;
+            if (next) {  // column kk + 1 first, and its pivot
+                const int jl = (kk + 1) / nct;
+                const double *cj = Sown + (long)jl * m;
+                __syncthreads();  // the column's step kk - 1 is done (by the warp it belongs to)
+                const double ck = cj[kk], x = cj[p] * inv;
+                double v[RPT];
+#pragma unroll
+                for (int t = 0; t < RPT; ++t) {
+                    const int i = tid + t * kPlaneThreads;
+                    v[t] = 0.0;
+                    if (worker && i < m) v[t] = i == kk ? x : fma(-f[i], x, i == p ? ck : cj[i]);
                 }
+                publish(kk + 1, jl, v);
             }
-            __syncthreads();
-            for (int idx = tid; idx < ncol * m; idx += kPlaneThreads) {
-                const int jl = idx / m, i = idx - jl * m;
-                double *cj = Sown + (long)jl * m;
-                if (c0 + jl == kk)
-                    cj[i] = i == kk ? inv : -floc[i] * inv;
-                else if (i != kk)
-                    cj[i] = fma(-floc[i], s_xk[jl], cj[i]);
+            if (next) cluster_arrive();
+            else if (kk + 1 < m) cluster_arrive_relaxed();  // nothing written for another CTA, reads consumed
+            if (!worker) {
+                if (lane == 0 && p != kk) {
+                    const int t = pil[kk];
+                    pil[kk] = pil[p];
+                    pil[p] = t;
+                }
+                continue;
             }
-            __syncthreads();
-        }
-        // ---- the gather pi_k and its inverse (every CTA, from the pivot history) ----
-        if (tid == 0) {
-            for (int i = 0; i < m; ++i) pil[i] = i;
-            for (int kk = 0; kk < m; ++kk) {
-                const int p = piv_hist[kk];
-                const int t = pil[kk];
-                pil[kk] = pil[p];
-                pil[p] = t;
+            double fr[RPL];
+#pragma unroll
+            for (int t = 0; t < RPL; ++t) fr[t] = f[min(lane + 32 * t, m - 1)];
+            // two columns of the warp side by side; the pivot column itself is 0 - f / pivot
+            for (int jl0 = warp; jl0 < ncol; jl0 += 2 * kWarps) {
+                double c[2][RPL], ck[2], x[2];
+                double *cj[2];
+                bool put[2];
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    const int jl = jl0 + u * kWarps, j = rank + jl * nct;
+                    put[u] = jl < ncol && !(next && j == kk + 1);
+                    cj[u] = Sown + (long)(put[u] ? jl : jl0) * m;
+                    ck[u] = j == kk ? 0.0 : cj[u][kk];
+                    x[u] = cj[u][p];
+#pragma unroll
+                    for (int t = 0; t < RPL; ++t) c[u][t] = j == kk ? 0.0 : cj[u][min(lane + 32 * t, m - 1)];
+                    const double xi = x[u] * inv;
+                    x[u] = j == kk ? inv : xi;
+                }
+                __syncwarp();
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    if (!put[u]) continue;  // uniform over the warp
+#pragma unroll
+                    for (int t = 0; t < RPL; ++t) {
+                        const int i = lane + 32 * t;
+                        const double r = fma(fr[t], -x[u], i == p ? ck[u] : c[u][t]);  // no branch around the FMA
+                        c[u][t] = i == kk ? x[u] : r;
+                    }
+#pragma unroll
+                    for (int t = 0; t < RPL; ++t)
+                        if (lane + 32 * t < m) cj[u][lane + 32 * t] = c[u][t];
+                }
+                __syncwarp();
             }
-            for (int i = 0; i < m; ++i) pinv[pil[i]] = i;
         }
         __syncthreads();
+        for (int i = tid; i < m; i += kFactorThreads) pinv[pil[i]] = i;
         // ---- X_k (own columns, row-major in global) and pi_k ----
         double *Xk = X + (long)k * m * m;
-        for (int idx = tid; idx < ncol * m; idx += kPlaneThreads) {
+        for (int idx = tid; idx < ncol * m; idx += kFactorThreads) {
             const int i = idx / ncol, jl = idx - i * ncol;
-            Xk[(long)i * m + c0 + jl] = Sown[(long)jl * m + i];
+            Xk[(long)i * m + rank + jl * nct] = Sown[(long)jl * m + i];
         }
         if (rank == 0)
-            for (int i = tid; i < m; i += kPlaneThreads) pi[(long)k * m + i] = pil[i];
+            for (int i = tid; i < m; i += kFactorThreads) pi[(long)k * m + i] = pil[i];
         cluster.sync();  // every CTA's X_k columns are final
         // ---- G_k = X_k Pi_k C_{k,q}, q the plane after k on this side (k+1 on
-        // side 0, k-1 on side 1), own columns j (rows of plane q) ----
-        if (!middle) {
+        // side 0, k-1 on side 1), own columns j (rows of plane q): a warp per column ----
+        if (!middle && worker) {
             double *Gk = Gm + (long)k * m * m;
             const int qb = side == 0 ? 2 * NI : 0;  // stencil entries towards plane q
-            for (int idx = tid; idx < ncol * m; idx += kPlaneThreads) {
-                const int i = idx / ncol, jl = idx - i * ncol;
-                const int j = c0 + jl, uj = j / bd, mj = j - uj * bd;
-                double v = 0.0;
+            for (int jl = warp; jl < ncol; jl += kWarps) {
+                const int j = rank + jl * nct, uj = j / bd, mj = j - uj * bd;
                 // rows s of plane k with C_{k,q}[s][j] != 0: the in-plane neighbours of uj
-                for (int a = 0; a < NI; ++a) {
-                    const int us = plane_nbr(G, uj, a);
-                    if (us < 0) continue;
-                    const int qq = plane_offset(G, us, uj) + qb;
-                    for (int ls = 0; ls < bd; ++ls) {
-                        const double u = st_val(Acs, G, Jbase + us, qq, ls, mj);
+                if (lane < NI * bd) {
+                    const int a = lane / bd, ls = lane - a * bd, us = plane_nbr(G, uj, a);
+                    double u = 0.0;
+                    unsigned at = ~0u;
+                    if (us >= 0) {
                         const int cc = pinv[us * bd + ls];
-                        const int ow = cc / cw;
-                        const double *xc = cluster.map_shared_rank(Sown, ow) + (long)(cc - ow * cw) * m;
-                        v = fma(xc[i], u, v);
+                        u = st_val(Acs, G, Jbase + us, plane_offset(G, us, uj) + qb, ls, mj);
+                        at = map_rank(Sown + (long)(cc / nct) * m, cc % nct);
                     }
+                    s_gval[warp][lane] = u;
+                    s_gcol[warp][lane] = at;  // ~0: no such row
                 }
-                Gk[(long)i * m + j] = v;
+                __syncwarp();
+                for (int i = lane; i < m; i += 32) {
+                    double v = 0.0;
+                    for (int e0 = 0; e0 < NI * bd; e0 += 9) {
+                        double x[9];
+#pragma unroll
+                        for (int e = 0; e < 9; ++e) {
+                            const unsigned at = e0 + e < NI * bd ? s_gcol[warp][e0 + e] : ~0u;
+                            x[e] = at != ~0u ? ld_rank(at + 8u * i) : 0.0;
+                        }
+#pragma unroll
+                        for (int e = 0; e < 9; ++e)
+                            if (e0 + e < NI * bd && s_gcol[warp][e0 + e] != ~0u) v = fma(x[e], s_gval[warp][e0 + e], v);
+                    }
+                    if (keep) Gown[(long)jl * m + i] = v;
+                    Gk[(long)i * m + j] = v;
+                }
+                __syncwarp();
             }
         }
         cluster.sync();  // remote reads of this plane's X columns are done before they are overwritten
     }
+}
+
+using PlaneFactorFn = void (*)(PlaneGeom, int, int, int, const double *, double *, double *, int *, int *);
+// the instance whose lanes hold a column of m rows
+static PlaneFactorFn plane_factor_fn(int m) {
+    return m <= 64 ? plane_factor_kernel<2> : m <= 128 ? plane_factor_kernel<4> : m <= 256 ? plane_factor_kernel<8>
+           : m <= 384 ? plane_factor_kernel<12> : plane_factor_kernel<24>;
 }
 
 // Application w = A_c^-1 v through the plane factors, in three launches
@@ -513,9 +702,9 @@ __global__ void __launch_bounds__(kPlaneThreads) plane_inverse_kernel(PlaneGeom 
 
 // ---- host side ----------------------------------------------------------------------
 
-static size_t factor_smem(int m, int nct) {
-    const int cw = (m + nct - 1) / nct;
-    return (size_t)cw * m * sizeof(double) + 3 * (size_t)m * sizeof(double) + 3 * (size_t)m * sizeof(int);
+static size_t factor_smem(int m, int nct, bool keep) {
+    const size_t cols = (size_t)((m + nct - 1) / nct) * m * sizeof(double);
+    return (keep ? 2 : 1) * cols + 3 * (size_t)m * sizeof(double) + 3 * (size_t)m * sizeof(int);
 }
 static size_t solve_smem(int m) { return 4 * (size_t)m * sizeof(double); }
 // with the staged copies (see plane_solve_kernel)
@@ -527,7 +716,8 @@ static size_t solve_smem_staged(const PlaneGeom &G, int nct) {
 
 constexpr size_t kPlaneSmemMax = 220 * 1024;
 
-static cudaLaunchConfig_t cluster_cfg(cudaLaunchAttribute *attr, int nct, size_t smem, cudaStream_t s, bool pdl) {
+static cudaLaunchConfig_t cluster_cfg(cudaLaunchAttribute *attr, int nct, size_t smem, cudaStream_t s, bool pdl,
+                                      int threads = kPlaneThreads) {
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = nct;
     attr[0].val.clusterDim.y = 1;
@@ -536,7 +726,7 @@ static cudaLaunchConfig_t cluster_cfg(cudaLaunchAttribute *attr, int nct, size_t
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(nct);
-    cfg.blockDim = dim3(kPlaneThreads);
+    cfg.blockDim = dim3(threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cfg.attrs = attr;
@@ -551,13 +741,16 @@ static int plane_cluster(int m) {
     static int cap = 0;  // set once per process; the attributes are per function
     static std::once_flag once;
     std::call_once(once, [] {
-        cap = 8;
-        if (cudaFuncSetAttribute(plane_factor_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) ==
-                cudaSuccess &&
-            cudaFuncSetAttribute(plane_solve_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) ==
-                cudaSuccess)
-            cap = 16;
-        cudaFuncSetAttribute(plane_factor_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPlaneSmemMax);
+        bool wide = true;  // non-portable cluster sizes
+        for (int rows : {64, 128, 256, 384, kPlaneMaxRows}) {
+            wide = cudaFuncSetAttribute(plane_factor_fn(rows), cudaFuncAttributeNonPortableClusterSizeAllowed, 1) ==
+                       cudaSuccess && wide;
+            cudaFuncSetAttribute(plane_factor_fn(rows), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)kPlaneSmemMax);
+        }
+        wide = cudaFuncSetAttribute(plane_solve_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) ==
+                   cudaSuccess && wide;
+        cap = wide ? kPlaneMaxCluster : 8;
         cudaFuncSetAttribute(plane_solve_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPlaneSmemMax);
         cudaGetLastError();
     });
@@ -565,13 +758,13 @@ static int plane_cluster(int m) {
     for (int nct = cap; nct >= 1; nct >>= 1) {
         if (nct > m) continue;
         const int cw = (m + nct - 1) / nct;
-        const size_t sf = factor_smem(m, nct);
-        if (cw > kPlaneMaxCols || sf > kPlaneSmemMax) return 0;  // smaller clusters need more per CTA
+        const size_t sf = factor_smem(m, nct, false);
+        if (cw > kPlaneMaxCols || m > kPlaneMaxRows || sf > kPlaneSmemMax) return 0;  // smaller clusters need more per CTA
         cudaLaunchAttribute attr[2];
-        cudaLaunchConfig_t cf = cluster_cfg(attr, nct, sf, nullptr, false);
+        cudaLaunchConfig_t cf = cluster_cfg(attr, nct, sf, nullptr, false, kFactorThreads);
         cudaLaunchConfig_t cs = cluster_cfg(attr, nct, solve_smem(m), nullptr, false);
         int nf = 0, ns = 0;
-        if (cudaOccupancyMaxActiveClusters(&nf, plane_factor_kernel, &cf) != cudaSuccess ||
+        if (cudaOccupancyMaxActiveClusters(&nf, plane_factor_fn(m), &cf) != cudaSuccess ||
             cudaOccupancyMaxActiveClusters(&ns, plane_solve_kernel, &cs) != cudaSuccess) {
             cudaGetLastError();
             continue;
@@ -629,19 +822,29 @@ msrsb_status plane_factor(int dim, const int nb[3], int bd, const double *Acs, C
     int *status = nullptr;
     MSRSB_TRY(dalloc(&status, 1, s));
     MSRSB_CUDA(cudaMemsetAsync(status, 0, sizeof(int), s));
-    const size_t sf = factor_smem(G.m, nct);
+    int keep = 0;  // the sides keep their last G_k's columns where shared memory allows it
+    {
+        cudaLaunchAttribute a2[2];
+        const size_t sk = factor_smem(G.m, nct, true);
+        cudaLaunchConfig_t ck = cluster_cfg(a2, nct, sk, nullptr, false, kFactorThreads);
+        int nk = 0;
+        if (sk <= kPlaneSmemMax && cudaOccupancyMaxActiveClusters(&nk, plane_factor_fn(G.m), &ck) == cudaSuccess && nk > 0)
+            keep = 1;
+        cudaGetLastError();
+    }
+    const size_t sf = factor_smem(G.m, nct, keep), sfm = factor_smem(G.m, nct, false);
     if (h > 0) {  // the two sides, one cluster each, concurrently
         cudaLaunchAttribute attr[2];
-        cudaLaunchConfig_t cfg = cluster_cfg(attr, nct, sf, s, false);
+        cudaLaunchConfig_t cfg = cluster_cfg(attr, nct, sf, s, false, kFactorThreads);
         cfg.gridDim = dim3((G.np - 1 - h > 0 ? 2 : 1) * nct);
         count_launch();
-        MSRSB_CUDA(cudaLaunchKernelEx(&cfg, plane_factor_kernel, G, h, 0, Acs, cp->X, cp->G, cp->pi, status));
+        MSRSB_CUDA(cudaLaunchKernelEx(&cfg, plane_factor_fn(G.m), G, h, 0, keep, Acs, cp->X, cp->G, cp->pi, status));
     }
     {  // the middle plane
         cudaLaunchAttribute attr[2];
-        cudaLaunchConfig_t cfg = cluster_cfg(attr, nct, sf, s, false);
+        cudaLaunchConfig_t cfg = cluster_cfg(attr, nct, sfm, s, false, kFactorThreads);
         count_launch();
-        MSRSB_CUDA(cudaLaunchKernelEx(&cfg, plane_factor_kernel, G, h, 1, Acs, cp->X, cp->G, cp->pi, status));
+        MSRSB_CUDA(cudaLaunchKernelEx(&cfg, plane_factor_fn(G.m), G, h, 1, 0, Acs, cp->X, cp->G, cp->pi, status));
     }
     int bad = 0;
     MSRSB_TRY(read_back(&bad, status, sizeof(int), s));
