@@ -144,9 +144,12 @@ template <typename TI, typename TO>
 msrsb_status permute_cast(long N, const TI *x, const int32_t *perm, TO *y, cudaStream_t s);
 template <typename T>
 msrsb_status block_diag_inverse(const msrsb_mat *A, T *dinv, cudaStream_t s);
-template <typename T, typename TA, typename TZ>
-msrsb_status gs_apply(const msrsb_handle *h, const TA *val, const T *dinv, int forward, const T *r, T *e, TZ *z,
-                      int assign, cudaStream_t s);
+template <typename T>
+msrsb_status gs_setup(msrsb_handle *h, cudaStream_t s);
+template <typename T, typename TV, typename TZ>
+msrsb_status gs_sweep(const msrsb_handle *h, int forward, const TV *v, T *x4, TZ *z, cudaStream_t s);
+template <typename T>
+msrsb_status gs_resid(const msrsb_handle *h, const T *x4, T *r, cudaStream_t s);
 template <typename T>
 msrsb_status convert(long n, const double *a, T *b, cudaStream_t s);
 template <typename TA, typename TX, typename TV, typename TY, typename TACC>
@@ -156,7 +159,7 @@ template <typename TP, typename TV>
 msrsb_status restrict_op(const msrsb_handle *h, const TP *P, const TV *v, double *vc, cudaStream_t s);
 template <typename TP, typename TZ>
 msrsb_status prolong_op(const msrsb_handle *h, const TP *P, const double *wc, const float *wc32, TZ *z, float *z32,
-                        int add, cudaStream_t s);
+                        TP *x4, int add, cudaStream_t s);
 template <typename TV>
 msrsb_status mdot(long N, int nvec, const TV *V, long ldv, const TV *w, double *partial, double *out, int accumulate,
                   cudaStream_t s, const int *gate = nullptr);
@@ -218,7 +221,8 @@ static msrsb_status setup_smoother(msrsb_handle *h, cudaStream_t s) {
     h->colour_ptr_h = (int32_t *)calloc(h->ncolours + 1, sizeof(int32_t));
     MSRSB_TRY(colour_classes(n, h->colour, h->ncolours, &h->colour_rows, h->colour_ptr_h, s));
     if (bd == 1) MSRSB_TRY(sell_copy(&A, h->opts.prec == MSRSB_F32, &h->asell, s));
-    if (h->opts.prec == MSRSB_F32 && bd != 1) {
+    // the block Gauss-Seidel sweeps have the blocks in their own layout
+    if (h->opts.prec == MSRSB_F32 && bd != 1 && h->opts.smoother != MSRSB_SMOOTH_GS) {
         float *alo = nullptr;
         MSRSB_TRY(dalloc(&alo, (size_t)A.nnz * bd * bd, s));
         MSRSB_TRY(convert<float>((long)A.nnz * bd * bd, A.val, alo, s));
@@ -259,6 +263,7 @@ static msrsb_status setup_smoother(msrsb_handle *h, cudaStream_t s) {
         MSRSB_TRY(dalloc(&dinv, (size_t)n * 9, s));
         h->dinv = dinv;
         MSRSB_TRY(block_diag_inverse<T>(&A, dinv, s));
+        MSRSB_TRY(gs_setup<T>(h, s));
     } else if (h->opts.smoother == MSRSB_SMOOTH_L1JAC) {
         T *dinv = nullptr;  // reciprocal l1 row norms, [n*bdim]
         MSRSB_TRY(dalloc(&dinv, (size_t)n * bd, s));
@@ -474,7 +479,7 @@ static msrsb_status setup_t(msrsb_handle *h, const void *p_init, cudaStream_t s)
     MSRSB_TRY(dalloc(&h->tmp_d, N, s));
     T *r = nullptr, *y = nullptr;
     MSRSB_TRY(dalloc(&r, N, s));
-    MSRSB_TRY(dalloc(&y, N, s));
+    MSRSB_TRY(dalloc(&y, bd == 3 ? 4 * (size_t)n : (size_t)N, s));
     h->r_t = r;
     h->y_t = y;
     MSRSB_TRY(dalloc(&h->partial, (size_t)kRedBlocksHost * 1024, s));
@@ -548,10 +553,9 @@ static msrsb_status apply_t(msrsb_handle *h, const TVI *v, TZ *z, cudaStream_t s
     // first post-smoothing residual reads (it rounds z to FP32 all the same)
     float *z32 = (coarse && post && (ilu || l1) && sizeof(T) == 4 && sizeof(TZ) == 8) ? h->z32 : nullptr;
     if (pre) {
-        // z = M_pre^-1 v
+        // z = M_pre^-1 v (block Gauss-Seidel: in y, and in z itself where no coarse stage follows)
         if (gs) {
-            MSRSB_TRY((copy_cast<TVI, T>(N, v, r, s)));
-            MSRSB_TRY((gs_apply<T, T, TZ>(h, aval_t, dinv, 1, r, y, z, 1, s)));
+            MSRSB_TRY((gs_sweep<T, TVI, TZ>(h, 1, v, y, coarse ? nullptr : z, s)));
         } else if (ic) {
             MSRSB_TRY((copy_cast<TVI, T>(N, v, r, s)));
             MSRSB_TRY((bic0_apply<T, TZ>(h, (const T *)h->bic_lu, dinv, r, z, 1, s)));
@@ -569,7 +573,8 @@ static msrsb_status apply_t(msrsb_handle *h, const TVI *v, TZ *z, cudaStream_t s
     }
     if (coarse) {
         if (pre) {  // coarse correction of the residual v - A z
-            MSRSB_TRY((resid_t<T, TZ, TVI>(h, aval_t, z, v, r, nullptr, s)));
+            if (gs) MSRSB_TRY((gs_resid<T>(h, y, r, s)));
+            else MSRSB_TRY((resid_t<T, TZ, TVI>(h, aval_t, z, v, r, nullptr, s)));
             MSRSB_TRY((restrict_op<T, T>(h, (const T *)h->pt_val, r, h->vc, s)));
         } else {
             MSRSB_TRY((restrict_op<T, TVI>(h, (const T *)h->pt_val, v, h->vc, s)));
@@ -579,14 +584,14 @@ static msrsb_status apply_t(msrsb_handle *h, const TVI *v, TZ *z, cudaStream_t s
         else
             MSRSB_TRY(plane_solve(h->grid.dim, h->nb, h->bdim, h->Acs, &h->planes, h->vc, h->wc,
                                   sizeof(T) == 4 ? h->wc32 : nullptr, s));
-        MSRSB_TRY((prolong_op<T, TZ>(h, P, h->wc, h->wc32, z, z32, pre ? 1 : 0, s)));
+        MSRSB_TRY((prolong_op<T, TZ>(h, P, h->wc, h->wc32, z, z32, gs ? y : nullptr, pre ? 1 : 0, s)));
     } else if (!pre) {
         MSRSB_CUDA(cudaMemsetAsync(z, 0, N * sizeof(TZ), s));  // smoothing only, from z = 0
+        if (gs) MSRSB_CUDA(cudaMemsetAsync(y, 0, 4 * (size_t)h->n * sizeof(T), s));
     }
     if (post) {
         if (gs) {
-            MSRSB_TRY((resid_t<T, TZ, TVI>(h, aval_t, z, v, r, nullptr, s)));
-            MSRSB_TRY((gs_apply<T, T, TZ>(h, aval_t, dinv, 0, r, y, z, 0, s)));
+            MSRSB_TRY((gs_sweep<T, TVI, TZ>(h, 0, v, y, z, s)));
         } else if (ic) {
             MSRSB_TRY((resid_t<T, TZ, TVI>(h, aval_t, z, v, r, nullptr, s)));
             MSRSB_TRY((bic0_apply<T, TZ>(h, (const T *)h->bic_lu, dinv, r, z, 0, s)));
@@ -1354,6 +1359,8 @@ static void handle_free(msrsb_handle *h) {
     dfree(h->dinv, s);
     dfree(h->bic_lu, s);
     dfree(h->a_lo, s);
+    dfree(h->gs.val, s);
+    dfree(h->gs.col, s);
     sell_free(&h->asell, s);
     dfree(h->vc, s);
     dfree(h->wc, s);

@@ -210,6 +210,16 @@ struct IluEll {
     void *lval = nullptr, *uval = nullptr, *udinv = nullptr;
 };
 
+// Blocks of the block Gauss-Seidel sweeps by colour (see gs.cu): per row of a
+// colour ng groups of blocks, the first ge of them towards earlier colours.
+struct GsEll {
+    int ncol = 0;
+    int ge[8] = {0}, ng[8] = {0};
+    long base[8] = {0};  // first group of each colour
+    void *val = nullptr;
+    int32_t *col = nullptr;
+};
+
 // ILU(0) factors in the line-block order: positions by colour, block, line,
 // x; the coefficients by neighbour line and x offset (see ilu_lines.cu).
 // Index 0: L (earlier in the order), 1: U.
@@ -323,6 +333,7 @@ struct msrsb_handle {
     // smoother factors in A's (block) pattern, handle precision
     msrsb::IluEll ilu;          // ILU(0) factors (colour order), handle precision
     msrsb::IluLines lines;      // ILU(0) factors (line-block order), handle precision
+    msrsb::GsEll gs;            // block Gauss-Seidel, handle precision
     int use_lines = 0;          // the ILU(0) smoother uses the line-block order
     int32_t *pos_of = nullptr;  // colour-order position of every fine row
     int32_t *diag_pos = nullptr;
@@ -334,7 +345,7 @@ struct msrsb_handle {
     double *vc = nullptr, *wc = nullptr, *tmp_d = nullptr;
     float *wc32 = nullptr;  // FP32 copy of w_c (FP32 prolongation)
     float *z32 = nullptr;   // FP32 copy of z after the coarse stage (scalar mixed form)
-    void *r_t = nullptr, *y_t = nullptr;
+    void *r_t = nullptr, *y_t = nullptr;  // y_t: padded to four components a node for the block Gauss-Seidel
     // Krylov workspace
     double *kv = nullptr, *kz = nullptr;   // GMRES V [(m+1)][N], Z [m][N]; PCG uses first columns
     void *kv32 = nullptr;                  // double-float GMRES basis of the mixed form: hi, lo planes

@@ -561,7 +561,7 @@ template msrsb_status ilu0_apply<double, double>(const msrsb_handle *, double *,
 template msrsb_status ilu0_apply<float, double>(const msrsb_handle *, float *, double *, cudaStream_t);
 template msrsb_status ilu0_apply<float, float>(const msrsb_handle *, float *, float *, cudaStream_t);
 
-// ---- block (3x3) Gauss-Seidel -------------------------------------------------
+// ---- block diagonal inverses of the block Gauss-Seidel (sweeps: gs.cu) ---------
 
 // inverse of every 3x3 diagonal block (FP64, adjugate / determinant)
 template <typename T>
@@ -611,68 +611,6 @@ msrsb_status block_diag_inverse(const msrsb_mat *A, T *dinv, cudaStream_t s) {
 }
 template msrsb_status block_diag_inverse<double>(const msrsb_mat *, double *, cudaStream_t);
 template msrsb_status block_diag_inverse<float>(const msrsb_mat *, float *, cudaStream_t);
-
-// one colour of a block Gauss-Seidel sweep: e_i = Dinv_i (r_i - sum_{k in
-// earlier colours of this sweep} A_ik e_k); z_i += e_i (or z_i = e_i)
-template <typename T, typename TA, typename TZ>
-__global__ void gs_colour_kernel(int cnt, const int32_t *__restrict__ rows, int c, int forward,
-                                 const int32_t *__restrict__ rowptr, const int32_t *__restrict__ colidx,
-                                 const uint8_t *__restrict__ colour, const TA *__restrict__ val,
-                                 const T *__restrict__ dinv, const T *__restrict__ r, T *__restrict__ e,
-                                 TZ *__restrict__ z, int assign) {
-    pdl_prologue();
-    int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= cnt) return;
-    int i = rows[t];
-    T a0 = r[3 * i], a1 = r[3 * i + 1], a2 = r[3 * i + 2];
-    for (int q = rowptr[i]; q < rowptr[i + 1]; ++q) {
-        int k = colidx[q];
-        int ck = colour[k];
-        if (forward ? ck >= c : ck <= c) continue;
-        const TA *b = val + (long)q * 9;
-        T e0 = e[3 * k], e1 = e[3 * k + 1], e2 = e[3 * k + 2];
-        a0 -= T(b[0]) * e0 + T(b[1]) * e1 + T(b[2]) * e2;
-        a1 -= T(b[3]) * e0 + T(b[4]) * e1 + T(b[5]) * e2;
-        a2 -= T(b[6]) * e0 + T(b[7]) * e1 + T(b[8]) * e2;
-    }
-    const T *d = dinv + (long)i * 9;
-    T x0 = d[0] * a0 + d[1] * a1 + d[2] * a2;
-    T x1 = d[3] * a0 + d[4] * a1 + d[5] * a2;
-    T x2 = d[6] * a0 + d[7] * a1 + d[8] * a2;
-    e[3 * i] = x0;
-    e[3 * i + 1] = x1;
-    e[3 * i + 2] = x2;
-    if (assign) {
-        z[3 * i] = TZ(x0);
-        z[3 * i + 1] = TZ(x1);
-        z[3 * i + 2] = TZ(x2);
-    } else {
-        z[3 * i] = TZ(z[3 * i] + TZ(x0));
-        z[3 * i + 1] = TZ(z[3 * i + 1] + TZ(x1));
-        z[3 * i + 2] = TZ(z[3 * i + 2] + TZ(x2));
-    }
-}
-
-template <typename T, typename TA, typename TZ>
-msrsb_status gs_apply(const msrsb_handle *h, const TA *val, const T *dinv, int forward, const T *r, T *e, TZ *z,
-                      int assign, cudaStream_t s) {
-    const msrsb_mat &A = h->A;
-    for (int q = 0; q < h->ncolours; ++q) {
-        int c = forward ? q : h->ncolours - 1 - q;
-        int cnt = h->colour_ptr_h[c + 1] - h->colour_ptr_h[c];
-        if (!cnt) continue;
-        MSRSB_PDL((gs_colour_kernel<T, TA, TZ>), ceil_div(cnt, 128), 128, 0, s, cnt,
-                  h->colour_rows + h->colour_ptr_h[c], c, forward, A.rowptr, A.colidx, h->colour, val, dinv, r, e, z,
-                  assign);
-    }
-    return MSRSB_OK;
-}
-template msrsb_status gs_apply<double, double, double>(const msrsb_handle *, const double *, const double *, int,
-                                                       const double *, double *, double *, int, cudaStream_t);
-template msrsb_status gs_apply<float, float, double>(const msrsb_handle *, const float *, const float *, int,
-                                                     const float *, float *, double *, int, cudaStream_t);
-template msrsb_status gs_apply<float, float, float>(const msrsb_handle *, const float *, const float *, int,
-                                                    const float *, float *, float *, int, cudaStream_t);
 
 // ---- block incomplete factorisation: IC(0) of Sec. 4.1 and 4.3 -------------------------
 //
