@@ -160,9 +160,6 @@ msrsb_status restrict_op(const msrsb_handle *h, const TP *P, const TV *v, double
 template <typename TP, typename TZ>
 msrsb_status prolong_op(const msrsb_handle *h, const TP *P, const double *wc, const float *wc32, TZ *z, float *z32,
                         TP *x4, int add, cudaStream_t s);
-template <typename TV>
-msrsb_status mdot(long N, int nvec, const TV *V, long ldv, const TV *w, double *partial, double *out, int accumulate,
-                  cudaStream_t s, const int *gate = nullptr);
 msrsb_status norm2(long N, const double *w, double *partial, double *out, cudaStream_t s);
 msrsb_status mvsub(long N, int nvec, const double *V, long ldv, const double *h, double *w, cudaStream_t s);
 template <typename TZ>
@@ -199,9 +196,10 @@ bool lines_multi_fit(const msrsb_handle *h);
 msrsb_status df_split(long N, const double *w, float *wh, float *wl, cudaStream_t s);
 template <typename TY>
 msrsb_status scale_by_inv(long N, const double *x, const double *den, TY *y, cudaStream_t s);
-msrsb_status axpy_dev(long N, const double *num, const double *den, double sign, const double *x, double *y,
-                      cudaStream_t s);
-msrsb_status xpay_dev(long N, const double *num, const double *den, const double *z, double *p, cudaStream_t s);
+msrsb_status pcg_dot(long N, int what, const double *a, const double *b, double *partial, double *sc, cudaStream_t s);
+msrsb_status pcg_update(long N, const double *p, const double *q, double *x, double *r, double *partial, double *sc,
+                        cudaStream_t s);
+msrsb_status pcg_direction(long N, const double *sc, const double *z, double *p, cudaStream_t s);
 template <typename TI, typename TO>
 msrsb_status copy_cast(long N, const TI *x, TO *y, cudaStream_t s);
 double *pinned_scratch();
@@ -1249,7 +1247,7 @@ static msrsb_status pcg(msrsb_handle *h, const double *b, double *x, double rtol
                         double *relres, double *hist, cudaStream_t s) {
     const long N = (long)h->n * h->bdim;
     double *r = h->kv, *zv = h->kv + N, *p = h->kv + 2 * N, *q = h->kv + 3 * N;
-    double *sc = h->kh;  // [0] |b| [1] rz [2] rz_new [3] pq [4] |r|
+    double *sc = h->kh;  // [0] |b| [1] r.z [4] |r| [5] r.z / p.q [6] the directions' ratio of r.z
     double bnorm = 0.0;
     MSRSB_TRY(norm2(N, b, h->partial, sc + 0, s));
     MSRSB_TRY(read_scalar(sc + 0, &bnorm, s));
@@ -1263,15 +1261,13 @@ static msrsb_status pcg(msrsb_handle *h, const double *b, double *x, double rtol
     MSRSB_TRY(fine_spmv(h, x, b, r, true, s));
     MSRSB_TRY(apply_any(h, r, zv, s));
     MSRSB_CUDA(cudaMemcpyAsync(p, zv, N * sizeof(double), cudaMemcpyDeviceToDevice, s));
-    MSRSB_TRY(mdot(N, 1, r, N, zv, h->partial, sc + 1, 0, s));
+    MSRSB_TRY(pcg_dot(N, 3, r, zv, h->partial, sc, s));
     int its = 0;
     for (;;) {
         MSRSB_TRY(fine_spmv(h, p, nullptr, q, false, s));
-        MSRSB_TRY(mdot(N, 1, p, N, q, h->partial, sc + 3, 0, s));
-        MSRSB_TRY(axpy_dev(N, sc + 1, sc + 3, 1.0, p, x, s));
-        MSRSB_TRY(axpy_dev(N, sc + 1, sc + 3, -1.0, q, r, s));
+        MSRSB_TRY(pcg_dot(N, 0, p, q, h->partial, sc, s));
+        MSRSB_TRY(pcg_update(N, p, q, x, r, h->partial, sc, s));
         ++its;
-        MSRSB_TRY(norm2(N, r, h->partial, sc + 4, s));
         double rn = 0.0;
         MSRSB_TRY(read_scalar(sc + 4, &rn, s));
         if (hist) hist[its] = rn / bnorm;
@@ -1291,9 +1287,8 @@ static msrsb_status pcg(msrsb_handle *h, const double *b, double *x, double rtol
             return fail(MSRSB_ENOCONV, "PCG reached %d iterations (relres %.3e)", its, rn / bnorm);
         }
         MSRSB_TRY(apply_any(h, r, zv, s));
-        MSRSB_TRY(mdot(N, 1, r, N, zv, h->partial, sc + 2, 0, s));
-        MSRSB_TRY(xpay_dev(N, sc + 2, sc + 1, zv, p, s));
-        MSRSB_CUDA(cudaMemcpyAsync(sc + 1, sc + 2, sizeof(double), cudaMemcpyDeviceToDevice, s));
+        MSRSB_TRY(pcg_dot(N, 1, r, zv, h->partial, sc, s));
+        MSRSB_TRY(pcg_direction(N, sc, zv, p, s));
     }
     *iters = its;
     return MSRSB_OK;
