@@ -97,8 +97,8 @@ void coarse_extent(const msrsb_grid *g, int nb[3]);
 msrsb_status stencil_to_dense(int dim, const int nb[3], int bd, const double *Acs, double *dense, cudaStream_t s);
 bool planes_fit(int dim, const int nb[3], int bd);
 msrsb_status plane_factor(int dim, const int nb[3], int bd, const double *Acs, CoarsePlanes *cp, cudaStream_t s);
-msrsb_status plane_solve(int dim, const int nb[3], int bd, const double *Acs, const CoarsePlanes *cp,
-                         const double *vc, double *wc, float *wc32, cudaStream_t s);
+msrsb_status plane_couplings(int dim, const int nb[3], int bd, const double *Acs, CoarsePlanes *cp, cudaStream_t s);
+msrsb_status plane_solve(const CoarsePlanes *cp, const double *vc, double *wc, float *wc32, cudaStream_t s);
 void plane_free(CoarsePlanes *cp, cudaStream_t s);
 msrsb_status plane_inverse(int dim, const int nb[3], int bd, const double *Acs, const CoarsePlanes *cp, double *Ainv,
                            cudaStream_t s);
@@ -435,6 +435,8 @@ static msrsb_status setup_t(msrsb_handle *h, const void *p_init, cudaStream_t s)
             MSRSB_TRY(dalloc(&h->Ainv, (size_t)h->nC * h->nC, s));
             MSRSB_TRY(plane_inverse(h->grid.dim, h->nb, bd, h->Acs, &h->planes, h->Ainv, s));
             plane_free(&h->planes, s);
+        } else {
+            MSRSB_TRY(plane_couplings(h->grid.dim, h->nb, bd, h->Acs, &h->planes, s));
         }
     } else {
         if (h->nC > 8192)
@@ -561,8 +563,7 @@ static msrsb_status apply_t(msrsb_handle *h, const TVI *v, TZ *z, cudaStream_t s
         if (h->Ainv)
             MSRSB_TRY(gemv(h->nC, h->Ainv, h->vc, h->wc, sizeof(T) == 4 ? h->wc32 : nullptr, s));
         else
-            MSRSB_TRY(plane_solve(h->grid.dim, h->nb, h->bdim, h->Acs, &h->planes, h->vc, h->wc,
-                                  sizeof(T) == 4 ? h->wc32 : nullptr, s));
+            MSRSB_TRY(plane_solve(&h->planes, h->vc, h->wc, sizeof(T) == 4 ? h->wc32 : nullptr, s));
         MSRSB_TRY((prolong_op<T, TZ>(h, P, h->wc, h->wc32, z, z32, gs ? y : nullptr, pre ? 1 : 0, s)));
     } else if (!pre) {
         MSRSB_CUDA(cudaMemsetAsync(z, 0, N * sizeof(TZ), s));  // smoothing only, from z = 0
@@ -987,7 +988,7 @@ static msrsb_status apply_multi_t(msrsb_handle *h, int k, const TVI *const *v, T
         MSRSB_TRY(gemm_multi(h->nC, k, h->Ainv, vcr, wc, wc32, s));
     } else {
         for (int c = 0; c < k; ++c)
-            MSRSB_TRY(plane_solve(h->grid.dim, h->nb, h->bdim, h->Acs, &h->planes, vc.p[c], wc.p[c], wc32.p[c], s));
+            MSRSB_TRY(plane_solve(&h->planes, vc.p[c], wc.p[c], wc32.p[c], s));
     }
     MSRSB_TRY((prolong_multi<T, TZ>(h, k, (const T *)h->p_val, wcr, wc32r, zo, z32, s)));
     if constexpr (sizeof(T) == 4) {

@@ -24,7 +24,7 @@
 // integer order of their FP64 bit patterns). Both the factorisation and the
 // application run as thread-block clusters (up to 16 CTAs on 16 SMs) whose
 // CTAs own columns (factorisation, dealt out in turn) or contiguous rows
-// (application) and exchange pivot columns and partial vectors through
+// (application, see there) and exchange pivot columns and partial vectors through
 // distributed shared memory, with hardware cluster barriers between steps (no
 // spin waits).
 #include "common.cuh"
@@ -480,143 +480,210 @@ static PlaneFactorFn plane_factor_fn(int m) {
            : m <= 384 ? plane_factor_kernel<12> : plane_factor_kernel<24>;
 }
 
-// Application w = A_c^-1 v through the plane factors, in three launches
-// (phase): 0: the two sides' forward sweeps, y_k = X_k Pi_k (v_k - C y_p)
-// with p the plane before k on its side (side 0: planes 0 .. h-1, p = k-1;
-// side 1: planes np-1 .. h+1, p = k+1), one cluster each; 1: the middle
-// plane, w_h = X_h Pi_h (v_h - C y_{h-1} - C y_{h+1}); 2: the back
-// substitution outwards, w_k = y_k - G_k w_q (q = k+1 on side 0, k-1 on
-// side 1). vc, wc: FP64 [np*m] in coarse dof order (y is kept in wc); wc32
-// (nullable) an FP32 copy of w. With stage set, every step's own rows of its
-// matrix (a contiguous block of the row-major X_k or G_k), the step's
-// couplings and the gather pi_k are copied to shared memory asynchronously
-// two steps ahead (double buffered; they do not depend on the recurrence),
-// so that each step waits only on the cluster barrier and its own arithmetic.
-// the plane of step st of a solve launch (see plane_solve_kernel)
-__device__ __forceinline__ int solve_plane(int phase, int side, int h, int np, int st) {
-    if (phase == 1) return h;
-    if (phase == 0) return side == 0 ? st : np - 1 - st;
-    return side == 0 ? h - 1 - st : h + 1 + st;
+// ---- application w = A_c^-1 v --------------------------------------------------------
+//
+// With H_k = X_k Pi_k C_{k,p} (p the plane before k on its side; the middle plane
+// has one towards each side) beside G_k = X_k Pi_k C_{k,q},
+//   u_k = X_k Pi_k v_k                              all planes at once,
+//   y_k = u_k - H_k y_p                             outwards in, one cluster a side,
+//   w_h = u_h - H_h0 y_{h-1} - H_h1 y_{h+1}         the middle plane,
+//   w_k = y_k - G_k w_q                             inwards out, one cluster a side.
+// The chain's step is then one dense product of a plane. (Applying C to y_p and X_k
+// Pi_k to the result at every step put the couplings, formed by every CTA of the
+// cluster, and the permutation on the chain: 100 us an application at 128^3, 82 at
+// 48^3 elasticity; a solve took 27.3 and 13.0 ms, now 26.0 and 11.2.) What is left
+// of a step is bound by the FP64 pipes of the cluster's 16 SMs, m^2 / 16 FMAs each
+// at one warp's FMA in 19 cycles, beside the row sums and the cluster barrier. A half-warp takes a row: its 16 lanes sum in four
+// steps and store the result into the 16 CTAs, one each.
+
+// pinv[pi_k[i]] = i into shared memory
+__device__ __forceinline__ void plane_pinv(const int *__restrict__ pk, int m, int *pinv) {
+    for (int i = threadIdx.x; i < m; i += blockDim.x) pinv[pk[i]] = i;
 }
 
-__global__ void __launch_bounds__(kPlaneThreads, 1) plane_solve_kernel(PlaneGeom G, int h, int phase,
-                                                                    const double *__restrict__ Acs,
-                                                                    const double *__restrict__ X,
-                                                                    const double *__restrict__ Gm,
-                                                                    const int *__restrict__ pi,
-                                                                    const double *__restrict__ vc,
-                                                                    double *__restrict__ wc, float *__restrict__ wc32,
-                                                                    int stage) {
+constexpr int kPlaneHRows = 16;
+
+// H_k, kPlaneHRows rows a CTA: blockIdx.y = plane, blockIdx.z = 0: the side's H_k
+// (the middle plane: towards h - 1), 1: the middle plane towards h + 1 (plane np of H).
+// A thread's column lists its at most 9 bd entries of C once for all the rows.
+__global__ void __launch_bounds__(256) plane_h_kernel(PlaneGeom G, int h, const double *__restrict__ Acs,
+                                                      const double *__restrict__ X, const int *__restrict__ pi,
+                                                      double *__restrict__ H) {
+    const int m = G.m, bd = G.bd, NI = G.NI, np = G.np, k = blockIdx.y;
+    const int to_prev = blockIdx.z ? 0 : (k <= h);  // couplings towards plane k - 1, else k + 1
+    if (blockIdx.z && k != h) return;
+    const int p = to_prev ? k - 1 : k + 1;
+    if (p < 0 || p >= np) return;
+    const int r0 = blockIdx.x * kPlaneHRows, nr = min(kPlaneHRows, m - r0);
+    extern __shared__ double sm[];
+    double *xs = sm;                                // the CTA's rows of X_k
+    int *pinv = (int *)(xs + (long)kPlaneHRows * m);
+    const double *Xk = X + (long)k * m * m + (long)r0 * m;
+    for (int t = threadIdx.x; t < nr * m; t += blockDim.x) xs[t] = Xk[t];
+    plane_pinv(pi + (long)k * m, m, pinv);
+    __syncthreads();
+    double *Hk = H + (long)(blockIdx.z ? np : k) * m * m + (long)r0 * m;
+    const int qb = to_prev ? 0 : 2 * NI, Jbase = k * G.PN;
+    for (int j = threadIdx.x; j < m; j += blockDim.x) {
+        const int uj = j / bd, mj = j - uj * bd;
+        double acc[kPlaneHRows];
+#pragma unroll
+        for (int r = 0; r < kPlaneHRows; ++r) acc[r] = 0.0;
+        for (int a = 0; a < NI; ++a) {  // rows s of plane k that couple with column j: the neighbours of uj
+            const int us = plane_nbr(G, uj, a);
+            if (us < 0) continue;
+            const int qq = plane_offset(G, us, uj) + qb;
+            for (int ls = 0; ls < bd; ++ls) {
+                const double c = st_val(Acs, G, Jbase + us, qq, ls, mj);
+                const double *x = xs + pinv[us * bd + ls];
+#pragma unroll
+                for (int r = 0; r < kPlaneHRows; ++r)
+                    if (r < nr) acc[r] = fma(x[(long)r * m], c, acc[r]);
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < kPlaneHRows; ++r)
+            if (r < nr) Hk[(long)r * m + j] = acc[r];
+    }
+}
+
+// sum over a half-warp (16 lanes a row), in every lane
+__device__ __forceinline__ double half_sum(double a) {
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+    return a;
+}
+
+constexpr int kPlaneURows = kPlaneThreads / 16;  // rows a CTA of the launches without a chain
+constexpr int kPlaneUPre = 16;   // entries of a row per lane read ahead
+
+// wc_k = u_k = X_k Pi_k v_k; the head of X's rows and pi are loaded before the wait
+__global__ void __launch_bounds__(kPlaneThreads) plane_u_kernel(int m, const double *__restrict__ X,
+                                                                const int *__restrict__ pi,
+                                                                const double *__restrict__ vc,
+                                                                double *__restrict__ wc) {
+    extern __shared__ double sm[];  // Pi_k v_k
+    const int k = blockIdx.y, hl = threadIdx.x & 15, i = blockIdx.x * kPlaneURows + (threadIdx.x >> 4);
+    const double *x = X + (long)k * m * m + (long)min(i, m - 1) * m;
+    double a[kPlaneUPre];
+#pragma unroll
+    for (int t = 0; t < kPlaneUPre; ++t) a[t] = __ldg(x + min(hl + 16 * t, m - 1));
+    const int j0 = threadIdx.x, p0 = j0 < m ? __ldg(pi + (long)k * m + j0) : 0;
+    pdl_prologue();
+    if (j0 < m) sm[j0] = vc[(long)k * m + p0];
+    for (int j = j0 + kPlaneThreads; j < m; j += kPlaneThreads) sm[j] = vc[(long)k * m + pi[(long)k * m + j]];
+    __syncthreads();
+    double s = 0.0;
+#pragma unroll
+    for (int t = 0; t < kPlaneUPre; ++t)
+        if (hl + 16 * t < m) s = fma(a[t], sm[hl + 16 * t], s);
+    for (int j = hl + 16 * kPlaneUPre; j < m; j += 16) s = fma(x[j], sm[j], s);
+    s = half_sum(s);
+    if (hl == 0 && i < m) wc[(long)k * m + i] = s;
+}
+
+// w_h = u_h - H_h0 y_{h-1} - H_h1 y_{h+1}
+__global__ void __launch_bounds__(kPlaneThreads) plane_middle_kernel(int m, int np, int h,
+                                                                     const double *__restrict__ H, double *wc,
+                                                                     float *__restrict__ wc32) {
+    const int hl = threadIdx.x & 15, i = blockIdx.x * kPlaneURows + (threadIdx.x >> 4);
+    const long row = (long)min(i, m - 1) * m;
+    const double *m0 = H + (long)h * m * m + row, *m1 = H + (long)np * m * m + row;
+    double a[kPlaneUPre], b[kPlaneUPre];
+#pragma unroll
+    for (int t = 0; t < kPlaneUPre; ++t) {
+        a[t] = h > 0 ? __ldg(m0 + min(hl + 16 * t, m - 1)) : 0.0;
+        b[t] = h + 1 < np ? __ldg(m1 + min(hl + 16 * t, m - 1)) : 0.0;
+    }
+    pdl_prologue();
+    double s = 0.0;
+    const double *y0 = wc + (long)max(h - 1, 0) * m, *y1 = wc + (long)min(h + 1, np - 1) * m;
+#pragma unroll
+    for (int t = 0; t < kPlaneUPre; ++t) {
+        const int j = hl + 16 * t;
+        if (j < m && h > 0) s = fma(a[t], y0[j], s);
+        if (j < m && h + 1 < np) s = fma(b[t], y1[j], s);
+    }
+#pragma unroll 4
+    for (int j = hl + 16 * kPlaneUPre; j < m; j += 16) {
+        if (h > 0) s = fma(m0[j], y0[j], s);
+        if (h + 1 < np) s = fma(m1[j], y1[j], s);
+    }
+    s = half_sum(s);
+    if (hl == 0 && i < m) {
+        const double w = wc[(long)h * m + i] - s;
+        wc[(long)h * m + i] = w;
+        if (wc32) wc32[(long)h * m + i] = (float)w;
+    }
+}
+
+// One cluster a side. forward: y_k = u_k - H_k y_p over the side's planes after its
+// first (whose y is u); backward: w_k = y_k - G_k w_q from the middle outwards. u, y
+// and w share wc; wc32 (nullable) gets an FP32 copy of w. A CTA owns rw rows of every
+// plane; with `stage` its rows of a step's matrix are copied to shared memory two
+// steps ahead (they do not depend on the chain), so that a step waits only for the
+// cluster barrier and its own products.
+__global__ void __launch_bounds__(kPlaneThreads, 1) plane_chain_kernel(int m, int np, int h, int forward, int stage,
+                                                                     const double *__restrict__ M, double *wc,
+                                                                     float *__restrict__ wc32) {
     cg::cluster_group cluster = cg::this_cluster();
     const int rank = (int)cluster.block_rank(), nct = (int)cluster.num_blocks();
-    const int m = G.m, bd = G.bd, NI = G.NI, np = G.np;
-    const int rw = (m + nct - 1) / nct;
-    const int r0 = rank * rw, r1 = min(m, r0 + rw), nr = max(0, r1 - r0);
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int side = phase == 1 ? 0 : (int)(blockIdx.x / nct);
-    const int nsteps = phase == 1 ? 1 : (side == 0 ? h : np - 1 - h);
-    const bool fwd = phase != 2;
-    const int cb = side == 0 ? 0 : 2 * NI;  // stencil entries towards the plane before (phase 0)
-    const int lowc = NI * bd * bd;  // coupling values per node towards one plane, contiguous in the stencil
-    extern __shared__ double sm[];
-    double *ybuf = sm;          // full plane vector, double buffered [2][m] (written by every CTA)
-    double *t = ybuf + 2 * m;   // right-hand side of the plane [m]
-    double *tp = t + m;         // t gathered by pi [m]
-    double *mat = tp + m;       // staged rows [2][rw*m]
-    double *stc = mat + 2 * (long)rw * m;             // staged couplings [2][PN*lowc]
-    int *spi = (int *)(stc + 2 * (long)G.PN * lowc);  // staged pi [2][m]
-    auto issue = [&](int st, int buf) {
+    const int rw = (m + nct - 1) / nct, r0 = rank * rw, nr = max(0, min(m, r0 + rw) - r0);
+    const int tid = threadIdx.x, hl = tid & 15, warp = tid >> 5, sub = (tid >> 4) & 1;
+    const int side = (int)(blockIdx.x / nct);
+    // planes k0, k0 + dk, ... (nsteps of them), after plane k0 - dk
+    const int dk = (side == 0) == (forward != 0) ? 1 : -1;
+    const int k0 = forward ? (side == 0 ? 1 : np - 2) : (side == 0 ? h - 1 : h + 1);
+    const int nsteps = forward ? (side == 0 ? h - 1 : np - 2 - h) : (side == 0 ? h : np - 1 - h);
+    extern __shared__ __align__(16) double sm[];
+    const int ms = (m + 1) & ~1;
+    double *prev = sm;               // the plane before, double buffered [2][ms] (written by every CTA)
+    double *mat = prev + 2 * ms;     // staged rows [2][rw * m], on a 16-byte boundary
+    const bool wide = (m & 1) == 0;  // rows of whole 16-byte vectors
+    auto issue = [&](int st) {
         if (stage && st < nsteps) {
-            const int k = solve_plane(phase, side, h, np, st);
-            const double *M = (fwd ? X : Gm) + (long)k * m * m + (long)r0 * m;
-            double *dst = mat + (long)buf * rw * m;
-            for (int q = tid; q < nr * m; q += kPlaneThreads) cp_async8(dst + q, M + q);
-            if (fwd) {
-                for (int q = tid; q < m; q += kPlaneThreads) cp_async4(spi + buf * m + q, pi + (long)k * m + q);
-                if (phase == 0 && st > 0) {
-                    double *sd = stc + (long)buf * G.PN * lowc;
-                    const double *src = Acs + (long)k * G.PN * G.nq * bd * bd + (long)cb * bd * bd;
-                    for (int q = tid; q < G.PN * lowc; q += kPlaneThreads) {
-                        const int u = q / lowc, r = q - u * lowc;
-                        cp_async8(sd + q, src + (long)u * G.nq * bd * bd + r);
-                    }
-                }
-            }
+            const double *src = M + (long)(k0 + st * dk) * m * m + (long)r0 * m;
+            double *dst = mat + (long)(st & 1) * rw * m;
+            if (wide)
+                for (int q = tid; q < nr * m / 2; q += kPlaneThreads) cp_async16(dst + 2 * q, src + 2 * q);
+            else
+                for (int q = tid; q < nr * m; q += kPlaneThreads) cp_async8(dst + q, src + q);
         }
         cp_async_commit();  // one group per step, empty or not
     };
-    // the factors are fixed for a solve: the first two steps' copies start
-    // before the wait on the previous kernel
-    issue(0, 0);
-    issue(1, 1);
+    issue(0);
+    issue(1);
     pdl_prologue();
+    if (nsteps > 0)
+        for (int j = tid; j < m; j += kPlaneThreads) prev[j] = wc[(long)(k0 - dk) * m + j];
+    cluster.sync();  // every CTA runs before another stores into its shared memory
+    const int i0 = 2 * warp + sub;  // this half-warp's first row of the CTA's
+    double head = nsteps > 0 && i0 < nr ? wc[(long)k0 * m + r0 + i0] : 0.0;  // its u or y, one step ahead
     for (int st = 0; st < nsteps; ++st) {
-        const int buf = st & 1, k = solve_plane(phase, side, h, np, st);
+        const int buf = st & 1, k = k0 + st * dk;
+        const double *y = prev + buf * ms, *rows = stage ? mat + (long)buf * rw * m : M + (long)k * m * m + (long)r0 * m;
+        const double next = st + 1 < nsteps && i0 < nr ? wc[(long)(k + dk) * m + r0 + i0] : 0.0;
         cp_async_wait<1>();
         __syncthreads();
-        const double *Mrows = stage ? mat + (long)buf * rw * m : nullptr;
-        const int Jbase = k * G.PN;
-        double *ynew = ybuf + buf * m;
-        const double *yprev = ybuf + (buf ^ 1) * m;
-        if (fwd) {  // ---- y_k = X_k Pi_k (v_k - couplings) ----
-            const double *sl = stc + (long)buf * G.PN * lowc;
-            for (int j = tid; j < m; j += kPlaneThreads) {
-                const int uj = j / bd, l = j - uj * bd;
-                double v = vc[(long)(Jbase + uj) * bd + l];
-                if (phase == 0 && st > 0) {  // the plane before, from the previous step
-                    for (int b = 0; b < NI; ++b) {
-                        const int tn = plane_nbr(G, uj, b);
-                        if (tn < 0) continue;
-                        for (int c = 0; c < bd; ++c) {
-                            const double a = stage ? sl[(long)uj * lowc + (b * bd + l) * bd + c]
-                                                   : st_val(Acs, G, Jbase + uj, b + cb, l, c);
-                            v = fma(-a, yprev[tn * bd + c], v);
-                        }
-                    }
-                } else if (phase == 1) {  // both neighbour planes' y, from the sweeps' output
-                    if (h > 0) v = sub_coupling(v, G, Acs, Jbase + uj, uj, l, 0, wc + (long)(h - 1) * G.PN * bd, 1);
-                    if (h + 1 < np)
-                        v = sub_coupling(v, G, Acs, Jbase + uj, uj, l, 2 * NI, wc + (long)(h + 1) * G.PN * bd, 1);
-                }
-                t[j] = v;
-            }
-            __syncthreads();
-            const int *pk = stage ? spi + buf * m : pi + (long)k * m;
-            for (int j = tid; j < m; j += kPlaneThreads) tp[j] = t[pk[j]];
-            __syncthreads();
-            const double *Xk = X + (long)k * m * m;
-            for (int i = r0 + warp; i < r1; i += kPlaneThreads / 32) {
-                const double *xr = stage ? Mrows + (long)(i - r0) * m : Xk + (long)i * m;
-                double s = 0.0;
-                for (int j = lane; j < m; j += 32) s = fma(xr[j], tp[j], s);
-                s = warp_sum(s);
-                if (lane == 0) {
-                    for (int r = 0; r < nct; ++r) cluster.map_shared_rank(ynew, r)[i] = s;
-                    const long q = (long)(Jbase + i / bd) * bd + i % bd;
-                    wc[q] = s;
-                    if (wc32 && phase == 1) wc32[q] = (float)s;
-                }
-            }
-        } else {  // ---- w_k = y_k - G_k w_q ----
-            const int kq = side == 0 ? k + 1 : k - 1;
-            const double *Gk = Gm + (long)k * m * m;
-            const double *wq = st > 0 ? yprev : wc + (long)kq * G.PN * bd;  // w_h from the middle launch
-            for (int i = r0 + warp; i < r1; i += kPlaneThreads / 32) {
-                const double *gr = stage ? Mrows + (long)(i - r0) * m : Gk + (long)i * m;
-                double s = 0.0;
-                for (int j = lane; j < m; j += 32) s = fma(gr[j], wq[j], s);
-                s = warp_sum(s);
-                if (lane == 0) {
-                    const long q = (long)(Jbase + i / bd) * bd + i % bd;
-                    const double w = wc[q] - s;
-                    for (int r = 0; r < nct; ++r) cluster.map_shared_rank(ynew, r)[i] = w;
-                    wc[q] = w;
-                    if (wc32) wc32[q] = (float)w;
+        for (int q = i0; q - sub < nr; q += 2 * (kPlaneThreads / 32)) {
+            const bool has = q < nr;
+            const double base = q == i0 ? head : has ? wc[(long)k * m + r0 + q] : 0.0;
+            const double *row = rows + (long)min(q, nr - 1) * m;
+            double s = 0.0;
+#pragma unroll 4
+            for (int j = hl; j < m; j += 16) s = fma(row[j], y[j], s);
+            const double w = base - half_sum(s);
+            if (has) {  // 16 lanes a row, a destination each
+                if (hl < nct) st_rank(map_rank(prev + (buf ^ 1) * ms + r0 + q, hl), w);
+                if (hl == 0) {
+                    wc[(long)k * m + r0 + q] = w;
+                    if (wc32 && !forward) wc32[(long)k * m + r0 + q] = (float)w;
                 }
             }
         }
-        __syncthreads();  // this step's staged buffers are no longer read
-        issue(st + 2, buf);
+        head = next;
+        __syncthreads();  // this step's staged rows are no longer read
+        issue(st + 2);
         cluster.sync();
     }
     asm volatile("cp.async.wait_all;" ::: "memory");
@@ -626,7 +693,7 @@ __global__ void __launch_bounds__(kPlaneThreads, 1) plane_solve_kernel(PlaneGeom
 // for coarse systems small enough that one dense product per application
 // beats the dependent plane steps: CTA b builds the columns
 // kInvCols*b .. kInvCols*b + kInvCols-1, the same recurrences as
-// plane_solve_kernel applied to identity columns, independent across CTAs.
+// the factored application on identity columns, independent across CTAs.
 constexpr int kInvCols = 4;
 
 // W_k = X_k Pi_k (e_k - C_{k,pa} W_pa - C_{k,pb} W_pb) for the CTA's columns
@@ -706,12 +773,11 @@ static size_t factor_smem(int m, int nct, bool keep) {
     const size_t cols = (size_t)((m + nct - 1) / nct) * m * sizeof(double);
     return (keep ? 2 : 1) * cols + 3 * (size_t)m * sizeof(double) + 3 * (size_t)m * sizeof(int);
 }
-static size_t solve_smem(int m) { return 4 * (size_t)m * sizeof(double); }
-// with the staged copies (see plane_solve_kernel)
-static size_t solve_smem_staged(const PlaneGeom &G, int nct) {
-    const int rw = (G.m + nct - 1) / nct;
-    return solve_smem(G.m) + 2 * (size_t)rw * G.m * sizeof(double) +
-           2 * (size_t)G.PN * G.NI * G.bd * G.bd * sizeof(double) + 2 * (size_t)G.m * sizeof(int);
+static size_t solve_smem(int m) { return 2 * (size_t)(m + 1) * sizeof(double); }
+// with the staged rows (see plane_chain_kernel)
+static size_t solve_smem_staged(int m, int nct) {
+    const int rw = (m + nct - 1) / nct;
+    return solve_smem(m) + 2 * (size_t)rw * m * sizeof(double);
 }
 
 constexpr size_t kPlaneSmemMax = 220 * 1024;
@@ -748,10 +814,11 @@ static int plane_cluster(int m) {
             cudaFuncSetAttribute(plane_factor_fn(rows), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)kPlaneSmemMax);
         }
-        wide = cudaFuncSetAttribute(plane_solve_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) ==
+        wide = cudaFuncSetAttribute(plane_chain_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) ==
                    cudaSuccess && wide;
         cap = wide ? kPlaneMaxCluster : 8;
-        cudaFuncSetAttribute(plane_solve_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPlaneSmemMax);
+        cudaFuncSetAttribute(plane_chain_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPlaneSmemMax);
+        cudaFuncSetAttribute(plane_h_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPlaneSmemMax);
         cudaGetLastError();
     });
     if (m < 1 || solve_smem(m) > kPlaneSmemMax) return 0;
@@ -765,7 +832,7 @@ static int plane_cluster(int m) {
         cudaLaunchConfig_t cs = cluster_cfg(attr, nct, solve_smem(m), nullptr, false);
         int nf = 0, ns = 0;
         if (cudaOccupancyMaxActiveClusters(&nf, plane_factor_fn(m), &cf) != cudaSuccess ||
-            cudaOccupancyMaxActiveClusters(&ns, plane_solve_kernel, &cs) != cudaSuccess) {
+            cudaOccupancyMaxActiveClusters(&ns, plane_chain_kernel, &cs) != cudaSuccess) {
             cudaGetLastError();
             continue;
         }
@@ -804,12 +871,12 @@ msrsb_status plane_factor(int dim, const int nb[3], int bd, const double *Acs, C
     cp->nct = nct;
     cp->stage = 0;
     {  // staged application where its shared memory fits and the cluster can be scheduled with it
-        const size_t ss = solve_smem_staged(G, nct);
+        const size_t ss = solve_smem_staged(G.m, nct);
         if (ss <= kPlaneSmemMax) {
             cudaLaunchAttribute a2[2];
             cudaLaunchConfig_t cs = cluster_cfg(a2, nct, ss, nullptr, false);
             int ns = 0;
-            if (cudaOccupancyMaxActiveClusters(&ns, plane_solve_kernel, &cs) == cudaSuccess && ns > 0) cp->stage = 1;
+            if (cudaOccupancyMaxActiveClusters(&ns, plane_chain_kernel, &cs) == cudaSuccess && ns > 0) cp->stage = 1;
             cudaGetLastError();
         }
     }
@@ -853,32 +920,43 @@ msrsb_status plane_factor(int dim, const int nb[3], int bd, const double *Acs, C
     return MSRSB_OK;
 }
 
-msrsb_status plane_solve(int dim, const int nb[3], int bd, const double *Acs, const CoarsePlanes *cp,
-                         const double *vc, double *wc, float *wc32, cudaStream_t s) {
+// The couplings H_k that the application needs (not the explicit inverse).
+msrsb_status plane_couplings(int dim, const int nb[3], int bd, const double *Acs, CoarsePlanes *cp, cudaStream_t s) {
     PlaneGeom G;
     plane_geom(dim, nb, bd, &G);
-    const int stage = cp->stage, h = cp->h;
-    const size_t staged = solve_smem_staged(G, cp->nct);
-    auto launch = [&](int phase, int clusters) -> msrsb_status {
+    MSRSB_TRY(dalloc(&cp->H, (size_t)(G.np + 1) * G.m * G.m, s));
+    if (G.np == 1) return MSRSB_OK;
+    const size_t smem = (size_t)kPlaneHRows * G.m * sizeof(double) + (size_t)G.m * sizeof(int);
+    plane_h_kernel<<<dim3(ceil_div(G.m, kPlaneHRows), G.np, 2), 256, smem, s>>>(G, cp->h, Acs, cp->X, cp->pi, cp->H);
+    MSRSB_LAUNCHED("plane_h_kernel");
+    return MSRSB_OK;
+}
+
+msrsb_status plane_solve(const CoarsePlanes *cp, const double *vc, double *wc, float *wc32, cudaStream_t s) {
+    const int m = cp->m, np = cp->np, h = cp->h;
+    auto chain = [&](int forward) -> msrsb_status {
         cudaLaunchAttribute attr[2];
-        cudaLaunchConfig_t cfg = cluster_cfg(attr, cp->nct, stage ? staged : solve_smem(G.m), s, true);
-        cfg.gridDim = dim3(clusters * cp->nct);
+        cudaLaunchConfig_t cfg = cluster_cfg(attr, cp->nct, cp->stage ? solve_smem_staged(m, cp->nct) : solve_smem(m), s,
+                                             true);
+        const int other = forward ? np - 2 - h : np - 1 - h;  // steps of side 1
+        cfg.gridDim = dim3((other > 0 ? 2 : 1) * cp->nct);
+        const double *M = forward ? cp->H : cp->G;
         count_launch();
-        cudaError_t e = cudaLaunchKernelEx(&cfg, plane_solve_kernel, G, h, phase, Acs, (const double *)cp->X,
-                                           (const double *)cp->G, (const int *)cp->pi, vc, wc, wc32, stage);
+        cudaError_t e = cudaLaunchKernelEx(&cfg, plane_chain_kernel, m, np, h, forward, cp->stage, M, wc, wc32);
         if (e == cudaErrorNotSupported || e == cudaErrorInvalidValue) {  // programmatic serialisation refused
             cudaGetLastError();
             cfg.numAttrs = 1;
-            e = cudaLaunchKernelEx(&cfg, plane_solve_kernel, G, h, phase, Acs, (const double *)cp->X,
-                                   (const double *)cp->G, (const int *)cp->pi, vc, wc, wc32, stage);
+            e = cudaLaunchKernelEx(&cfg, plane_chain_kernel, m, np, h, forward, cp->stage, M, wc, wc32);
         }
         MSRSB_CUDA(e);
         return MSRSB_OK;
     };
-    const int sides = G.np - 1 - h > 0 ? 2 : 1;
-    if (h > 0) MSRSB_TRY(launch(0, sides));
-    MSRSB_TRY(launch(1, 1));
-    if (h > 0) MSRSB_TRY(launch(2, sides));
+    const int tiles = ceil_div(m, kPlaneURows);
+    MSRSB_PDL((plane_u_kernel), dim3(tiles, np), kPlaneThreads, (size_t)m * sizeof(double), s, m, (const double *)cp->X,
+              (const int *)cp->pi, vc, wc);
+    if (h > 1) MSRSB_TRY(chain(1));  // side 0 is never the shorter one
+    MSRSB_PDL((plane_middle_kernel), tiles, kPlaneThreads, 0, s, m, np, h, (const double *)cp->H, wc, wc32);
+    if (h > 0) MSRSB_TRY(chain(0));
     return MSRSB_OK;
 }
 
@@ -904,6 +982,7 @@ msrsb_status plane_inverse(int dim, const int nb[3], int bd, const double *Acs, 
 void plane_free(CoarsePlanes *cp, cudaStream_t s) {
     dfree(cp->X, s);
     dfree(cp->G, s);
+    dfree(cp->H, s);
     dfree(cp->pi, s);
 }
 

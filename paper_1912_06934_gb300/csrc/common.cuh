@@ -45,12 +45,16 @@ __device__ __forceinline__ void pdl_prologue() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
-// Asynchronous global -> shared copies (cp.async, 4 or 8 bytes, both
+// Asynchronous global -> shared copies (cp.async, 4, 8 or 16 bytes, both
 // addresses aligned to the size); a thread's copies become visible to it
 // after the group wait, to the other threads after a barrier that follows.
 __device__ __forceinline__ void cp_async8(void *dst, const void *src) {
     const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
     asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async16(void *dst, const void *src) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
 }
 __device__ __forceinline__ void cp_async4(void *dst, const void *src) {
     const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
@@ -200,12 +204,14 @@ struct CoarseInverseWork {
 
 // Block-LU factors of the coarse operator over coarse planes (see
 // coarse_planes.cu): per plane X_k (m x m, row-major) with S_k^-1 = X_k Pi_k,
-// the gather pi_k, and G_k = S_k^-1 U_k.
+// the gather pi_k, G_k = S_k^-1 U_k, and for the application H_k = S_k^-1 L_k
+// (U and L as seen from the side plane k is eliminated on; H[np]: the middle
+// plane towards h + 1).
 struct CoarsePlanes {
     int m = 0, np = 0, nct = 0;
     int h = 0;      // the middle plane: planes below it are eliminated upwards, those above downwards
     int stage = 0;  // the application stages its operands in shared memory
-    double *X = nullptr, *G = nullptr;
+    double *X = nullptr, *G = nullptr, *H = nullptr;
     int *pi = nullptr;
 };
 

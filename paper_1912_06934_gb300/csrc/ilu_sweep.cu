@@ -36,11 +36,6 @@ namespace msrsb {
 template <typename T>
 using LineVec = typename std::conditional<sizeof(T) == 4, float4, double2>::type;
 
-__device__ __forceinline__ void cp_async16(void *dst, const void *src) {
-    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
-}
-
 // groups 0 .. ng-1 of a record (`stride` vectors apart) into registers, zeros after
 template <typename T, int N>
 __device__ __forceinline__ void line_load(T (&v)[N], int ng, const LineVec<T> *p, int stride) {

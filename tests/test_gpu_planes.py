@@ -87,3 +87,16 @@ def test_plane_solver_matches_host_elastic(M, ne, H):
                              krylov=M.msrsb.MSRSB_PCG))
     _check(M, h, 3, 1e-9, 7)
     h.destroy()
+
+
+# more than 1024 coarse unknowns, where the plane factors are kept and applied (not
+# the explicit inverse): planes of 1 and 3 rows, odd rows (no 16-byte copies), rows
+# that do not fit the staged copies, chains of many planes. Tolerance as above.
+@pytest.mark.parametrize("nb", [(1, 1030), (3, 345), (11, 11, 9), (27, 5, 8), (16, 13, 5), (258, 4), (520, 5)], ids=str)
+def test_kept_planes_match_host(M, nb):
+    dims = tuple(2 * b for b in nb)
+    A = _matrix(dims, 7)
+    h = M.msrsb_setup(M.Mat.from_host(A.indptr, A.indices, A.data), M.grid(dims, (2,) * len(nb)),
+                      M.opts(smoother=M.msrsb.MSRSB_SMOOTH_NONE, post=0, tol=0.0, max_iter=5))
+    _check(M, h, 1, 1e-11, 8)
+    h.destroy()
