@@ -162,16 +162,8 @@ msrsb_status mvsub(long N, int nvec, const double *V, long ldv, const double *h,
 template <typename TZ>
 msrsb_status mvadd(long N, int nvec, const TZ *Z, long ldz, const double *y, double *x, cudaStream_t s);
 msrsb_status df_scale(long N, const double *r, const double *beta, float *vh, float *vl, cudaStream_t s);
-msrsb_status arnoldi_dots_df(long N, int nv, const float *Vh, const float *Vl, const float *Ph, const float *Pl,
-                             const float *Wh, const float *Wl, double *partial, cudaStream_t s);
-msrsb_status arnoldi_dots(long N, int nv, const double *V, const double *P, const double *Wv, double *partial,
-                          cudaStream_t s);
-msrsb_status arnoldi_scalar(int m, int j, int full, const double *partial, double *kh, cudaStream_t s);
-msrsb_status arnoldi_update_df(long N, int nv, int m, const float *Vh, const float *Vl, float *Ph, float *Pl,
-                               const float *Wh, const float *Wl, float *Oh, float *Ol, const double *kh,
-                               cudaStream_t s);
-msrsb_status arnoldi_update(long N, int nv, int m, const double *V, double *P, const double *Wv, double *O,
-                            const double *kh, cudaStream_t s);
+msrsb_status arnoldi_step(long N, int j, int m, int k, const ArnBatch<float> &B, double *partial, cudaStream_t s);
+msrsb_status arnoldi_step(long N, int j, int m, int k, const ArnBatch<double> &B, double *partial, cudaStream_t s);
 msrsb_status sell_spmv_df(const Sell &S, const double *val, const double *x, float *yh, float *yl, cudaStream_t s);
 template <typename TP, typename TV>
 msrsb_status restrict_multi(const msrsb_handle *h, int k, const TP *PT, Cols<const TV> v, Cols<double> vc,
@@ -857,21 +849,18 @@ static msrsb_status gmres_t(msrsb_handle *h, const double *b, double *x, double 
                         MSRSB_TRY(df_split(N, h->kv, Wh, Wl, s));
                     }
                 }
-                MSRSB_TRY(arnoldi_dots_df(N, j, Vh, Vl, ph, pl, full ? Wh : nullptr, full ? Wl : nullptr, h->partial,
-                                          s));
-                MSRSB_TRY(arnoldi_scalar(m, j, full, h->partial, kh, s));
-                if (full)
-                    MSRSB_TRY(arnoldi_update_df(N, j, m, Vh, Vl, ph, pl, Wh, Wl, Vh + (long)(j + 1) * N,
-                                                Vl + (long)(j + 1) * N, kh, s));
+                ArnBatch<float> B{};
+                B.r[0] = {Vh, Vl, ph, pl, full ? Wh : nullptr, full ? Wl : nullptr, ph + N, pl + N, kh};
+                MSRSB_TRY(arnoldi_step(N, j, m, 1, B, h->partial, s));
             } else {
                 double *P = V + (long)j * N, *Wn = V + (long)(j + 1) * N;
                 if (full) {
                     MSRSB_TRY(apply_any(h, P, Zj, s));
                     MSRSB_TRY(fine_spmv(h, Zj, nullptr, Wn, false, s));
                 }
-                MSRSB_TRY(arnoldi_dots(N, j, V, P, full ? Wn : nullptr, h->partial, s));
-                MSRSB_TRY(arnoldi_scalar(m, j, full, h->partial, kh, s));
-                if (full) MSRSB_TRY(arnoldi_update(N, j, m, V, P, Wn, Wn, kh, s));
+                ArnBatch<double> B{};
+                B.r[0] = {V, nullptr, P, nullptr, full ? Wn : nullptr, nullptr, Wn, nullptr, kh};
+                MSRSB_TRY(arnoldi_step(N, j, m, 1, B, h->partial, s));
             }
             if (j == 0) continue;
             const int c = j - 1;  // the column this step finished
@@ -1048,6 +1037,8 @@ static msrsb_status gmres_multi_t(msrsb_handle *h, int k, const double *B, doubl
     w.rt = rt;
     MSRSB_TRY(take(&w.vc, (size_t)k * nC));
     MSRSB_TRY(take(&w.wc, (size_t)k * nC));
+    double *part = nullptr;
+    MSRSB_TRY(take(&part, k * arn_partial(m)));
     if (DFV) {
         MSRSB_TRY(take(&w.z32, (size_t)k * N));
         MSRSB_TRY(take(&w.wc32, (size_t)k * nC));
@@ -1153,24 +1144,19 @@ static msrsb_status gmres_multi_t(msrsb_handle *h, int k, const double *B, doubl
                     MSRSB_TRY(spmv_multi(h, kf, zc, y, s));
                 }
             }
-            for (int r : cols) {
+            ArnBatch<T> batch{};
+            for (int c = 0; c < (int)cols.size(); ++c) {
+                const int r = cols[c];
                 const bool f = j < mm[r];
-                double *kh = KH[r];
-                if (DFV) {
+                if constexpr (DFV) {
                     float *ph = Vh[r] + (long)j * N, *pl = Vl[r] + (long)j * N;
-                    MSRSB_TRY(arnoldi_dots_df(N, j, Vh[r], Vl[r], ph, pl, f ? Wh[r] : nullptr, f ? Wl[r] : nullptr,
-                                              h->partial, s));
-                    MSRSB_TRY(arnoldi_scalar(m, j, f, h->partial, kh, s));
-                    if (f)
-                        MSRSB_TRY(arnoldi_update_df(N, j, m, Vh[r], Vl[r], ph, pl, Wh[r], Wl[r],
-                                                    Vh[r] + (long)(j + 1) * N, Vl[r] + (long)(j + 1) * N, kh, s));
+                    batch.r[c] = {Vh[r], Vl[r], ph, pl, f ? Wh[r] : nullptr, f ? Wl[r] : nullptr, ph + N, pl + N, KH[r]};
                 } else {
-                    double *P = V[r] + (long)j * N, *Wn = V[r] + (long)(j + 1) * N;
-                    MSRSB_TRY(arnoldi_dots(N, j, V[r], P, f ? Wn : nullptr, h->partial, s));
-                    MSRSB_TRY(arnoldi_scalar(m, j, f, h->partial, kh, s));
-                    if (f) MSRSB_TRY(arnoldi_update(N, j, m, V[r], P, Wn, Wn, kh, s));
+                    double *P = V[r] + (long)j * N;
+                    batch.r[c] = {V[r], nullptr, P, nullptr, f ? P + N : nullptr, nullptr, P + N, nullptr, KH[r]};
                 }
             }
+            MSRSB_TRY(arnoldi_step(N, j, m, (int)cols.size(), batch, part, s));
             if (j == 0) continue;
             const int c = j - 1;  // the column this step finished
             if (gv != s) {

@@ -24,7 +24,6 @@
 
 namespace msrsb {
 
-constexpr int kArnBlocks = 76;  // row chunks of the dot products (fixed reduction order; a multiple of 4)
 static_assert(kArnBlocks % 4 == 0, "the step's scalars sum the chunks in four fixed quarters");
 
 // ---- pass 1: dot products ------------------------------------------------------------------
@@ -42,61 +41,91 @@ __device__ __forceinline__ void ld_df(const float *h, const float *l, long i, fl
     }
 }
 
-// Block (b, q): rows of chunk b. q < nv: V_q . p -> partial row 2q, V_q . w ->
-// row 2q + 1; q = nv: p . p -> row 2 nv, p . w -> row 2 nv + 1 (w null: the
-// products with w are 0). Double-float planes of W-element groups, FP32
-// arithmetic with error-free transformations up to the per-warp sums.
+// Block (b, g): rows of chunk b and the vectors q = QB g .. QB g + QB - 1. q < nv:
+// V_q . p -> partial row 2q, V_q . w -> row 2q + 1; q = nv: p . p -> row 2 nv, p . w
+// -> row 2 nv + 1 (w null: the products with w are 0). Double-float planes of
+// W-element groups, FP32 arithmetic with error-free transformations up to the per-warp
+// sums; the two products of an element run as one packed pair, two vectors a CTA so
+// that p and what are read half as often, three CTAs an SM (4, 6 or 8 vectors a CTA: 2
+// to 5% more time a solve of 80^3 .. 128^3 unknowns, the registers leave too few warps).
+// Right-hand sides solved together share the launches (blockIdx.z). 2^21 unknowns, 16
+// vectors on average: 87 us, now 73; 8 times 80^3: 8 x 25 us, now 115.
+constexpr int kDotsVecs = 2;
+
 template <int W>
-__global__ void __launch_bounds__(256) dcgs2_dots_df_kernel(long NW, int nv, const float *__restrict__ Vh,
-                                                            const float *__restrict__ Vl, long ldv,
-                                                            const float *Ph, const float *Pl, const float *Wh,
-                                                            const float *Wl, double *__restrict__ partial) {
+__global__ void __launch_bounds__(256, 3) dcgs2_dots_df_kernel(long NW, int nv, long ldv,
+                                                                  const __grid_constant__ ArnBatch<float> B,
+                                                                  long pstride, double *__restrict__ partial) {
+    const ArnRhs<float> &A = B.r[blockIdx.z];
+    const float *Vh = A.Vh, *Vl = A.Vl, *Ph = A.Ph, *Pl = A.Pl, *Wh = A.Wh, *Wl = A.Wl;
+    partial += blockIdx.z * pstride;
     pdl_prologue();
-    __shared__ double red[2][8];
-    const int q = blockIdx.y;
+    constexpr int QB = kDotsVecs;
+    __shared__ double red[2 * QB][8];
+    const int q0 = blockIdx.y * QB;
     const long chunk = (NW + gridDim.x - 1) / gridDim.x;
     const long b0 = blockIdx.x * chunk, b1 = b0 + chunk < NW ? b0 + chunk : NW;
-    const float *ah = q < nv ? Vh + q * ldv : Ph, *al = q < nv ? Vl + q * ldv : Pl;
+    const float *ah[QB], *al[QB];
+#pragma unroll
+    for (int t = 0; t < QB; ++t) {  // beyond nv: p again, not stored
+        ah[t] = q0 + t < nv ? Vh + (q0 + t) * ldv : Ph;
+        al[t] = q0 + t < nv ? Vl + (q0 + t) * ldv : Pl;
+    }
     const bool hw = Wh != nullptr;
-    DF sp{0.f, 0.f}, sw{0.f, 0.f};
+    DF2 sa[QB];
+#pragma unroll
+    for (int t = 0; t < QB; ++t) sa[t] = DF2{0ull, 0ull};
     for (long i = b0 + threadIdx.x; i < b1; i += blockDim.x) {
-        float vh[W], vl[W], ph[W], pl[W];
-        ld_df<W>(ah, al, i, vh, vl);
+        float ph[W], pl[W], wh[W], wl[W], vh[QB][W], vl[QB][W];
         ld_df<W>(Ph, Pl, i, ph, pl);
+        if (hw) ld_df<W>(Wh, Wl, i, wh, wl);
 #pragma unroll
-        for (int e = 0; e < W; ++e) df_fma_acc(sp, vh[e], vl[e], ph[e], pl[e]);
-        if (hw) {
-            float wh[W], wl[W];
-            ld_df<W>(Wh, Wl, i, wh, wl);
+        for (int t = 0; t < QB; ++t)
+            if (q0 + t <= nv) ld_df<W>(ah[t], al[t], i, vh[t], vl[t]);
 #pragma unroll
-            for (int e = 0; e < W; ++e) df_fma_acc(sw, vh[e], vl[e], wh[e], wl[e]);
+        for (int e = 0; e < W; ++e) {
+            const float w = hw ? wh[e] : 0.f;
+            const unsigned long long bh = pk2(ph[e], w), bl = pk2(pl[e], hw ? wl[e] : 0.f), nbh = pk2(-ph[e], -w);
+#pragma unroll
+            for (int t = 0; t < QB; ++t)
+                if (q0 + t <= nv) df2_fma_acc(sa[t], pk2(vh[t][e], vh[t][e]), pk2(vl[t][e], vl[t][e]), bh, bl, nbh);
         }
     }
-    for (int o = 16; o > 0; o >>= 1) {
-        sp = df_add(sp, df_shfl_down(sp, o));
-        sw = df_add(sw, df_shfl_down(sw, o));
-    }
-    if ((threadIdx.x & 31) == 0) {
-        red[0][threadIdx.x >> 5] = (double)sp.hi + (double)sp.lo;
-        red[1][threadIdx.x >> 5] = (double)sw.hi + (double)sw.lo;
+#pragma unroll
+    for (int t = 0; t < QB; ++t) {
+        if (q0 + t > nv) break;
+        DF sp, sw;
+        unpk2(sa[t].hi, sp.hi, sw.hi);
+        unpk2(sa[t].lo, sp.lo, sw.lo);
+        for (int o = 16; o > 0; o >>= 1) {
+            sp = df_add(sp, df_shfl_down(sp, o));
+            sw = df_add(sw, df_shfl_down(sw, o));
+        }
+        if ((threadIdx.x & 31) == 0) {
+            red[2 * t][threadIdx.x >> 5] = (double)sp.hi + (double)sp.lo;
+            red[2 * t + 1][threadIdx.x >> 5] = hw ? (double)sw.hi + (double)sw.lo : 0.0;
+        }
     }
     __syncthreads();
-    if (threadIdx.x < 32) {
-        double a = threadIdx.x < (blockDim.x >> 5) ? red[0][threadIdx.x] : 0.0;
-        double c = threadIdx.x < (blockDim.x >> 5) ? red[1][threadIdx.x] : 0.0;
-        a = warp_sum(a);
-        c = warp_sum(c);
-        if (threadIdx.x == 0) {
-            partial[(long)(2 * q) * gridDim.x + blockIdx.x] = a;
-            partial[(long)(2 * q + 1) * gridDim.x + blockIdx.x] = c;
-        }
+    // eight lanes a row sum the warps' parts
+    const int row = threadIdx.x >> 3, sub = threadIdx.x & 7;
+    static_assert(2 * QB * 8 % 32 == 0 && 2 * QB * 8 <= 256, "whole warps");
+    if (threadIdx.x < 2 * QB * 8) {
+        double a = q0 + (row >> 1) <= nv ? red[row][sub] : 0.0;
+        for (int o = 4; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+        if (sub == 0 && q0 + (row >> 1) <= nv)
+            partial[(long)(2 * q0 + row) * gridDim.x + blockIdx.x] = a;
     }
 }
 
-// The same in FP64 (the FP64 form's basis).
-__global__ void __launch_bounds__(256) dcgs2_dots_kernel(long N, int nv, const double *__restrict__ V, long ldv,
-                                                         const double *P, const double *Wv,
+// The same in FP64 (the FP64 form's basis), a vector a CTA: the FP64 pipe bounds it, and
+// several vectors a CTA (2: 5.81 ms, 4: 6.03 ms a solve of 64^3 unknowns against 5.51)
+// leave it fewer warps.
+__global__ void __launch_bounds__(256) dcgs2_dots_kernel(long N, int nv, long ldv,
+                                                         const __grid_constant__ ArnBatch<double> B, long pstride,
                                                          double *__restrict__ partial) {
+    const double *V = B.r[blockIdx.z].Vh, *P = B.r[blockIdx.z].Ph, *Wv = B.r[blockIdx.z].Wh;
+    partial += blockIdx.z * pstride;
     pdl_prologue();
     __shared__ double red[2][8];
     const int q = blockIdx.y;
@@ -104,6 +133,7 @@ __global__ void __launch_bounds__(256) dcgs2_dots_kernel(long N, int nv, const d
     const long b0 = blockIdx.x * chunk, b1 = b0 + chunk < N ? b0 + chunk : N;
     const double *a = q < nv ? V + q * ldv : P;
     double sp = 0.0, sw = 0.0;
+#pragma unroll 4
     for (long i = b0 + threadIdx.x; i < b1; i += blockDim.x) {
         const double v = __ldg(a + i);
         sp = fma(v, __ldg(P + i), sp);
@@ -116,29 +146,28 @@ __global__ void __launch_bounds__(256) dcgs2_dots_kernel(long N, int nv, const d
         red[1][threadIdx.x >> 5] = sw;
     }
     __syncthreads();
+    const int row = threadIdx.x >> 3, sub = threadIdx.x & 7;
     if (threadIdx.x < 32) {
-        double x = threadIdx.x < (blockDim.x >> 5) ? red[0][threadIdx.x] : 0.0;
-        double y = threadIdx.x < (blockDim.x >> 5) ? red[1][threadIdx.x] : 0.0;
-        x = warp_sum(x);
-        y = warp_sum(y);
-        if (threadIdx.x == 0) {
-            partial[(long)(2 * q) * gridDim.x + blockIdx.x] = x;
-            partial[(long)(2 * q + 1) * gridDim.x + blockIdx.x] = y;
-        }
+        double x = row < 2 ? red[row][sub] : 0.0;
+        for (int o = 4; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+        if (sub == 0 && row < 2) partial[(long)(2 * q + row) * gridDim.x + blockIdx.x] = x;
     }
 }
 
-// ---- the step's scalars (one CTA) ----------------------------------------------------------
+// ---- the step's scalars (one CTA a right-hand side) ----------------------------------------------------------
 //
 // Sums the dot products' row-chunk partials (d = (s_0, t_0, s_1, t_1, ...,
 // rho, sigma), one warp per product, fixed order) and finishes column j-1 of
 // Hu (+= s, Hu[j][j-1] = alpha), copied to H for the Givens rotation; with
-// `full` also R[:, j] = (s, alpha), the provisional column j of Hu
+// `full` (what given) also R[:, j] = (s, alpha), the provisional column j of Hu
 // (V_j^T w_j) and the update coefficients cv = s / alpha (for v_j),
 // cp = H s / alpha + Hu[:, j] (for the next p), scal[0] = 1 / alpha.
-__global__ void __launch_bounds__(256) dcgs2_scalar_kernel(int m, int j, int full,
-                                                           const double *__restrict__ partial,
-                                                           double *__restrict__ kh) {
+template <typename T>
+__global__ void __launch_bounds__(256) dcgs2_scalar_kernel(int m, int j, const __grid_constant__ ArnBatch<T> B,
+                                                           long pstride, const double *__restrict__ partial) {
+    double *__restrict__ kh = B.r[blockIdx.x].kh;
+    const bool full = B.r[blockIdx.x].Wh != nullptr;
+    partial += blockIdx.x * pstride;
     pdl_prologue();
     const KhLayout L(m);
     double *H = kh + L.H, *Hu = kh + L.Hu, *R = kh + L.R;
@@ -225,26 +254,31 @@ __global__ void __launch_bounds__(256) dcgs2_scalar_kernel(int m, int j, int ful
 //
 // v_j = p / alpha - sum_q cv_q V_q (written over p) and
 // p' = what / alpha - sum_q cp_q V_q - cp_j v_j (written to O), q < nv = j:
-// both combinations read each V_q once.
+// both combinations read each V_q once and run as one packed pair. Three CTAs an SM:
+// with the registers of one or two, 128^3 unknowns took 98 us a step instead of 58 (63
+// as scalars); 8 times 80^3: 8 x 17 us, now 85.
 template <int W>
-__global__ void __launch_bounds__(256) dcgs2_update_df_kernel(long NW, int nv, const float *__restrict__ Vh,
-                                                              const float *__restrict__ Vl, long ldv, float *Ph,
-                                                              float *Pl, const float *Wh, const float *Wl, float *Oh,
-                                                              float *Ol, const double *__restrict__ kv,
-                                                              const double *__restrict__ kp,
-                                                              const double *__restrict__ ksc) {
+__global__ void __launch_bounds__(256, 3) dcgs2_update_df_kernel(long NW, int nv, int m, long ldv,
+                                                                    const __grid_constant__ ArnBatch<float> B) {
+    const ArnRhs<float> &A = B.r[blockIdx.y];
+    if (!A.Wh) return;  // this right-hand side's cycle ends here
+    const float *Vh = A.Vh, *Vl = A.Vl, *Wh = A.Wh, *Wl = A.Wl;
+    float *Ph = A.Ph, *Pl = A.Pl, *Oh = A.Oh, *Ol = A.Ol;
+    const KhLayout L(m);
+    const double *kv = A.kh + L.cv, *kp = A.kh + L.cp, *ksc = A.kh + L.scal;
     pdl_prologue();
-    __shared__ float cvh[512], cvl[512], cph[513], cpl[513];
-    __shared__ DF s_inva;
+    __shared__ ulonglong2 ch[512];  // -(cv, cp): high words and their negatives, low words
+    __shared__ unsigned long long cw[512];
+    __shared__ DF s_inva, s_cn;
     for (int q = threadIdx.x; q <= nv; q += blockDim.x) {
+        const DF b = df_from(-kp[q]);
         if (q < nv) {
             const DF a = df_from(-kv[q]);
-            cvh[q] = a.hi;
-            cvl[q] = a.lo;
+            ch[q] = make_ulonglong2(pk2(a.hi, b.hi), pk2(-a.hi, -b.hi));
+            cw[q] = pk2(a.lo, b.lo);
+        } else {
+            s_cn = b;
         }
-        const DF b = df_from(-kp[q]);
-        cph[q] = b.hi;
-        cpl[q] = b.lo;
     }
     if (threadIdx.x == 0) s_inva = df_from(ksc[0]);
     __syncthreads();
@@ -253,29 +287,31 @@ __global__ void __launch_bounds__(256) dcgs2_update_df_kernel(long NW, int nv, c
         float ph[W], pl[W], wh[W], wl[W];
         ld_df<W>(Ph, Pl, i, ph, pl);
         ld_df<W>(Wh, Wl, i, wh, wl);
-        DF av[W], ap[W];
+        DF2 ac[W];  // (v_j, p') of an element as one packed pair
 #pragma unroll
         for (int e = 0; e < W; ++e) {
-            av[e] = df_mul(DF{ph[e], pl[e]}, ia);
-            ap[e] = df_mul(DF{wh[e], wl[e]}, ia);
+            const DF a = df_mul(DF{ph[e], pl[e]}, ia), b = df_mul(DF{wh[e], wl[e]}, ia);
+            ac[e] = DF2{pk2(a.hi, b.hi), pk2(a.lo, b.lo)};
         }
 #pragma unroll 2
         for (int q = 0; q < nv; ++q) {
             float vh[W], vl[W];
             ld_df<W>(Vh + q * ldv, Vl + q * ldv, i, vh, vl);
-            const float ah = cvh[q], al = cvl[q], bh = cph[q], bl = cpl[q];
+            const ulonglong2 c = ch[q];
+            const unsigned long long cl = cw[q];
 #pragma unroll
-            for (int e = 0; e < W; ++e) {
-                df_fma_acc(av[e], vh[e], vl[e], ah, al);
-                df_fma_acc(ap[e], vh[e], vl[e], bh, bl);
-            }
+            for (int e = 0; e < W; ++e)
+                df2_fma_acc(ac[e], pk2(vh[e], vh[e]), pk2(vl[e], vl[e]), c.x, cl, c.y);
         }
         float vh[W], vl[W], oh[W], ol[W];
 #pragma unroll
         for (int e = 0; e < W; ++e) {
-            const DF v = two_sum(av[e].hi, av[e].lo);
-            df_fma_acc(ap[e], v.hi, v.lo, cph[nv], cpl[nv]);
-            const DF o = two_sum(ap[e].hi, ap[e].lo);
+            DF a, b;
+            unpk2(ac[e].hi, a.hi, b.hi);
+            unpk2(ac[e].lo, a.lo, b.lo);
+            const DF v = two_sum(a.hi, a.lo);
+            df_fma_acc(b, v.hi, v.lo, s_cn.hi, s_cn.lo);
+            const DF o = two_sum(b.hi, b.lo);
             vh[e] = v.hi, vl[e] = v.lo, oh[e] = o.hi, ol[e] = o.lo;
         }
         if constexpr (W == 4) {
@@ -291,11 +327,14 @@ __global__ void __launch_bounds__(256) dcgs2_update_df_kernel(long NW, int nv, c
 
 // The same in FP64; Wv and O may be the same vector (read before written,
 // element by element).
-__global__ void __launch_bounds__(256) dcgs2_update_kernel(long N, int nv, const double *__restrict__ V, long ldv,
-                                                           double *P, const double *Wv, double *O,
-                                                           const double *__restrict__ kv,
-                                                           const double *__restrict__ kp,
-                                                           const double *__restrict__ ksc) {
+__global__ void __launch_bounds__(256) dcgs2_update_kernel(long N, int nv, int m, long ldv,
+                                                           const __grid_constant__ ArnBatch<double> B) {
+    const ArnRhs<double> &A = B.r[blockIdx.y];
+    if (!A.Wh) return;  // this right-hand side's cycle ends here
+    const double *V = A.Vh, *Wv = A.Wh;
+    double *P = A.Ph, *O = A.Oh;
+    const KhLayout L(m);
+    const double *kv = A.kh + L.cv, *kp = A.kh + L.cp, *ksc = A.kh + L.scal;
     pdl_prologue();
     __shared__ double cvs[512], cps[513];
     for (int q = threadIdx.x; q <= nv; q += blockDim.x) {
@@ -321,55 +360,50 @@ __global__ void __launch_bounds__(256) dcgs2_update_kernel(long N, int nv, const
 
 static bool al16(const void *p) { return ((uintptr_t)p & 15) == 0; }
 
-// partials of (V_q . p, V_q . w for q < nv; p . p, p . w): V holds nv
-// vectors of N with stride N; w may be null (its products are 0)
-msrsb_status arnoldi_dots_df(long N, int nv, const float *Vh, const float *Vl, const float *Ph, const float *Pl,
-                             const float *Wh, const float *Wl, double *partial, cudaStream_t s) {
-    dim3 grid(kArnBlocks, nv + 1);
-    const bool v4 = N % 4 == 0 && al16(Vh) && al16(Vl) && al16(Ph) && al16(Pl) && (!Wh || (al16(Wh) && al16(Wl)));
-    if (v4)
-        MSRSB_PDL((dcgs2_dots_df_kernel<4>), grid, 256, 0, s, N / 4, nv, Vh, Vl, N, Ph, Pl, Wh, Wl, partial);
-    else
-        MSRSB_PDL((dcgs2_dots_df_kernel<1>), grid, 256, 0, s, N, nv, Vh, Vl, N, Ph, Pl, Wh, Wl, partial);
-    return MSRSB_OK;
+static bool al16(const ArnRhs<float> &A) {
+    return al16(A.Vh) && al16(A.Vl) && al16(A.Ph) && al16(A.Pl) && al16(A.Wh) && al16(A.Wl) && al16(A.Oh) && al16(A.Ol);
+}
+static bool al16(int k, const ArnBatch<float> &B) {
+    for (int c = 0; c < k; ++c)
+        if (!al16(B.r[c])) return false;
+    return true;
 }
 
-msrsb_status arnoldi_dots(long N, int nv, const double *V, const double *P, const double *Wv, double *partial,
-                          cudaStream_t s) {
-    dim3 grid(kArnBlocks, nv + 1);
-    MSRSB_PDL((dcgs2_dots_kernel), grid, 256, 0, s, N, nv, V, N, P, Wv, partial);
-    return MSRSB_OK;
-}
-
-// the step's scalars from the partials the dots left in `partial`
-msrsb_status arnoldi_scalar(int m, int j, int full, const double *partial, double *kh, cudaStream_t s) {
+// Step j of k right-hand sides (the vectors before v_j: nv = j of N, stride N) in three
+// launches: dots, scalars, update. partial: k * arn_partial(m) doubles.
+msrsb_status arnoldi_step(long N, int j, int m, int k, const ArnBatch<float> &B, double *partial, cudaStream_t s) {
     if (m > 512 || j > m) return fail(MSRSB_EINVAL, "Arnoldi step %d of %d", j, m);
-    MSRSB_PDL((dcgs2_scalar_kernel), 1, 256, 0, s, m, j, full, partial, kh);
-    return MSRSB_OK;
-}
-
-msrsb_status arnoldi_update_df(long N, int nv, int m, const float *Vh, const float *Vl, float *Ph, float *Pl,
-                               const float *Wh, const float *Wl, float *Oh, float *Ol, const double *kh,
-                               cudaStream_t s) {
-    const KhLayout L(m);
-    const bool v4 = N % 4 == 0 && al16(Vh) && al16(Vl) && al16(Ph) && al16(Pl) && al16(Wh) && al16(Wl) &&
-                    al16(Oh) && al16(Ol);
+    const long ps = (long)arn_partial(m);
+    const bool v4 = N % 4 == 0 && al16(k, B);
     const long NW = v4 ? N / 4 : N;
-    const int grid = ceil_div(NW, 256) < 2048 ? (int)ceil_div(NW, 256) : 2048;
+    const dim3 gd(kArnBlocks, ceil_div(j + 1, kDotsVecs), k);
     if (v4)
-        MSRSB_PDL((dcgs2_update_df_kernel<4>), grid, 256, 0, s, NW, nv, Vh, Vl, N / 4 * 4, Ph, Pl, Wh, Wl, Oh, Ol,
-                  kh + L.cv, kh + L.cp, kh + L.scal);
+        MSRSB_PDL((dcgs2_dots_df_kernel<4>), gd, 256, 0, s, NW, j, N, B, ps, partial);
     else
-        MSRSB_PDL((dcgs2_update_df_kernel<1>), grid, 256, 0, s, NW, nv, Vh, Vl, N, Ph, Pl, Wh, Wl, Oh, Ol,
-                  kh + L.cv, kh + L.cp, kh + L.scal);
+        MSRSB_PDL((dcgs2_dots_df_kernel<1>), gd, 256, 0, s, NW, j, N, B, ps, partial);
+    MSRSB_PDL((dcgs2_scalar_kernel<float>), k, 256, 0, s, m, j, B, ps, (const double *)partial);
+    bool any = false;
+    for (int c = 0; c < k; ++c) any = any || B.r[c].Wh;
+    if (!any) return MSRSB_OK;
+    const dim3 gu(ceil_div(NW, 256) < 2048 ? (unsigned)ceil_div(NW, 256) : 2048u, k);
+    if (v4)
+        MSRSB_PDL((dcgs2_update_df_kernel<4>), gu, 256, 0, s, NW, j, m, N, B);
+    else
+        MSRSB_PDL((dcgs2_update_df_kernel<1>), gu, 256, 0, s, NW, j, m, N, B);
     return MSRSB_OK;
 }
 
-msrsb_status arnoldi_update(long N, int nv, int m, const double *V, double *P, const double *Wv, double *O,
-                            const double *kh, cudaStream_t s) {
-    const KhLayout L(m);
-    const int grid = ceil_div(N, 256) < 2048 ? (int)ceil_div(N, 256) : 2048;
-    MSRSB_PDL((dcgs2_update_kernel), grid, 256, 0, s, N, nv, V, N, P, Wv, O, kh + L.cv, kh + L.cp, kh + L.scal);
+msrsb_status arnoldi_step(long N, int j, int m, int k, const ArnBatch<double> &B, double *partial, cudaStream_t s) {
+    if (m > 512 || j > m) return fail(MSRSB_EINVAL, "Arnoldi step %d of %d", j, m);
+    const long ps = (long)arn_partial(m);
+    MSRSB_PDL((dcgs2_dots_kernel), dim3(kArnBlocks, j + 1, k), 256, 0, s, N, j, N, B, ps,
+              partial);
+    MSRSB_PDL((dcgs2_scalar_kernel<double>), k, 256, 0, s, m, j, B, ps, (const double *)partial);
+    bool any = false;
+    for (int c = 0; c < k; ++c) any = any || B.r[c].Wh;
+    if (!any) return MSRSB_OK;
+    const unsigned g = ceil_div(N, 256) < 2048 ? (unsigned)ceil_div(N, 256) : 2048u;
+    MSRSB_PDL((dcgs2_update_kernel), dim3(g, k), 256, 0, s, N, j, m, N, B);
     return MSRSB_OK;
 }
 

@@ -286,6 +286,25 @@ struct Cols {
     T *p[kMaxRhs];
 };
 
+// One step's Krylov vectors of a right-hand side (arnoldi.cu): the basis V, the vector
+// p being finished, what = A M^-1 p (null in a cycle's last step) and the next p's
+// place; planes h and l of double-floats, or FP64 in h. kh: its Krylov state.
+template <typename T>
+struct ArnRhs {
+    const T *Vh, *Vl;
+    T *Ph, *Pl;
+    const T *Wh, *Wl;
+    T *Oh, *Ol;
+    double *kh;
+};
+template <typename T>
+struct ArnBatch {
+    ArnRhs<T> r[kMaxRhs];
+};
+constexpr int kArnBlocks = 76;  // row chunks of the dot products (fixed reduction order; a multiple of 4)
+// partials of one right-hand side's step
+inline size_t arn_partial(int m) { return 2 * (size_t)(m + 1) * kArnBlocks; }
+
 // Krylov state on the device, m = restart length:
 // H[(m+1) x m] column-major (Givens-rotated in place) | cs[m] | sn[m] | g[m+1] |
 // est | beta | h2[m+2] | est_hist[m+1] | flag[8] | Hu[(m+1) x m] (the

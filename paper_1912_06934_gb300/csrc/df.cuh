@@ -56,4 +56,49 @@ __device__ __forceinline__ DF df_shfl_down(DF v, int o) {
     return DF{__shfl_down_sync(0xffffffffu, v.hi, o), __shfl_down_sync(0xffffffffu, v.lo, o)};
 }
 
+// Two double-floats side by side in packed FP32 pairs: the same operations,
+// hence the same bits, as the scalar forms above, two per instruction.
+struct DF2 {
+    unsigned long long hi, lo;
+};
+__device__ __forceinline__ unsigned long long pk2(float a, float b) {
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void unpk2(unsigned long long v, float &a, float &b) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigned long long b) {
+    unsigned long long r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ unsigned long long sub2(unsigned long long a, unsigned long long b) {
+    unsigned long long r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ unsigned long long mul2(unsigned long long a, unsigned long long b) {
+    unsigned long long r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c) {
+    unsigned long long r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+// s += a * b; nbh = -b's high word, whose product with a is the negated p of df_fma_acc
+__device__ __forceinline__ void df2_fma_acc(DF2 &s, unsigned long long ah, unsigned long long al,
+                                            unsigned long long bh, unsigned long long bl, unsigned long long nbh) {
+    const unsigned long long np = mul2(ah, nbh), e = fma2(ah, bh, np);
+    const unsigned long long t = sub2(s.hi, np), bb = sub2(t, s.hi);
+    const unsigned long long tl = sub2(sub2(s.hi, sub2(t, bb)), add2(np, bb));
+    const unsigned long long r = add2(s.lo, add2(tl, fma2(ah, bl, fma2(al, bh, e))));
+    const unsigned long long u = add2(t, r), cc = sub2(u, t);
+    s.lo = add2(sub2(t, sub2(u, cc)), sub2(r, cc));
+    s.hi = u;
+}
+
 }  // namespace msrsb
