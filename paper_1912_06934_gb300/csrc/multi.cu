@@ -47,30 +47,51 @@ __global__ void __launch_bounds__(256) restrict_multi_kernel(int nc, int k, cons
     }
 }
 
-// ---- coarse product w_c = A_c^-1 v_c (dense inverse), one warp per row -------------------
-__global__ void __launch_bounds__(256) gemm_multi_kernel(int n, int k, const double *__restrict__ M,
-                                                         Cols<const double> x, Cols<double> y, Cols<float> y32) {
-    const int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    const int lane = threadIdx.x & 31;
-    pdl_prologue();
-    if (row >= n) return;
+// ---- coarse product w_c = A_c^-1 v_c (dense inverse) --------------------------------------
+//
+// A CTA takes a row, a warp of it kGemmRhs right-hand sides, in the one-vector kernel's
+// order. Bound by the FP64 pipe (one warp's FMA in 19 cycles of an SM), so the work is
+// dealt out evenly: n CTAs of at most two warps (8 rows a CTA leave 27 SMs without one
+// at n = 1000). The row's entries are loaded before the wait. n = 1000, 8 right-hand
+// sides: 94 us with a warp a row and all right-hand sides, now 30.
+constexpr int kGemmRhs = 4;
+constexpr int kGemmPre = 16;
+
+__global__ void __launch_bounds__(32 * kMaxRhs / kGemmRhs) gemm_multi_kernel(int n, int k, const double *__restrict__ M,
+                                                                            Cols<const double> x, Cols<double> y,
+                                                                            Cols<float> y32) {
+    const int row = blockIdx.x, lane = threadIdx.x & 31, c0 = (threadIdx.x >> 5) * kGemmRhs;
     const double *mr = M + (long)row * n;
-    double s[kMaxRhs];
+    double m[kGemmPre];
 #pragma unroll
-    for (int c = 0; c < kMaxRhs; ++c) s[c] = 0.0;
-    for (int j = lane; j < n; j += 32) {  // the one-vector kernel's order
-        const double m = __ldg(mr + j);
+    for (int t = 0; t < kGemmPre; ++t) m[t] = __ldg(mr + min(lane + 32 * t, n - 1));
+    pdl_prologue();
+    const double *xp[kGemmRhs];
+    double s[kGemmRhs];
 #pragma unroll
-        for (int c = 0; c < kMaxRhs; ++c)
-            if (c < k) s[c] = fma(m, x.p[c][j], s[c]);
+    for (int c = 0; c < kGemmRhs; ++c) {
+        xp[c] = x.p[c0 + c < k ? c0 + c : c0];
+        s[c] = 0.0;
     }
 #pragma unroll
-    for (int c = 0; c < kMaxRhs; ++c) {
-        if (c >= k) break;
+    for (int t = 0; t < kGemmPre; ++t)
+        if (lane + 32 * t < n) {
+#pragma unroll
+            for (int c = 0; c < kGemmRhs; ++c) s[c] = fma(m[t], xp[c][lane + 32 * t], s[c]);
+        }
+#pragma unroll 4
+    for (int j = lane + 32 * kGemmPre; j < n; j += 32) {
+        const double a = __ldg(mr + j);
+#pragma unroll
+        for (int c = 0; c < kGemmRhs; ++c) s[c] = fma(a, xp[c][j], s[c]);
+    }
+#pragma unroll
+    for (int c = 0; c < kGemmRhs; ++c) {
+        if (c0 + c >= k) break;
         const double t = warp_sum(s[c]);
         if (lane == 0) {
-            y.p[c][row] = t;
-            if (y32.p[c]) y32.p[c][row] = (float)t;
+            y.p[c0 + c][row] = t;
+            if (y32.p[c0 + c]) y32.p[c0 + c][row] = (float)t;
         }
     }
 }
@@ -226,7 +247,7 @@ template msrsb_status restrict_multi<double, double>(const msrsb_handle *, int, 
 
 msrsb_status gemm_multi(int n, int k, const double *M, Cols<const double> x, Cols<double> y, Cols<float> y32,
                         cudaStream_t s) {
-    MSRSB_PDL((gemm_multi_kernel), ceil_div(n, 8), 256, 0, s, n, k, M, x, y, y32);
+    MSRSB_PDL((gemm_multi_kernel), n, 32 * ceil_div(k, kGemmRhs), 0, s, n, k, M, x, y, y32);
     return MSRSB_OK;
 }
 
