@@ -158,7 +158,6 @@ template <typename TP, typename TZ>
 msrsb_status prolong_op(const msrsb_handle *h, const TP *P, const double *wc, const float *wc32, TZ *z, float *z32,
                         TP *x4, int add, cudaStream_t s);
 msrsb_status norm2(long N, const double *w, double *partial, double *out, cudaStream_t s);
-msrsb_status mvsub(long N, int nvec, const double *V, long ldv, const double *h, double *w, cudaStream_t s);
 template <typename TZ>
 msrsb_status mvadd(long N, int nvec, const TZ *Z, long ldz, const double *y, double *x, cudaStream_t s);
 msrsb_status df_scale(long N, const double *r, const double *beta, float *vh, float *vl, cudaStream_t s);
@@ -717,29 +716,96 @@ __global__ void givens_kernel(int m, int j, double *__restrict__ kh) {
 // back substitution H(0:k,0:k) y = g(0:k), then R(0:k,0:k) u = y (R upper
 // triangular, column-major with leading dimension m: the basis the solution
 // update uses is Zhat = Z R); u written over g. Column oriented: once an
-// unknown is known, thread i < c removes its column's entry from row i.
-__global__ void hess_solve_kernel(int m, int k, double *__restrict__ kh) {
+// unknown is known, thread i < c removes its column's entry from row i. A block a
+// right-hand side. The 2k columns are a chain: what a column costs is an unknown
+// (a multiplication by its reciprocal diagonal, formed for all unknowns beforehand, and
+// the correction by the remainder that rounds the quotient), one barrier and a row's
+// update; the columns are loaded four ahead. (With a division and the column's load on
+// the chain 70 us for k = 32, 34 now with the launch.)
+constexpr int kHessThreads = 256;
+constexpr int kHessRows = 4;   // rows a thread: k <= 1024
+constexpr int kHessAhead = 4;  // columns loaded ahead
+
+struct HessBatch {
+    double *kh[kMaxRhs];
+    int k[kMaxRhs];
+};
+
+__global__ void __launch_bounds__(kHessThreads) hess_solve_kernel(int m, const __grid_constant__ HessBatch B) {
     pdl_prologue();
     const KhLayout L(m);
-    double *g = kh + L.g;
-    __shared__ double gs[1024];
-    __shared__ double yc;
-    for (int i = threadIdx.x; i < k; i += blockDim.x) gs[i] = g[i];
-    __syncthreads();
+    double *kh = B.kh[blockIdx.x], *g = kh + L.g;
+    const int k = B.k[blockIdx.x], tid = threadIdx.x, nt = blockDim.x;
+    __shared__ double s_d[2][kHessThreads * kHessRows], s_r[2][kHessThreads * kHessRows], s_y[2];
+    double gi[kHessRows];
+#pragma unroll
+    for (int u = 0; u < kHessRows; ++u) {
+        const int i = tid + u * nt;
+        gi[u] = i < k ? g[i] : 0.0;
+        if (i < k) {
+            const double d0 = kh[L.H + (long)i * (m + 1) + i], d1 = kh[L.R + (long)i * m + i];
+            s_d[0][i] = d0;
+            s_d[1][i] = d1;
+            s_r[0][i] = 1.0 / d0;
+            s_r[1][i] = 1.0 / d1;
+        }
+    }
     for (int pass = 0; pass < 2; ++pass) {
         const double *T = pass == 0 ? kh + L.H : kh + L.R;
         const long ld = pass == 0 ? m + 1 : m;
-        for (int c = k - 1; c >= 0; --c) {
-            const double *tc = T + (long)c * ld;
-            if (threadIdx.x == 0) yc = gs[c] / tc[c];
-            __syncthreads();
-            const double y = yc;
-            for (int i = threadIdx.x; i < c; i += blockDim.x) gs[i] -= tc[i] * y;
-            if (threadIdx.x == 0) gs[c] = y;
-            __syncthreads();
+        double cur[kHessAhead][kHessRows], nxt[kHessAhead][kHessRows];
+        auto load = [&](int c0, double (&t)[kHessAhead][kHessRows]) {  // columns c0, c0 - 1, ...
+#pragma unroll
+            for (int a = 0; a < kHessAhead; ++a)
+#pragma unroll
+                for (int u = 0; u < kHessRows; ++u) {
+                    const int i = tid + u * nt;
+                    t[a][u] = c0 - a >= 0 && i < c0 - a ? T[(long)(c0 - a) * ld + i] : 0.0;
+                }
+        };
+        load(k - 1, cur);
+        for (int c0 = k - 1; c0 >= 0; c0 -= kHessAhead) {
+            load(c0 - kHessAhead, nxt);
+#pragma unroll
+            for (int a = 0; a < kHessAhead; ++a) {
+                const int c = c0 - a;
+                if (c < 0) break;
+                if (a == 0) __syncthreads();  // (first pass: s_d, s_r; then the last s_y of the block before)
+#pragma unroll
+                for (int u = 0; u < kHessRows; ++u)
+                    if (tid + u * nt == c) {
+                        const double d = s_d[pass][c], r = s_r[pass][c], q = gi[u] * r;
+                        const double y =
+                            fabs(d) <= 1e140 && fabs(r) <= 1e140 && fabs(q) <= 1e140 ? fma(fma(-q, d, gi[u]), r, q) : gi[u] / d;
+                        s_y[c & 1] = y;
+                        gi[u] = y;
+                    }
+                __syncthreads();
+                const double y = s_y[c & 1];
+#pragma unroll
+                for (int u = 0; u < kHessRows; ++u)
+                    if (tid + u * nt < c) gi[u] -= cur[a][u] * y;
+            }
+#pragma unroll
+            for (int a = 0; a < kHessAhead; ++a)
+#pragma unroll
+                for (int u = 0; u < kHessRows; ++u) cur[a][u] = nxt[a][u];
         }
     }
-    for (int i = threadIdx.x; i < k; i += blockDim.x) g[i] = gs[i];
+#pragma unroll
+    for (int u = 0; u < kHessRows; ++u)
+        if (tid + u * nt < k) g[tid + u * nt] = gi[u];
+}
+
+// the update coefficients of nr right-hand sides, k[c] columns each
+static msrsb_status hess_solve(int m, int nr, const HessBatch &B, cudaStream_t s) {
+    int kmax = 1;
+    for (int c = 0; c < nr; ++c) kmax = B.k[c] > kmax ? B.k[c] : kmax;
+    if (kmax > kHessThreads * kHessRows) return fail(MSRSB_EINVAL, "Hessenberg system of %d columns", kmax);
+    const int nt = kmax >= kHessThreads ? kHessThreads : (kmax + 31) & ~31;
+    hess_solve_kernel<<<nr, nt, 0, s>>>(m, B);  // follows the wait on the Givens stream: no PDL
+    MSRSB_LAUNCHED("hess_solve_kernel");
+    return MSRSB_OK;
 }
 
 __global__ void gmres_init_kernel(int m, double *__restrict__ kh, const double *__restrict__ beta) {
@@ -904,8 +970,10 @@ static msrsb_status gmres_t(msrsb_handle *h, const double *b, double *x, double 
         }
         const int k = conv >= 0 ? conv + 1 : launched;
         its += k;
-        hess_solve_kernel<<<1, 256, 0, s>>>(m, k, kh);  // follows the wait on the Givens stream: no PDL
-        MSRSB_LAUNCHED("hess_solve_kernel");
+        HessBatch hb{};
+        hb.kh[0] = kh;
+        hb.k[0] = k;
+        MSRSB_TRY(hess_solve(m, 1, hb, s));
         MSRSB_TRY(mvadd<double>(N, k, Z, N, kh + L.g, x, s));
     }
     *iters = its;
@@ -1197,13 +1265,16 @@ static msrsb_status gmres_multi_t(msrsb_handle *h, int k, const double *B, doubl
                     if (e <= stop[r]) conv[r] = q;
                 }
         }
-        for (int r : act) {
-            const int kk = conv[r] >= 0 ? conv[r] + 1 : launched[r];
-            its[r] += kk;
-            hess_solve_kernel<<<1, 256, 0, s>>>(m, kk, KH[r]);
-            MSRSB_LAUNCHED("hess_solve_kernel");
-            MSRSB_TRY(mvadd<double>(N, kk, Z[r], N, KH[r] + L.g, X + r * N, s));
+        HessBatch hb{};
+        for (int c = 0; c < (int)act.size(); ++c) {
+            const int r = act[c];
+            hb.kh[c] = KH[r];
+            hb.k[c] = conv[r] >= 0 ? conv[r] + 1 : launched[r];
+            its[r] += hb.k[c];
         }
+        MSRSB_TRY(hess_solve(m, (int)act.size(), hb, s));
+        for (int c = 0; c < (int)act.size(); ++c)
+            MSRSB_TRY(mvadd<double>(N, hb.k[c], Z[act[c]], N, hb.kh[c] + L.g, X + act[c] * N, s));
     }
     for (int r = 0; r < k; ++r) iters[r] = its[r];
     return MSRSB_OK;
