@@ -126,7 +126,7 @@ template <typename T, typename TZ>
 msrsb_status ilu0_apply(const msrsb_handle *h, T *ry, TZ *z, cudaStream_t s);
 bool lines_fit(const msrsb_grid *g);
 template <typename TF>
-msrsb_status lines_setup(msrsb_handle *h, TF *lu, cudaStream_t s);
+msrsb_status lines_setup(msrsb_handle *h, cudaStream_t s);
 msrsb_status stencil_check(const msrsb_mat *A, const msrsb_grid *g, cudaStream_t s);
 template <typename T, typename TZ>
 msrsb_status lines_apply(const msrsb_handle *h, T *ry, TZ *z, cudaStream_t s);
@@ -205,7 +205,11 @@ static msrsb_status setup_smoother(msrsb_handle *h, cudaStream_t s) {
     const int n = h->n, bd = h->bdim;
     h->ncolours = 1 << h->grid.dim;
     h->colour_ptr_h = (int32_t *)calloc(h->ncolours + 1, sizeof(int32_t));
-    MSRSB_TRY(colour_classes(n, h->colour, h->ncolours, &h->colour_rows, h->colour_ptr_h, s));
+    const bool ilu = h->opts.smoother == MSRSB_SMOOTH_ILU0 || (h->opts.smoother == MSRSB_SMOOTH_IC0 && bd == 1);
+    const bool lines = ilu && bd == 1 && h->opts.ordering == MSRSB_ORDER_LINES && lines_fit(&h->grid);
+    // the smoothers ordered by point colours
+    if (!lines && (ilu || h->opts.smoother == MSRSB_SMOOTH_GS || h->opts.smoother == MSRSB_SMOOTH_IC0))
+        MSRSB_TRY(colour_classes(n, h->colour, h->ncolours, &h->colour_rows, h->colour_ptr_h, s));
     if (bd == 1) MSRSB_TRY(sell_copy(&A, h->opts.prec == MSRSB_F32, &h->asell, s));
     // the block Gauss-Seidel sweeps have the blocks in their own layout
     if (h->opts.prec == MSRSB_F32 && bd != 1 && h->opts.smoother != MSRSB_SMOOTH_GS) {
@@ -214,7 +218,6 @@ static msrsb_status setup_smoother(msrsb_handle *h, cudaStream_t s) {
         MSRSB_TRY(convert<float>((long)A.nnz * bd * bd, A.val, alo, s));
         h->a_lo = alo;
     }
-    const bool ilu = h->opts.smoother == MSRSB_SMOOTH_ILU0 || (h->opts.smoother == MSRSB_SMOOTH_IC0 && bd == 1);
     // the ordered smoothers sweep a colour (or line block) per launch
     if (ilu || h->opts.smoother == MSRSB_SMOOTH_IC0 || h->opts.smoother == MSRSB_SMOOTH_GS)
         MSRSB_TRY(stencil_check(&A, &h->grid, s));
@@ -230,19 +233,19 @@ static msrsb_status setup_smoother(msrsb_handle *h, cudaStream_t s) {
     } else if (ilu) {
         if (bd != 1) return fail(MSRSB_EINVAL, "ILU(0) smoother needs a scalar operator; use MSRSB_SMOOTH_GS or IC0");
         // factorised in the smoother's precision (FP32 in the mixed form)
-        T *lu = nullptr;
-        MSRSB_TRY(dalloc(&lu, A.nnz, s));
-        MSRSB_TRY(convert<T>(A.nnz, A.val, lu, s));
-        if (h->opts.ordering == MSRSB_ORDER_LINES && lines_fit(&h->grid)) {
+        if (lines) {
             h->use_lines = 1;
-            MSRSB_TRY(lines_setup<T>(h, lu, s));
+            MSRSB_TRY(lines_setup<T>(h, s));
         } else {
+            T *lu = nullptr;
+            MSRSB_TRY(dalloc(&lu, A.nnz, s));
+            MSRSB_TRY(convert<T>(A.nnz, A.val, lu, s));
             MSRSB_TRY(dalloc(&h->diag_pos, n, s));
             MSRSB_TRY(
                 ilu0_factor<T>(&A, h->colour, h->ncolours, h->colour_rows, h->colour_ptr_h, h->diag_pos, lu, s));
             MSRSB_TRY(ilu_build_ell<T>(h, lu, s));
+            dfree(lu, s);
         }
-        dfree(lu, s);
     } else if (h->opts.smoother == MSRSB_SMOOTH_GS) {
         if (bd != 3) return fail(MSRSB_EINVAL, "block Gauss-Seidel smoother needs a 3x3 block operator");
         T *dinv = nullptr;

@@ -24,263 +24,259 @@
 #include <cstring>
 #include <type_traits>
 #include <vector>
-#include <cub/device/device_radix_sort.cuh>
 
 namespace msrsb {
 
 
-void diag_pos_launch(int n, const int32_t *rowptr, const int32_t *colidx, int32_t *dpos, int *status, cudaStream_t s);
+// ---- the order ------------------------------------------------------------------------
+//
+// Colour c's lines start at line cl[c] (a line has nx positions); its blocks follow
+// row of blocks by row of blocks, and only the last block along y or z is thinner than
+// two lines, so a line's place in the order is arithmetic.
+struct LineGrid {
+    int dim, nx, ny, nz;
+    int cl[5];  // first line of each colour (+ end)
+    int Ly[2];  // lines along y in blocks of even and of odd index
+};
 
-// sort key of every row: colour, block, line inside the block, x
-__global__ void line_key_kernel(int n, int dim, int nx, int ny, int nz, uint32_t *__restrict__ key,
-                                int32_t *__restrict__ idx) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const int x = i % nx, y = (i / nx) % ny, z = dim == 3 ? i / (nx * ny) : 0;
-    const int by = y >> 1, bz = z >> 1, nby = (ny + 1) >> 1, nbz = dim == 3 ? (nz + 1) >> 1 : 1;
-    const int c = (by & 1) | (dim == 3 ? ((bz & 1) << 1) : 0);
-    const int sub = (y & 1) | (dim == 3 ? ((z & 1) << 1) : 0);
-    const long blk = (long)by + (long)nby * bz;
-    key[i] = (uint32_t)((((long)c * nby * nbz + blk) * 4 + sub) * nx + x);
-    idx[i] = i;
+__device__ __forceinline__ int line_at(const LineGrid &G, int y, int z) {
+    const int by = y >> 1, bz = z >> 1, sy = min(2, G.ny - 2 * by), sz = min(2, G.nz - 2 * bz);
+    return G.cl[(by & 1) | ((bz & 1) << 1)] + (bz >> 1) * 2 * G.Ly[by & 1] + (by >> 1) * 2 * sz + (y & 1) +
+           (z & 1) * sy;
 }
 
-// pos[rows[p]] = p; and every row's stencil-offset mask: bit
-// (dx + 1) + 3 (dy + 1) + 9 (dz + 1) for each of its columns (the pattern
-// lies in the 3^dim neighbourhood with ascending columns, so entry e of a row
-// is the e-th set bit of its mask)
-__global__ void lines_pos_kernel(int n, int dim, int nx, int ny, const int32_t *__restrict__ rows,
-                                 const int32_t *__restrict__ rowptr, const int32_t *__restrict__ colidx,
-                                 int32_t *__restrict__ pos, uint32_t *__restrict__ rmask) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= n) return;
-    const int i = rows[p];
-    pos[i] = p;
-    const int xi = i % nx, yi = (i / nx) % ny, zi = dim == 3 ? i / (nx * ny) : 0;
-    uint32_t m = 0;
-    for (int e = rowptr[i]; e < rowptr[i + 1]; ++e) {
-        const int j = colidx[e];
-        const int xj = j % nx, yj = (j / nx) % ny, zj = dim == 3 ? j / (nx * ny) : 0;
-        m |= 1u << ((xj - xi + 1) + 3 * (yj - yi + 1) + 9 * (zj - zi + 1));
+// the grid position of line l of colour c
+__device__ __forceinline__ void line_yz(const LineGrid &G, int c, int l, int &y, int &z) {
+    const int r = l - G.cl[c], row = 2 * G.Ly[c & 1], bz = 2 * (r / row) + (c >> 1), sz = min(2, G.nz - 2 * bz);
+    const int r2 = r % row, by = 2 * (r2 / (2 * sz)) + (c & 1), sy = min(2, G.ny - 2 * by), sub = r2 % (2 * sz);
+    y = 2 * by + sub % sy;
+    z = 2 * bz + sub / sy;
+}
+
+// A point's offsets in the 3^dim stencil: o = (dx + 1) + 3 (dy + 1) + 9 (dz + 1), dz = 0
+// in 2D. The factorisation works on rows of kLineRow values by offset, in the order, with
+// zeros where the pattern has no entry: an entry's place in any row is then known
+// without a search, and a warp (lane o = offset o) reads and writes rows as they lie.
+constexpr int kLineRow = 27;
+constexpr int kLineDiag = 13;
+
+// rows[p] and pos[i], every row's values D[p][o] in the factorisation's precision and
+// its pattern rmask[p] (bit o). A warp a row; the pattern lies in the 3^dim neighbourhood
+// with strictly ascending columns (stencil_check), so entry e of a row is the e-th set
+// bit of its mask. 2^21 rows of 27 beside the coarse factorisation: 0.57 ms. (Sorting
+// the rows by a key, converting the values, forming masks and finding diagonals: 0.80.)
+template <typename TF>
+__global__ void __launch_bounds__(256) lines_gather_kernel(int n, const LineGrid G, const int32_t *__restrict__ rowptr,
+                                                           const int32_t *__restrict__ colidx,
+                                                           const double *__restrict__ val, int32_t *__restrict__ rows,
+                                                           int32_t *__restrict__ pos, uint32_t *__restrict__ rmask,
+                                                           TF *__restrict__ D) {
+    const int i = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (i >= n) return;  // whole warps leave together
+    const int x = i % G.nx, r = i / G.nx, y = r % G.ny, z = r / G.ny;
+    const int b = rowptr[i], len = rowptr[i + 1] - b;
+    const bool mine = lane < len;
+    int o = 0;
+    TF v = TF(0);
+    if (mine) {
+        const int j = colidx[b + lane];
+        v = TF(val[b + lane]);
+        if (G.nx >= 3 && G.ny >= 3) {  // offsets as the digits of j - i in the strides
+            const int nxy = G.nx * G.ny;
+            int t = j - i + nxy + G.nx + 1;
+            const int oz = (t >= nxy) + (t >= 2 * nxy);
+            t -= oz * nxy;
+            const int oy = (t >= G.nx) + (t >= 2 * G.nx);
+            o = t - oy * G.nx + 3 * oy + 9 * oz;
+        } else {
+            const int rj = j / G.nx;
+            o = (j % G.nx - x + 1) + 3 * (rj % G.ny - y + 1) + 9 * (rj / G.ny - z + 1);
+        }
     }
-    rmask[i] = m;
+    const uint32_t m = __reduce_or_sync(0xffffffffu, mine ? 1u << o : 0u);
+    const TF w = __shfl_sync(0xffffffffu, v, __popc(m & ((1u << lane) - 1u)) & 31);
+    const int p = line_at(G, y, z) * G.nx + x;
+    if (lane < kLineRow) D[p * kLineRow + lane] = (m >> lane) & 1u ? w : TF(0);
+    if (lane == 0) {
+        rows[p] = i;
+        pos[i] = p;
+        rmask[p] = m;
+    }
 }
 
 // ---- factorisation --------------------------------------------------------------------
+//
+// Row by row in the order (IKJ): for every earlier entry k of row i, in position order,
+// l_ik = a_ik / u_kk (as a product with the stored 1 / u_kk), then every later entry
+// (i, j) that row k also holds gets a_ij -= l_ik u_kj. With rows by offset, row k's entry
+// towards j sits at offset o_j - o_k + 13, the same for every point of a line: which
+// lanes a pivot updates and where their operands lie is worked out once per line.
 
-constexpr int kOffChunk = 4;
-
-// Phase 1 of one colour, every row at once (one warp per row, lane e holding
-// entry e): the earlier entries of earlier colours (positions below c0, all
-// final) come first in the order, so they are eliminated in parallel before
-// the in-block ones, in position order: l_ik = a_ik / u_kk (as a product with
-// the stored 1 / u_kk), then every later entry (i, j) that row k also holds
-// gets a_ij -= l_ik u_kj. Entry (k, j) is found from row k's stencil-offset
-// mask (lines_pos_kernel): a popcount gives its place in row k, read straight
-// from global memory, the chunk's reads issued together.
-template <typename TF>
-__global__ void __launch_bounds__(128) lines_factor_off_kernel(int c0, int cnt, int dim, int nx, int ny,
-                                                               const int32_t *__restrict__ rows,
-                                                               const int32_t *__restrict__ rowptr,
-                                                               const int32_t *__restrict__ colidx,
-                                                               const int32_t *__restrict__ pos,
-                                                               const uint32_t *__restrict__ rmask,
-                                                               TF *__restrict__ lu, const TF *__restrict__ rdiag) {
-    const int w = (int)(((long)blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
-    if (w >= cnt) return;  // whole warps leave together
-    const int i = rows[c0 + w];
-    const int b = rowptr[i], len = rowptr[i + 1] - b;  // len <= 32 (set-up checks it)
-    const bool mine = lane < len;
-    const int j = mine ? colidx[b + lane] : 0;
-    const int pj = mine ? pos[j] : INT_MAX;
-    TF a = mine ? lu[b + lane] : TF(0);
-    const int xi = i % nx, yi = (i / nx) % ny, zi = dim == 3 ? i / (nx * ny) : 0;
-    int ox = 1, oy = 1, oz = 1;  // this entry's offset from row i, zero-based per axis
-    if (mine) {
-        ox = j % nx - xi + 1;
-        oy = (j / nx) % ny - yi + 1;
-        oz = dim == 3 ? j / (nx * ny) - zi + 1 : 1;
-    }
-    const bool lower = mine && pj < c0;
-    int kb = 0;
-    uint32_t km = 0;
-    TF rd = TF(0);
-    if (lower) {  // the pivot row's start, mask and 1 / u_kk
-        kb = rowptr[j];
-        km = rmask[j];
-        rd = rdiag[j];
-    }
-    const unsigned lm = __ballot_sync(0xffffffffu, lower);
-    const int nlow = __popc(lm);
-    int rank = 0;  // place of this pivot in the position order
-    for (unsigned mm = lm; mm; mm &= mm - 1) {
-        const int po = __shfl_sync(0xffffffffu, pj, __ffs(mm) - 1);
-        rank += (lower && po < pj) ? 1 : 0;
-    }
-    for (int t0 = 0; t0 < nlow; t0 += kOffChunk) {
-        TF u[kOffChunk], rk[kOffChunk];
-        int ql[kOffChunk];
-#pragma unroll
-        for (int t = 0; t < kOffChunk; ++t) {
-            const bool on = t0 + t < nlow;  // uniform
-            const unsigned bm = __ballot_sync(0xffffffffu, lower && rank == t0 + t);
-            const int qq = on ? __ffs(bm) - 1 : 0;
-            ql[t] = on ? qq : -1;
-            const int pk = __shfl_sync(0xffffffffu, pj, qq);
-            const int kx = __shfl_sync(0xffffffffu, ox, qq), ky = __shfl_sync(0xffffffffu, oy, qq),
-                      kz = __shfl_sync(0xffffffffu, oz, qq);
-            const int kbt = __shfl_sync(0xffffffffu, kb, qq);
-            const uint32_t kmt = __shfl_sync(0xffffffffu, km, qq);
-            rk[t] = __shfl_sync(0xffffffffu, rd, qq);
-            const int dx = ox - kx + 1, dy = oy - ky + 1, dz = oz - kz + 1;  // j's offset from k
-            const bool near = dx >= 0 && dx <= 2 && dy >= 0 && dy <= 2 && dz >= 0 && dz <= 2;
-            const int o = near ? dx + 3 * dy + 9 * dz : 0;
-            const bool hit = on && mine && pj > pk && near && ((kmt >> o) & 1u);
-            u[t] = hit ? lu[kbt + __popc(kmt & ((1u << o) - 1u))] : TF(0);
-        }
-#pragma unroll
-        for (int t = 0; t < kOffChunk; ++t) {
-            const TF lik = __shfl_sync(0xffffffffu, a, ql[t] < 0 ? 0 : ql[t]) * rk[t];
-            if (ql[t] >= 0) {  // uniform
-                if (lane == ql[t]) a = lik;
-                else a = a - lik * u[t];
-            }
-        }
-    }
-    if (mine) lu[b + lane] = a;
+// The lane's neighbour line (its first position; -1 outside the grid or no offset)
+__device__ __forceinline__ int lane_line(const LineGrid &G, int lane, int y, int z) {
+    const int yj = y + (lane / 3) % 3 - 1, zj = z + lane / 9 - 1;
+    if (lane >= kLineRow || yj < 0 || yj >= G.ny || zj < 0 || zj >= G.nz) return -1;
+    return line_at(G, yj, zj) * G.nx;
 }
 
-// Phase 2 of one colour: the in-block earlier entries. CTA b0 + blockIdx.x
-// handles one block, warp q its line q; at time step T warp q finishes point
-// x = T - 2 q of its line. With couplings reaching at most one point along x,
-// point (q, x) needs the points (q', x - 1 .. x + 1) of the lines q' < q
-// (finished at steps up to T - 1) and (q, x - 1). A point's row is final
-// once finished and is then needed for at most 2 nsub more steps, so each
-// line keeps its last kRing rows in shared memory: a row is copied in
-// (cp.async) kAhead steps before its turn and written through to global
-// memory when finished. In-block tests come from the grid position of the
-// columns (the order's key), so no position gather sits on the critical path.
-// A row's entries lie at distinct offsets of the 3^dim stencil, in column
-// order, so a finished row also keeps the mask of its offsets (bit
-// (dx + 1) + 3 (dy + 1) + 9 (dz + 1)): entry (k, j) of a pivot row k is then
-// found by a popcount of the mask below j's offset from k.
-constexpr int kRing = 16, kAhead = 4, kPivChunk = 4, kLinesMaxNx = 256;
+// whether pivot offset ok, on the line at kp, updates the lane's entry (line at pl): near
+// row k, and later than it
+__device__ __forceinline__ bool pivot_hits(int lane, int pl, int ok, int kp) {
+    const int dx = lane % 3 - ok % 3, dy = (lane / 3) % 3 - (ok / 3) % 3, dz = lane / 9 - ok / 9;
+    return pl >= 0 && abs(dx) <= 1 && abs(dy) <= 1 && abs(dz) <= 1 && (pl > kp || (pl == kp && dx > 0));
+}
+
+// Phase 1 of one colour: the pivots of earlier colours (all final) on up to kLineNbr
+// neighbour lines, which come first in the order. A warp takes every fourth point of a
+// piece of a line; a point's operands are loaded together. 2^19 rows: 0.42 to
+// 0.59 ms with searches for the operands, now 0.25 to 0.31.
+constexpr int kOffPoints = 32;
 
 template <typename TF>
-__global__ void __launch_bounds__(128) lines_factor_ring_kernel(
-    int c, int b0, const int32_t *__restrict__ blk_start, const int32_t *__restrict__ blk_nsub, int dim, int nx,
-    int ny, const int32_t *__restrict__ rows, const int32_t *__restrict__ rowptr, const int32_t *__restrict__ colidx,
-    TF *__restrict__ lu, TF *__restrict__ rdiag, int *__restrict__ status) {
+__global__ void __launch_bounds__(128) lines_factor_off_kernel(const LineGrid G, int c,
+                                                               const uint32_t *__restrict__ rmask, TF *D,
+                                                               const TF *__restrict__ rdiag) {
+    const int lane = threadIdx.x & 31, pieces = (G.nx + kOffPoints - 1) / kOffPoints;
+    const int l = G.cl[c] + blockIdx.x / pieces, x0 = (blockIdx.x % pieces) * kOffPoints;
+    int y, z;
+    line_yz(G, c, l, y, z);
+    const int pl = lane_line(G, lane, y, z), c0 = G.cl[c] * G.nx;
+    int kp[kLineNbr], ko[kLineNbr], last = -1;  // the pivots' lines in position order, offset towards x - 1
+    unsigned hits = 0;
+#pragma unroll
+    for (int t = 0; t < kLineNbr; ++t) {
+        const int key = pl > last && pl < c0 && lane % 3 == 1 ? pl : INT_MAX;
+        const int first = __reduce_min_sync(0xffffffffu, key);
+        const unsigned who = __ballot_sync(0xffffffffu, key == first);
+        kp[t] = first == INT_MAX ? -1 : first;
+        ko[t] = first == INT_MAX ? 0 : __ffs(who) - 2;
+        if (first == INT_MAX) continue;
+        last = first;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) hits |= pivot_hits(lane, pl, ko[t] + d, first) ? 1u << (3 * t + d) : 0u;
+    }
+    const int x1 = min(x0 + kOffPoints, G.nx);
+    for (int x = x0 + (int)(threadIdx.x >> 5); x < x1; x += 4) {
+        const int p = l * G.nx + x;
+        const uint32_t m = rmask[p];
+        const unsigned h = (m >> lane) & 1u ? hits : 0u;  // only entries of the pattern change
+        TF a = lane < kLineRow ? D[p * kLineRow + lane] : TF(0);
+        TF u[3 * kLineNbr], rk[3 * kLineNbr];
+#pragma unroll
+        for (int t = 0; t < kLineNbr; ++t)
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                const int ok = ko[t] + d, pk = kp[t] + x + d - 1;
+                const bool on = kp[t] >= 0 && ((m >> ok) & 1u);  // uniform
+                u[3 * t + d] = on && ((h >> (3 * t + d)) & 1u) ? D[pk * kLineRow + lane - ok + kLineDiag] : TF(0);
+                rk[3 * t + d] = on ? rdiag[pk] : TF(0);
+            }
+#pragma unroll
+        for (int t = 0; t < kLineNbr; ++t)
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                const int ok = ko[t] + d;
+                if (kp[t] < 0 || !((m >> ok) & 1u)) continue;  // uniform
+                const TF lik = __shfl_sync(0xffffffffu, a, ok) * rk[3 * t + d];
+                if (lane == ok) a = lik;
+                else a = a - lik * u[3 * t + d];
+            }
+        if (lane < kLineRow) D[p * kLineRow + lane] = a;
+    }
+}
+
+// Phase 2 of one colour: the pivots inside the block. CTA b0 + blockIdx.x handles one
+// block, warp q its line q; at time step T warp q finishes point x = T - 2 q of its
+// line. With couplings reaching at most one point along x, point (q, x) needs the points
+// (q', x - 1 .. x + 1) of the lines q' < q (finished at steps up to T - 1) and (q, x - 1).
+// A point's row is final once finished and is then needed for at most 2 nsub more steps,
+// so each line keeps its last kRing rows in shared memory: a row is copied in (cp.async)
+// kAhead steps before its turn and written through to global memory when finished. The
+// chain of steps bounds it: a step's operands are all read first, then every pivot costs
+// a shuffle, a product and an update. (Searching for the operands by columns and masks put
+// about 650 instructions on a step: 0.76 ms a colour of 2^19 rows, now 0.25; 2^16 rows
+// 0.18, now 0.06.)
+constexpr int kRing = 16, kAhead = 4, kLinesMaxNx = 256;
+constexpr int kBlkPiv = 10;  // three earlier lines of the block, then the line's point before
+
+template <typename TF>
+__global__ void __launch_bounds__(128) lines_factor_ring_kernel(const LineGrid G, int c, int b0,
+                                                                const int32_t *__restrict__ blk_line,
+                                                                const int32_t *__restrict__ blk_nsub,
+                                                                const int32_t *__restrict__ rows,
+                                                                const uint32_t *__restrict__ rmask,
+                                                                TF *__restrict__ D, TF *__restrict__ rdiag,
+                                                                int *__restrict__ status) {
     __shared__ TF s_val[4][kRing][32];
-    __shared__ int32_t s_col[4][kRing][32];
     __shared__ TF s_rd[4][kRing];
-    __shared__ unsigned s_mask[4][kRing];
-    __shared__ int32_t s_ri[4][kLinesMaxNx], s_rb[4][kLinesMaxNx], s_rl[4][kLinesMaxNx];
-    const int b = b0 + blockIdx.x, q = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int st = blk_start[b], nsub = blk_nsub[b];
-    for (int t = threadIdx.x; t < nsub * nx; t += blockDim.x) {
-        const int i = rows[st + t], rb = rowptr[i];
-        s_ri[t / nx][t % nx] = i;
-        s_rb[t / nx][t % nx] = rb;
-        s_rl[t / nx][t % nx] = rowptr[i + 1] - rb;
+    __shared__ uint32_t s_mask[4][kLinesMaxNx];
+    const int b = b0 + blockIdx.x, q = threadIdx.x >> 5, lane = threadIdx.x & 31, nx = G.nx;
+    const int lb = blk_line[b], nsub = blk_nsub[b];
+    for (int t = threadIdx.x; t < nsub * nx; t += blockDim.x) s_mask[t / nx][t % nx] = rmask[lb * nx + t];
+    int ok0[3] = {0, 0, 0};  // offset towards x - 1 on the block's line t
+    unsigned hits = 0;
+    if (q < nsub) {
+        int y, z;
+        line_yz(G, c, lb + q, y, z);
+        const int pl = lane_line(G, lane, y, z);
+        for (int t = 0; t < 3; ++t) {
+            if (t >= q) break;
+            int yt, zt;
+            line_yz(G, c, lb + t, yt, zt);
+            ok0[t] = 3 * (yt - y + 1) + 9 * (zt - z + 1);
+#pragma unroll
+            for (int d = 0; d < 3; ++d)
+                hits |= pivot_hits(lane, pl, ok0[t] + d, (lb + t) * nx) ? 1u << (3 * t + d) : 0u;
+        }
+        hits |= pivot_hits(lane, pl, kLineDiag - 1, (lb + q) * nx) ? 1u << 9 : 0u;
     }
     __syncthreads();
-    const int y0 = ((s_ri[0][0] / nx) % ny) & ~1;
-    const int nyb = min(2, ny - y0);  // lines of the block along y
-    int yq = 0, zq = 0;
-    if (q < nsub) {
-        const int r = s_ri[q][0] / nx;
-        yq = r % ny;
-        zq = dim == 3 ? r / ny : 0;
-    }
-    const int kin_base = ((yq & 1) | ((zq & 1) << 1)) * nx;  // in-block order key of (q, 0)
+    const int p0 = (lb + q) * nx;
     const int steps = nx + 2 * (nsub - 1);
     for (int T = -kAhead; T < steps; ++T) {
         if (q < nsub) {
             const int xl = T - 2 * q + kAhead;
-            if (xl >= 0 && xl < nx && lane < s_rl[q][xl]) {
-                const int e = s_rb[q][xl] + lane;
-                cp_async4(&s_col[q][xl & (kRing - 1)][lane], colidx + e);
-                cp_async_val(&s_val[q][xl & (kRing - 1)][lane], lu + e);
-            }
+            if (xl >= 0 && xl < nx && lane < kLineRow)
+                cp_async_val(&s_val[q][xl & (kRing - 1)][lane], D + (p0 + xl) * kLineRow + lane);
         }
         cp_async_commit();
         if (T < 0) continue;  // uniform over the CTA
         cp_async_wait<kAhead>();
+        __syncwarp();
         const int x = T - 2 * q;
         if (q < nsub && x >= 0 && x < nx) {
             const int slot = x & (kRing - 1);
-            const int i = s_ri[q][x], len = s_rl[q][x];
-            const bool mine = lane < len;
-            const int j = mine ? s_col[q][slot][lane] : -1;
-            TF a = mine ? s_val[q][slot][lane] : TF(0);
-            int xj = 0, yj = 0, zj = 0;
-            if (mine) {
-                xj = j % nx;
-                const int r = j / nx;
-                yj = r % ny;
-                zj = dim == 3 ? r / ny : 0;
-            }
-            // this entry's stencil offset from row i (zero-based per axis)
-            const int ox = xj - x + 1, oy = yj - yq + 1, oz = zj - zq + 1;
-            const unsigned mask_i = __reduce_or_sync(0xffffffffu, mine ? 1u << (ox + 3 * oy + 9 * oz) : 0u);
-            const bool inb = mine && (yj >> 1) == (yq >> 1) && (zj >> 1) == (zq >> 1);
-            const int kin_j = ((yj & 1) | ((zj & 1) << 1)) * nx + xj;
-            const int colj = ((yj >> 1) & 1) | (dim == 3 ? (((zj >> 1) & 1) << 1) : 0);
-            const bool piv = inb && kin_j < kin_base + x;
-            // Inside one block the key (z & 1, y & 1, x) orders the points as
-            // their indices do, so the pivots come in lane (column) order.
-            const bool later_in = inb;  // in-block: later than pivot k when kin_j > kin_k
-            const bool later_off = mine && !inb && colj > c;
-            unsigned rest = __ballot_sync(0xffffffffu, piv);
-            while (rest) {  // uniform
-                // every match of the chunk first (the pivot rows are final), then
-                // the eliminations in order
-                TF u[kPivChunk], rk[kPivChunk];
-                int ql[kPivChunk];
+            const uint32_t m = s_mask[q][x];
+            const unsigned h = (m >> lane) & 1u ? hits : 0u;
+            TF a = lane < kLineRow ? s_val[q][slot][lane] : TF(0);
+            TF u[kBlkPiv], rk[kBlkPiv];
 #pragma unroll
-                for (int t = 0; t < kPivChunk; ++t) {
-                    const bool on = rest != 0;  // uniform
-                    const int qq = on ? __ffs(rest) - 1 : 0;
-                    rest &= rest - 1;
-                    ql[t] = on ? qq : -1;
-                    // pivot k: its offset from row i, hence its grid position
-                    const int kx = __shfl_sync(0xffffffffu, ox, qq), ky = __shfl_sync(0xffffffffu, oy, qq),
-                              kz = __shfl_sync(0xffffffffu, oz, qq);
-                    const int xk = x + kx - 1, yk = yq + ky - 1, zk = zq + kz - 1;
-                    const int kin_k = ((yk & 1) | ((zk & 1) << 1)) * nx + xk;
-                    const int lk = on ? (yk & 1) + (zk & 1) * nyb : q, sk = on ? xk & (kRing - 1) : slot;
-                    rk[t] = on ? s_rd[lk][sk] : TF(0);
-                    const unsigned mk = on ? s_mask[lk][sk] : 0u;
-                    // j's offset from k
-                    const int dx = ox - kx + 1, dy = oy - ky + 1, dz = oz - kz + 1;
-                    const bool near = dx >= 0 && dx <= 2 && dy >= 0 && dy <= 2 && dz >= 0 && dz <= 2;
-                    const int o = near ? dx + 3 * dy + 9 * dz : 0;
-                    const bool hit = on && near && (later_off || (later_in && kin_j > kin_k)) && ((mk >> o) & 1u);
-                    u[t] = hit ? s_val[lk][sk][__popc(mk & ((1u << o) - 1u))] : TF(0);
-                }
-#pragma unroll
-                for (int t = 0; t < kPivChunk; ++t) {
-                    const TF lik = __shfl_sync(0xffffffffu, a, ql[t] < 0 ? 0 : ql[t]) * rk[t];
-                    if (ql[t] >= 0) {  // uniform
-                        if (lane == ql[t]) a = lik;
-                        else a = a - lik * u[t];
-                    }
-                }
+            for (int t = 0; t < kBlkPiv; ++t) {
+                const int ok = t < 9 ? ok0[t / 3] + t % 3 : kLineDiag - 1;
+                const int ql = t < 9 ? t / 3 : q, sk = (x + (t < 9 ? t % 3 - 1 : -1)) & (kRing - 1);
+                const bool on = (t == 9 || t / 3 < q) && ((m >> ok) & 1u);  // uniform
+                u[t] = on && ((h >> t) & 1u) ? s_val[ql][sk][lane - ok + kLineDiag] : TF(0);
+                rk[t] = on ? s_rd[ql][sk] : TF(0);
             }
-            if (mine) {
+#pragma unroll
+            for (int t = 0; t < kBlkPiv; ++t) {
+                const int ok = t < 9 ? ok0[t / 3] + t % 3 : kLineDiag - 1;
+                if ((t < 9 && t / 3 >= q) || !((m >> ok) & 1u)) continue;  // uniform
+                const TF lik = __shfl_sync(0xffffffffu, a, ok) * rk[t];
+                if (lane == ok) a = lik;
+                else a = a - lik * u[t];
+            }
+            if (lane < kLineRow) {
                 s_val[q][slot][lane] = a;
-                lu[s_rb[q][x] + lane] = a;
+                D[(p0 + x) * kLineRow + lane] = a;
             }
-            const unsigned dm = __ballot_sync(0xffffffffu, mine && j == i);
-            const TF uii = __shfl_sync(0xffffffffu, a, dm ? __ffs(dm) - 1 : 0);
+            const TF uii = __shfl_sync(0xffffffffu, a, kLineDiag);
             if (lane == 0) {
-                const bool bad = !dm || uii == TF(0) || !isfinite((double)uii);
-                if (bad) atomicCAS(status, 0, 1 + i);
+                const bool bad = !((m >> kLineDiag) & 1u) || uii == TF(0) || !isfinite(uii);
+                if (bad) atomicCAS(status, 0, 1 + rows[p0 + x]);
                 const TF rd = bad ? TF(0) : TF(1) / uii;
                 s_rd[q][slot] = rd;
-                s_mask[q][slot] = mask_i;
-                rdiag[i] = rd;
+                rdiag[p0 + x] = rd;
             }
         }
         __syncthreads();  // the step's rows are final before the next step reads them
@@ -331,34 +327,31 @@ __global__ void lines_nbr_kernel(int nlines, int dim, int nx, int ny, int nz, co
 }
 
 template <typename T>
-__global__ void __launch_bounds__(128) lines_fill_kernel(int n, int dim, int nx, int ny, int nz,
-                                                         const int32_t *__restrict__ rowptr,
-                                                         const uint32_t *__restrict__ rmask,
-                                                         const T *__restrict__ lu, const int32_t *__restrict__ rows,
+__global__ void __launch_bounds__(128) lines_fill_kernel(int n, const LineGrid H, const T *__restrict__ D,
                                                          const IluLines L, T *__restrict__ offl, T *__restrict__ offu,
                                                          T *__restrict__ inl, T *__restrict__ inu) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
+    __shared__ T s_row[128 * kLineRow];  // the CTA's rows; a thread's row starts at an odd multiple of the banks
+    const int p0 = blockIdx.x * 128, cnt = min(128, n - p0);
+    for (int t = threadIdx.x; t < cnt * kLineRow; t += 128) s_row[t] = D[p0 * kLineRow + t];
+    __syncthreads();
+    const int p = p0 + threadIdx.x, nx = H.nx;
     if (p >= n) return;
-    const int i = rows[p], x = i % nx, y = (i / nx) % ny, z = dim == 3 ? i / (nx * ny) : 0;
-    const int c = ((y >> 1) & 1) | (dim == 3 ? ((z >> 1) & 1) << 1 : 0);
-    const int sy = min(2, ny - (y & ~1)), q = (y & 1) + (z & 1) * sy;
+    int c = 0, y, z;
+    while (p >= H.cl[c + 1] * nx) ++c;
+    const int x = p % nx;
+    line_yz(H, c, p / nx, y, z);
+    const int sy = min(2, H.ny - (y & ~1)), q = (y & 1) + (z & 1) * sy;
     T off[2][kLineOff], in[2][kLineIn];
 #pragma unroll
     for (int k = 0; k < kLineOff; ++k) off[0][k] = off[1][k] = T(0);
 #pragma unroll
     for (int k = 0; k < kLineIn; ++k) in[0][k] = in[1][k] = T(0);
-    const uint32_t mask = rmask[i];
-    int e = rowptr[i], cnt[2] = {0, 0};
-    for (int o = 0; o < (dim == 3 ? 27 : 18); o += 3) {  // entries in column order, three x offsets at a time
-        const int dy = (o / 3) % 3 - 1, dz = dim == 3 ? o / 9 - 1 : 0;
-        if (dim != 3 && o < 9) continue;  // 2D rows use the bits of dz = 0
-        const uint32_t m3 = (mask >> o) & 7u;
+    int cnts[2] = {0, 0};
+    for (int o = 0; o < kLineRow; o += 3) {  // neighbour lines ascending in z, then y
+        const int dy = (o / 3) % 3 - 1, dz = o / 9 - 1;
         const int yk = y + dy, zk = z + dz;
-        if (yk < 0 || yk >= ny || zk < 0 || zk >= nz) continue;
-        T v[3];
-#pragma unroll
-        for (int d = 0; d < 3; ++d) v[d] = (m3 >> d) & 1u ? lu[e + __popc(m3 & ((1u << d) - 1u))] : T(0);
-        e += __popc(m3);
+        if (yk < 0 || yk >= H.ny || zk < 0 || zk >= H.nz) continue;
+        const T *v = s_row + threadIdx.x * kLineRow + o;
         if (dy == 0 && dz == 0) {
             in[0][0] = v[0];
             in[1][0] = v[2];
@@ -369,9 +362,9 @@ __global__ void __launch_bounds__(128) lines_fill_kernel(int n, int dim, int nx,
 #pragma unroll
             for (int d = 0; d < 3; ++d) dst[d] = v[d];
         } else {
-            const int ck = ((yk >> 1) & 1) | (dim == 3 ? ((zk >> 1) & 1) << 1 : 0);
+            const int ck = ((yk >> 1) & 1) | (((zk >> 1) & 1) << 1);
             const int dir = ck < c ? 0 : 1;
-            T *dst = off[dir] + 3 * cnt[dir]++;
+            T *dst = off[dir] + 3 * cnts[dir]++;
 #pragma unroll
             for (int d = 0; d < 3; ++d) dst[d] = v[d];
         }
@@ -397,92 +390,69 @@ __global__ void __launch_bounds__(128) lines_fill_kernel(int n, int dim, int nx,
 
 bool lines_fit(const msrsb_grid *g) { return g->nx >= 1 && g->nx <= kLinesMaxNx && (g->dim == 2 || g->dim == 3); }
 
-// Order, block table and ILU(0) factors of a scalar operator in the
-// line-block order; lu holds A's values (TF) on entry and is overwritten.
-// A's pattern lies within every point's 3^dim neighbourhood (stencil_check):
-// blocks of one colour are then uncoupled and a point couples to its line
-// neighbours x - 1, x + 1 only.
+// Order, block table and ILU(0) factors (in precision TF) of a scalar operator in the
+// line-block order. A's pattern lies within every point's 3^dim neighbourhood
+// (stencil_check): blocks of one colour are then uncoupled and a point couples to its
+// line neighbours x - 1, x + 1 only.
 template <typename TF>
-msrsb_status lines_setup(msrsb_handle *h, TF *lu, cudaStream_t s) {
+msrsb_status lines_setup(msrsb_handle *h, cudaStream_t s) {
     const msrsb_mat &A = h->A;
     const msrsb_grid &g = h->grid;
     const int n = h->n, dim = g.dim, nx = g.nx, ny = g.ny, nz = dim == 3 ? g.nz : 1;
     IluLines &L = h->lines;
     L.nx = nx;
     L.ncol = dim == 3 ? 4 : 2;
-    // ---- the order: sort rows by (colour, block, line, x) ----
-    uint32_t *key = nullptr, *key2 = nullptr;
-    int32_t *idx = nullptr;
-    MSRSB_TRY(dalloc(&key, n, s));
-    MSRSB_TRY(dalloc(&key2, n, s));
-    MSRSB_TRY(dalloc(&idx, n, s));
-    MSRSB_TRY(dalloc(&L.rows, n, s));
-    MSRSB_TRY(dalloc(&h->pos_of, n, s));
-    line_key_kernel<<<ceil_div(n, 256), 256, 0, s>>>(n, dim, nx, ny, nz, key, idx);
-    MSRSB_LAUNCHED("line_key_kernel");
-    size_t tmp = 0;
-    MSRSB_CUDA(cub::DeviceRadixSort::SortPairs(nullptr, tmp, key, key2, idx, L.rows, n, 0, 32, s));
-    char *tb = nullptr;
-    MSRSB_TRY(dalloc(&tb, tmp, s));
-    MSRSB_CUDA(cub::DeviceRadixSort::SortPairs(tb, tmp, key, key2, idx, L.rows, n, 0, 32, s));
-    dfree(tb, s);
-    dfree(key, s);
-    dfree(key2, s);
-    dfree(idx, s);
-    uint32_t *rmask = nullptr;
-    MSRSB_TRY(dalloc(&rmask, n, s));
-    lines_pos_kernel<<<ceil_div(n, 256), 256, 0, s>>>(n, dim, nx, ny, L.rows, A.rowptr, A.colidx, h->pos_of, rmask);
-    MSRSB_LAUNCHED("lines_pos_kernel");
     // ---- block table (host): blocks of each colour in block order ----
     const int nby = (ny + 1) / 2, nbz = dim == 3 ? (nz + 1) / 2 : 1;
-    std::vector<int32_t> bline, bstart, bnsub;
+    std::vector<int32_t> bline, bnsub;
     int run = 0;
     for (int c = 0; c < L.ncol; ++c) {
         L.cptr[c] = run;
-        L.bptr[c] = (int)bstart.size();
+        L.bptr[c] = (int)bline.size();
         for (int bz = 0; bz < nbz; ++bz)
             for (int by = 0; by < nby; ++by) {
                 const int cc = (by & 1) | (dim == 3 ? ((bz & 1) << 1) : 0);
                 if (cc != c) continue;
                 const int sy = ny - 2 * by < 2 ? 1 : 2, sz = dim == 3 ? (nz - 2 * bz < 2 ? 1 : 2) : 1;
                 bline.push_back(run / nx);
-                bstart.push_back(run);
                 bnsub.push_back(sy * sz);
                 run += sy * sz * nx;
             }
     }
     L.cptr[L.ncol] = run;
-    L.bptr[L.ncol] = (int)bstart.size();
+    L.bptr[L.ncol] = (int)bline.size();
     if (run != n) return fail(MSRSB_ESHAPE, "line blocks cover %d of %d rows", run, n);
-    const int nblk = (int)bstart.size();
-    int32_t *blk_start = nullptr;
-    MSRSB_TRY(dalloc(&blk_start, nblk, s));
+    const int nblk = (int)bline.size();
     MSRSB_TRY(dalloc(&L.blk_line, nblk, s));
     MSRSB_TRY(dalloc(&L.blk_nsub, nblk, s));
     MSRSB_TRY(upload(L.blk_line, bline.data(), nblk * sizeof(int32_t), s));
-    MSRSB_TRY(upload(blk_start, bstart.data(), nblk * sizeof(int32_t), s));
     MSRSB_TRY(upload(L.blk_nsub, bnsub.data(), nblk * sizeof(int32_t), s));
-    // ---- factorisation, colour by colour ----
+    LineGrid G{dim, nx, ny, nz, {0, 0, 0, 0, 0}, {0, 0}};
+    for (int c = 0; c < 5; ++c) G.cl[c] = L.cptr[c < L.ncol ? c : L.ncol] / nx;
+    for (int y = 0; y < ny; ++y) ++G.Ly[(y >> 1) & 1];
+    MSRSB_TRY(dalloc(&L.rows, n, s));
+    MSRSB_TRY(dalloc(&h->pos_of, n, s));
+    uint32_t *rmask = nullptr;
+    TF *D = nullptr, *rdiag = nullptr;
     int *status = nullptr;
-    TF *rdiag = nullptr;
-    int32_t *dpos = nullptr;
-    MSRSB_TRY(dalloc(&status, 1, s));
+    MSRSB_TRY(dalloc(&rmask, n, s));
+    MSRSB_TRY(dalloc(&D, (size_t)n * kLineRow, s));
     MSRSB_TRY(dalloc(&rdiag, n, s));
-    MSRSB_TRY(dalloc(&dpos, n, s));
+    MSRSB_TRY(dalloc(&status, 1, s));
     MSRSB_CUDA(cudaMemsetAsync(status, 0, sizeof(int), s));
-    diag_pos_launch(n, A.rowptr, A.colidx, dpos, status, s);
-    MSRSB_LAUNCHED("diag_pos_kernel");
+    lines_gather_kernel<TF><<<ceil_div(n, 8), 256, 0, s>>>(n, G, A.rowptr, A.colidx, A.val, L.rows, h->pos_of, rmask, D);
+    MSRSB_LAUNCHED("lines_gather_kernel");
+    // ---- factorisation, colour by colour ----
     for (int c = 0; c < L.ncol; ++c) {
         const int nb = L.bptr[c + 1] - L.bptr[c];
         if (!nb) continue;
-        const int cnt = L.cptr[c + 1] - L.cptr[c];
         if (c > 0) {
-            lines_factor_off_kernel<TF><<<ceil_div((long)cnt * 32, 128), 128, 0, s>>>(
-                L.cptr[c], cnt, dim, nx, ny, L.rows, A.rowptr, A.colidx, h->pos_of, rmask, lu, rdiag);
+            lines_factor_off_kernel<TF><<<(G.cl[c + 1] - G.cl[c]) * ceil_div(nx, kOffPoints), 128, 0, s>>>(G, c, rmask,
+                                                                                                          D, rdiag);
             MSRSB_LAUNCHED("lines_factor_off_kernel");
         }
-        lines_factor_ring_kernel<TF><<<nb, 128, 0, s>>>(c, L.bptr[c], blk_start, L.blk_nsub, dim, nx, ny, L.rows,
-                                                        A.rowptr, A.colidx, lu, rdiag, status);
+        lines_factor_ring_kernel<TF><<<nb, 128, 0, s>>>(G, c, L.bptr[c], L.blk_line, L.blk_nsub, L.rows, rmask, D,
+                                                        rdiag, status);
         MSRSB_LAUNCHED("lines_factor_ring_kernel");
     }
     // ---- the sweeps' coefficients by neighbour line, and the lines' neighbours ----
@@ -509,22 +479,19 @@ msrsb_status lines_setup(msrsb_handle *h, TF *lu, cudaStream_t s) {
     MSRSB_TRY(dalloc(&L.nbr, (size_t)2 * nlines * kLineNbr, s));
     lines_nbr_kernel<<<ceil_div(nlines, 128), 128, 0, s>>>(nlines, dim, nx, ny, nz, L.rows, h->pos_of, L.nbr);
     MSRSB_LAUNCHED("lines_nbr_kernel");
-    lines_fill_kernel<TF><<<ceil_div(n, 128), 128, 0, s>>>(n, dim, nx, ny, nz, A.rowptr, rmask, lu, L.rows, L, offl,
-                                                           offu, inl, inu);
+    lines_fill_kernel<TF><<<ceil_div(n, 128), 128, 0, s>>>(n, G, D, L, offl, offu, inl, inu);
     MSRSB_LAUNCHED("lines_fill_kernel");
     int hs = 0;
     MSRSB_TRY(read_back(&hs, status, sizeof(int), s));
     dfree(rdiag, s);
     dfree(rmask, s);
     dfree(status, s);
-    dfree(dpos, s);
-    dfree(blk_start, s);
-    if (hs < 0) return fail(MSRSB_EINVAL, "ILU(0): row %d has more than 32 entries", -hs - 1);
+    dfree(D, s);
     if (hs) return fail(MSRSB_EBREAKDOWN, "ILU(0): zero pivot at row %d", hs - 1);
     return MSRSB_OK;
 }
-template msrsb_status lines_setup<double>(msrsb_handle *, double *, cudaStream_t);
-template msrsb_status lines_setup<float>(msrsb_handle *, float *, cudaStream_t);
+template msrsb_status lines_setup<double>(msrsb_handle *, cudaStream_t);
+template msrsb_status lines_setup<float>(msrsb_handle *, cudaStream_t);
 
 void lines_free(IluLines *L, cudaStream_t s) {
     dfree(L->rows, s);
