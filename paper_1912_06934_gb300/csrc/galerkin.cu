@@ -7,6 +7,7 @@
 // forms its row of A P, one entry per coarse node it couples to; (2) one CTA
 // per coarse node J sums P_iJ (A P)_i* over the rows of J's support.
 #include "common.cuh"
+#include <type_traits>
 #include <cub/device/device_radix_sort.cuh>
 #include <cub/device/device_scan.cuh>
 
@@ -78,138 +79,177 @@ msrsb_status build_transpose(int n, int W, int nc, const int32_t *p_ids, int32_t
     return MSRSB_OK;
 }
 
-// Residue code of every coarse node, code(L) = sum_d (L_d mod 3) 3^d. The
+// Residue code of a coarse node, code(L) = sum_d (L_d mod 3) 3^d. The
 // coarse nodes met in one fine row's neighbourhood span at most three
 // consecutive coarse coordinates per axis (a row on a coarse-node line sees
 // L-1..L+1, any other row L..L+2), so their codes are all different; and every
 // L that couples with J through a fine row of supp(J) satisfies |L_d - J_d| <= 1.
-__global__ void coarse_code_kernel(int nc, int nb0, int nb1, int dim, int8_t *__restrict__ code) {
-    int L = blockIdx.x * blockDim.x + threadIdx.x;
-    if (L >= nc) return;
-    int l0 = L % nb0, l1 = (L / nb0) % nb1, l2 = L / (nb0 * nb1);
-    code[L] = (int8_t)(l0 % 3 + 3 * (l1 % 3) + (dim == 3 ? 9 * (l2 % 3) : 0));
+// code[i][t]: that of row i's slot t, kNoCode where it is not used.
+constexpr unsigned kNoCode = 255;
+
+__global__ void coarse_code_kernel(long nW, int nb0, int nb1, int dim, const int32_t *__restrict__ p_ids,
+                                   uint8_t *__restrict__ code) {
+    const long e = (long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= nW) return;
+    const int L = p_ids[e];
+    unsigned c = kNoCode;
+    if (L >= 0) {
+        const int l0 = L % nb0, l1 = (L / nb0) % nb1, l2 = L / (nb0 * nb1);
+        c = l0 % 3 + 3 * (l1 % 3) + (dim == 3 ? 9 * (l2 % 3) : 0);
+    }
+    code[e] = (uint8_t)c;
 }
 
-// Pass 1, one thread per fine (block) row i:
-// AP[i][s][l][m] = sum_k A_ik[l][m] P^m_{k,L} over the coarse nodes L with
+// a value in FP64. FP32 to FP64 conversions share the narrow FP64 pipe with the FMAs
+// they feed, so values are widened by their bits: sign, exponent rebased by 1023 - 127,
+// fraction moved up by 29; subnormals are scaled into the normal range first (exactly,
+// by 2^32), infinities and NaN keep the largest exponent. Without a branch, in which a
+// conversion would be issued all the same.
+__device__ __forceinline__ double widen(double v) { return v; }
+__device__ __forceinline__ double widen(float v) {
+    const unsigned e = __float_as_uint(v) & 0x7f800000u;
+    const unsigned u = __float_as_uint(e == 0u ? v * 4294967296.0f : v), mag = u & 0x7fffffffu;
+    const unsigned base = e == 0u ? 0x38000000u - (32u << 20) : e == 0x7f800000u ? 0x70000000u : 0x38000000u;
+    const unsigned hi = (u & 0x80000000u) | (mag != 0u ? (mag >> 3) + base : 0u);
+    return __hiloint2double((int)hi, (int)(u << 29));
+}
+
+// Pass 1, one thread per fine (block) row i and component l (blockIdx.y):
+// AP[i][l][s][m] = sum_k A_ik[l][m] P^m_{k,L} over the coarse nodes L with
 // code s met through row i (FP64, fixed order: A's row order, then slots).
-template <typename T, int BD>
-__global__ void __launch_bounds__(128) ap_kernel(int n, int W, int ncode, const int32_t *__restrict__ rowptr,
-                                                 const int32_t *__restrict__ colidx, const double *__restrict__ val,
-                                                 const int32_t *__restrict__ p_ids, const T *__restrict__ P,
-                                                 const int8_t *__restrict__ code, double *__restrict__ AP) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
+// Bound by the FP64 pipe. The sums lie in a shared-memory column a thread (the code is
+// data-dependent); the slots of a row k have different codes, so their sums are read, updated
+// and written together; a row's codes are one vector, and its values too where P's
+// alignment allows it; the CTA's block of AP is written as it lies. FP32 basis, 2^21 scalar
+// rows of 27 entries: 2.0 ms with conversions and a sum at a time, now 1.29; 3x3
+// blocks, 49^3 rows: 0.99 ms with the sums in local memory, now 0.58.
+constexpr int kApThreads = 64;
+
+template <typename T, int BD, int NCODE, int W>
+__global__ void __launch_bounds__(kApThreads) ap_kernel(int n, int vec, const int32_t *__restrict__ rowptr,
+                                                            const int32_t *__restrict__ colidx,
+                                                            const double *__restrict__ val,
+                                                            const uint8_t *__restrict__ code,
+                                                            const T *__restrict__ P, double *__restrict__ AP) {
+    constexpr int TH = kApThreads, NS = NCODE * BD;
+    __shared__ double s_acc[NS * TH];
+    const int tx = threadIdx.x, i0 = blockIdx.x * TH, i = i0 + tx, l = blockIdx.y;
     const long nW = (long)n * W;
-    double acc[27 * BD * BD];
-    for (int q = 0; q < ncode * BD * BD; ++q) acc[q] = 0.0;
-    for (int e = rowptr[i]; e < rowptr[i + 1]; ++e) {
-        const int k = colidx[e];
-        double a[BD * BD];
 #pragma unroll
-        for (int q = 0; q < BD * BD; ++q) a[q] = val[(long)e * BD * BD + q];
-        for (int t = 0; t < W; ++t) {
-            const int L = p_ids[(long)k * W + t];
-            if (L < 0) continue;
-            const int s = code[L];
+    for (int q = 0; q < NS; ++q) s_acc[q * TH + tx] = 0.0;
+    if (i < n) {
+        for (int e = rowptr[i]; e < rowptr[i + 1]; ++e) {
+            const int k = colidx[e];
+            unsigned cw[W / 4];
+            alignas(16) T p[BD][W];
+#pragma unroll
+            for (int q = 0; q < W / 4; ++q) cw[q] = __ldg(reinterpret_cast<const unsigned *>(code + (long)k * W) + q);
 #pragma unroll
             for (int m = 0; m < BD; ++m) {
-                const double pkl = (double)P[m * nW + (long)k * W + t];
+                const T *src = P + m * nW + (long)k * W;
+                if (vec) {
 #pragma unroll
-                for (int l = 0; l < BD; ++l) acc[(s * BD + l) * BD + m] = fma(a[l * BD + m], pkl, acc[(s * BD + l) * BD + m]);
+                    for (int q = 0; q < W * (int)sizeof(T) / 16; ++q)
+                        reinterpret_cast<uint4 *>(p[m])[q] = __ldg(reinterpret_cast<const uint4 *>(src) + q);
+                } else {
+#pragma unroll
+                    for (int t = 0; t < W; ++t) p[m][t] = __ldg(src + t);
+                }
             }
+            double r[BD][W];
+            int at[W];
+#pragma unroll
+            for (int t = 0; t < W; ++t) {
+                const unsigned c = (cw[t >> 2] >> (8 * (t & 3))) & 255u;
+                at[t] = c == kNoCode ? -1 : (int)c * BD * TH + tx;
+#pragma unroll
+                for (int m = 0; m < BD; ++m)
+                    if (at[t] >= 0) r[m][t] = s_acc[at[t] + m * TH];
+            }
+#pragma unroll
+            for (int m = 0; m < BD; ++m) {
+                const double a = BD == 1 ? val[e] : val[((long)e * BD + l) * BD + m];
+#pragma unroll
+                for (int t = 0; t < W; ++t)
+                    if (at[t] >= 0) r[m][t] = fma(a, widen(p[m][t]), r[m][t]);
+            }
+#pragma unroll
+            for (int t = 0; t < W; ++t)
+#pragma unroll
+                for (int m = 0; m < BD; ++m)
+                    if (at[t] >= 0) s_acc[at[t] + m * TH] = r[m][t];
         }
     }
-    double *out = AP + (long)i * ncode * BD * BD;
-    for (int q = 0; q < ncode * BD * BD; ++q) out[q] = acc[q];
+    __syncthreads();
+    const int rows = min(TH, n - i0);
+    for (int idx = tx; idx < rows * NS; idx += TH) {
+        const int r = idx / NS, q = idx - r * NS;
+        AP[((long)(i0 + r) * BD + l) * NS + q] = s_acc[q * TH + r];
+    }
 }
 
-// Pass 2, one CTA per coarse node J: A_c[J*BD+l][L*BD+m] = sum over fine rows
-// i of supp(J) (ascending) of P^l_{iJ} AP[i][code(L)][l][m]; thread-private
-// sums, then a fixed-order block reduction. Writes J's whole stencil row:
-// Acs[J][q][l][m], q = sum_d (L_d - J_d + 1) 3^d, zero where L is off the grid.
-template <typename T, int BD>
-__global__ void __launch_bounds__(128) ptap_kernel(int n, int W, int nc, int ncode, int dim, int nb0, int nb1, int nb2,
+// Pass 2 for block operators, one CTA per coarse node J and component l (blockIdx.y):
+// A_c[J*BD+l][L*BD+m] = sum over fine rows i of supp(J) of P^l_{iJ} AP[i][l][code(L)][m].
+// A warp takes every eighth row, its lanes the row's sums (read as they lie); the
+// warps' sums are added in a fixed order. Writes J's whole stencil row: Acs[J][q][l][m],
+// q = sum_d (L_d - J_d + 1) 3^d, zero where L is off the grid. (A thread a row with 243
+// sums in local memory took 1.45 ms of 49^3 rows, now 0.39.)
+template <typename T, int BD, int NCODE>
+__global__ void __launch_bounds__(256) ptap_kernel(int n, int W, int dim, int nb0, int nb1, int nb2,
                                                    const T *__restrict__ P, const int32_t *__restrict__ pt_ptr,
                                                    const int32_t *__restrict__ pt_rows,
                                                    const int8_t *__restrict__ jslot, const double *__restrict__ AP,
                                                    double *__restrict__ Acs) {
-    constexpr int NQ = 27 * BD * BD;
-    __shared__ double red[NQ][4];
-    const int J = blockIdx.x;
-    const int sj = jslot[J];
-    const long nW = (long)n * W;
-    const int nq = ncode * BD * BD;
-    double acc[NQ];
-    for (int q = 0; q < nq; ++q) acc[q] = 0.0;
-    for (int r = pt_ptr[J] + threadIdx.x; r < pt_ptr[J + 1]; r += blockDim.x) {
-        const int i = pt_rows[r];
-        const double *api = AP + (long)i * nq;
+    constexpr int NS = NCODE * BD, NL = (NS + 31) / 32, RB = 4;  // sums, sums a lane, rows in flight
+    __shared__ double red[8][NS];
+    const int J = blockIdx.x, l = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const T *Pj = P + (long)l * n * W + jslot[J];
+    double acc[NL];
 #pragma unroll
-        for (int l = 0; l < BD; ++l) {
-            const double p = (double)P[l * nW + (long)i * W + sj];
-            for (int s = 0; s < ncode; ++s)
+    for (int q = 0; q < NL; ++q) acc[q] = 0.0;
+    const int r1 = pt_ptr[J + 1];
+    for (int r0 = pt_ptr[J] + warp; r0 < r1; r0 += 8 * RB) {
+        double v[RB][NL], p[RB];
 #pragma unroll
-                for (int m = 0; m < BD; ++m) acc[(s * BD + l) * BD + m] = fma(p, api[(s * BD + l) * BD + m], acc[(s * BD + l) * BD + m]);
+        for (int b = 0; b < RB; ++b) {
+            const bool on = r0 + 8 * b < r1;
+            const int i = pt_rows[on ? r0 + 8 * b : r0];
+            p[b] = on ? widen(Pj[(long)i * W]) : 0.0;
+#pragma unroll
+            for (int q = 0; q < NL; ++q)
+                v[b][q] = on && lane + 32 * q < NS ? AP[((long)i * BD + l) * NS + lane + 32 * q] : 0.0;
+        }
+#pragma unroll
+        for (int b = 0; b < RB; ++b) {
+            if (r0 + 8 * b >= r1) break;
+#pragma unroll
+            for (int q = 0; q < NL; ++q) acc[q] = fma(p[b], v[b][q], acc[q]);
         }
     }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int q = 0; q < nq; ++q) {
-        double v = warp_sum(acc[q]);
-        if (lane == 0) red[q][warp] = v;
-    }
+#pragma unroll
+    for (int q = 0; q < NL; ++q)
+        if (lane + 32 * q < NS) red[warp][lane + 32 * q] = acc[q];
     __syncthreads();
     // coarse coordinates of J
     const int j0 = J % nb0, j1 = (J / nb0) % nb1, j2 = dim == 3 ? J / (nb0 * nb1) : 0;
-    for (int q = threadIdx.x; q < nq; q += blockDim.x) {
-        const double v = (red[q][0] + red[q][1]) + (red[q][2] + red[q][3]);
-        const int m = q % BD, l = (q / BD) % BD, s = q / (BD * BD);
-        const int r0 = s % 3, r1 = (s / 3) % 3, r2 = s / 9;
-        // the coarse coordinate in {J_d-1, J_d, J_d+1} with residue r_d
-        const int L0 = j0 - 1 + ((r0 - (j0 - 1)) % 3 + 3) % 3;
-        const int L1 = j1 - 1 + ((r1 - (j1 - 1)) % 3 + 3) % 3;
-        const int L2 = dim == 3 ? j2 - 1 + ((r2 - (j2 - 1)) % 3 + 3) % 3 : 0;
+    for (int q = threadIdx.x; q < NS; q += 256) {
+        double v = 0.0;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) v += red[w][q];
+        const int m = q % BD, s = q / BD;
+        const int c0 = s % 3, c1 = (s / 3) % 3, c2 = s / 9;
+        // the coarse coordinate in {J_d-1, J_d, J_d+1} with residue c_d
+        const int L0 = j0 - 1 + ((c0 - (j0 - 1)) % 3 + 3) % 3;
+        const int L1 = j1 - 1 + ((c1 - (j1 - 1)) % 3 + 3) % 3;
+        const int L2 = dim == 3 ? j2 - 1 + ((c2 - (j2 - 1)) % 3 + 3) % 3 : 0;
         const bool in = !(L0 < 0 || L0 >= nb0 || L1 < 0 || L1 >= nb1 || L2 < 0 || L2 >= nb2);
         const int qo = (L0 - j0 + 1) + 3 * (L1 - j1 + 1) + (dim == 3 ? 9 * (L2 - j2 + 1) : 0);
-        Acs[(((long)J * ncode + qo) * BD + l) * BD + m] = in ? v : 0.0;
+        Acs[(((long)J * NCODE + qo) * BD + l) * BD + m] = in ? v : 0.0;
     }
 }
 
-// Scalar operators: the same two passes with the accumulators off local
-// memory. Pass 1 keeps each thread's NCODE sums in a shared-memory column
-// (the code index is data-dependent) and writes the CTA's contiguous block
-// of AP coalesced; pass 2 takes the code count as a compile-time constant so
-// that its sums stay in registers. Same FMA sequence per sum as above.
-constexpr int kAp1Threads = 128;
-
-template <typename T, int NCODE>
-__global__ void __launch_bounds__(kAp1Threads) ap1_kernel(int n, int W, const int32_t *__restrict__ rowptr,
-                                                         const int32_t *__restrict__ colidx,
-                                                         const double *__restrict__ val,
-                                                         const int32_t *__restrict__ p_ids, const T *__restrict__ P,
-                                                         const int8_t *__restrict__ code, double *__restrict__ AP) {
-    __shared__ double s_acc[NCODE][kAp1Threads];
-    const int tx = threadIdx.x, i0 = blockIdx.x * kAp1Threads, i = i0 + tx;
-#pragma unroll
-    for (int q = 0; q < NCODE; ++q) s_acc[q][tx] = 0.0;
-    if (i < n) {
-        for (int e = rowptr[i]; e < rowptr[i + 1]; ++e) {
-            const int k = colidx[e];
-            const double a = val[e];
-            for (int t = 0; t < W; ++t) {
-                const int L = p_ids[(long)k * W + t];
-                if (L < 0) continue;
-                const int sc = code[L];
-                s_acc[sc][tx] = fma(a, (double)P[(long)k * W + t], s_acc[sc][tx]);
-            }
-        }
-    }
-    __syncthreads();
-    const int rows = min(kAp1Threads, n - i0);
-    double *out = AP + (long)i0 * NCODE;
-    for (int idx = tx; idx < rows * NCODE; idx += kAp1Threads) out[idx] = s_acc[idx % NCODE][idx / NCODE];
-}
-
+// Pass 2 for scalar operators, one CTA per coarse node, a thread a row with its NCODE
+// sums in registers, then a fixed-order block reduction.
 template <typename T, int NCODE>
 __global__ void __launch_bounds__(128) ptap1_kernel(int n, int W, int nc, int dim, int nb0, int nb1, int nb2,
                                                     const T *__restrict__ P, const int32_t *__restrict__ pt_ptr,
@@ -225,7 +265,7 @@ __global__ void __launch_bounds__(128) ptap1_kernel(int n, int W, int nc, int di
     for (int r = pt_ptr[J] + threadIdx.x; r < pt_ptr[J + 1]; r += blockDim.x) {
         const int i = pt_rows[r];
         const double *api = AP + (long)i * NCODE;
-        const double p = (double)P[(long)i * W + sj];
+        const double p = widen(P[(long)i * W + sj]);
 #pragma unroll
         for (int q = 0; q < NCODE; ++q) acc[q] = fma(p, api[q], acc[q]);
     }
@@ -271,29 +311,43 @@ msrsb_status galerkin(const msrsb_mat *A, const msrsb_grid *g, int W, int nc, co
     int nb[3];
     coarse_extent(g, nb);
     if (nb[0] * nb[1] * nb[2] != nc) return fail(MSRSB_ESHAPE, "grid implies %d coarse nodes, got %d", nb[0] * nb[1] * nb[2], nc);
-    int8_t *code = nullptr;
+    if (W != 4 && W != 8) return fail(MSRSB_ESHAPE, "%d slots a row", W);
+    uint8_t *code = nullptr;
     double *AP = nullptr;
-    MSRSB_TRY(dalloc(&code, nc, s));
+    MSRSB_TRY(dalloc(&code, (size_t)n * W, s));
     MSRSB_TRY(dalloc(&AP, (size_t)n * ncode * BD * BD, s));
-    coarse_code_kernel<<<ceil_div(nc, 256), 256, 0, s>>>(nc, nb[0], nb[1], dim, code);
+    coarse_code_kernel<<<ceil_div((long)n * W, 256), 256, 0, s>>>((long)n * W, nb[0], nb[1], dim, p_ids, code);
     MSRSB_LAUNCHED("coarse_code_kernel");
+    // rows of P as 16-byte vectors where every component's begin on them
+    const int vec = ((uintptr_t)P & 15) == 0 && ((size_t)W * sizeof(T)) % 16 == 0;
+    auto ap = [&](auto bd, auto nq, auto w) -> msrsb_status {
+        constexpr int B = decltype(bd)::value, Q = decltype(nq)::value, WW = decltype(w)::value;
+        ap_kernel<T, B, Q, WW><<<dim3(ceil_div(n, kApThreads), B), kApThreads, 0, s>>>(
+            n, vec, A->rowptr, A->colidx, A->val, code, P, AP);
+        MSRSB_LAUNCHED("ap_kernel");
+        return MSRSB_OK;
+    };
+    using std::integral_constant;
+    auto aps = [&](auto bd, auto nq) -> msrsb_status {
+        return W == 8 ? ap(bd, nq, integral_constant<int, 8>{}) : ap(bd, nq, integral_constant<int, 4>{});
+    };
     if (BD == 1 && ncode == 27) {
-        ap1_kernel<T, 27><<<ceil_div(n, kAp1Threads), kAp1Threads, 0, s>>>(n, W, A->rowptr, A->colidx, A->val, p_ids,
-                                                                           P, code, AP);
-        MSRSB_LAUNCHED("ap1_kernel");
+        MSRSB_TRY(aps(integral_constant<int, 1>{}, integral_constant<int, 27>{}));
         ptap1_kernel<T, 27><<<nc, 128, 0, s>>>(n, W, nc, dim, nb[0], nb[1], nb[2], Pl, pt_ptr, pt_rows, jslot, AP, Ac);
         MSRSB_LAUNCHED("ptap1_kernel");
     } else if (BD == 1) {
-        ap1_kernel<T, 9><<<ceil_div(n, kAp1Threads), kAp1Threads, 0, s>>>(n, W, A->rowptr, A->colidx, A->val, p_ids,
-                                                                          P, code, AP);
-        MSRSB_LAUNCHED("ap1_kernel");
+        MSRSB_TRY(aps(integral_constant<int, 1>{}, integral_constant<int, 9>{}));
         ptap1_kernel<T, 9><<<nc, 128, 0, s>>>(n, W, nc, dim, nb[0], nb[1], nb[2], Pl, pt_ptr, pt_rows, jslot, AP, Ac);
         MSRSB_LAUNCHED("ptap1_kernel");
+    } else if (ncode == 27) {
+        MSRSB_TRY(aps(integral_constant<int, 3>{}, integral_constant<int, 27>{}));
+        ptap_kernel<T, 3, 27><<<dim3(nc, 3), 256, 0, s>>>(n, W, dim, nb[0], nb[1], nb[2], Pl, pt_ptr, pt_rows, jslot,
+                                                          AP, Ac);
+        MSRSB_LAUNCHED("ptap_kernel");
     } else {
-        ap_kernel<T, 3><<<ceil_div(n, 128), 128, 0, s>>>(n, W, ncode, A->rowptr, A->colidx, A->val, p_ids, P, code, AP);
-        MSRSB_LAUNCHED("ap_kernel");
-        ptap_kernel<T, 3><<<nc, 128, 0, s>>>(n, W, nc, ncode, dim, nb[0], nb[1], nb[2], Pl, pt_ptr, pt_rows, jslot, AP,
-                                            Ac);
+        MSRSB_TRY(aps(integral_constant<int, 3>{}, integral_constant<int, 9>{}));
+        ptap_kernel<T, 3, 9><<<dim3(nc, 3), 256, 0, s>>>(n, W, dim, nb[0], nb[1], nb[2], Pl, pt_ptr, pt_rows, jslot,
+                                                         AP, Ac);
         MSRSB_LAUNCHED("ptap_kernel");
     }
     dfree(code, s);
