@@ -253,6 +253,42 @@ struct IluLines {
 // ---- device helpers -------------------------------------------------------
 __device__ __forceinline__ unsigned long long dbits(double x) { return (unsigned long long)__double_as_longlong(x); }
 
+// FP32 to FP64 and back. The conversion instructions share the narrow FP64 pipe with
+// the FMAs around them (a warp's in 19 cycles of an SM), so values change precision by
+// their bits, with the same results. widen: sign, exponent rebased by 1023 - 127, fraction
+// moved up by 29; subnormals are scaled into the normal range first (exactly, by 2^32),
+// infinities and NaN keep the largest exponent. narrow: round to nearest even; what does
+// not end in FP32's normal range (and is not 0) is converted out of line. A row of
+// A z in double-floats costs 29 FP64 instructions instead of 32 (eight right-hand sides
+// of 80^3: 28.1 -> 27.8 ms a solve).
+__device__ __forceinline__ double widen(double v) { return v; }
+__device__ __forceinline__ double widen(float v) {
+    const unsigned e = __float_as_uint(v) & 0x7f800000u;
+    const unsigned u = __float_as_uint(e == 0u ? v * 4294967296.0f : v), mag = u & 0x7fffffffu;
+    const unsigned base = e == 0u ? 0x38000000u - (32u << 20) : e == 0x7f800000u ? 0x70000000u : 0x38000000u;
+    const unsigned hi = (u & 0x80000000u) | (mag != 0u ? (mag >> 3) + base : 0u);
+    return __hiloint2double((int)hi, (int)(u << 29));
+}
+static __device__ __noinline__ float narrow_rare(double v) { return (float)v; }
+__device__ __forceinline__ float narrow(double v) {
+    const unsigned long long b = dbits(v), mag = b & 0x7fffffffffffffffULL;
+    const unsigned sign = (unsigned)(b >> 32) & 0x80000000u;
+    // magnitudes that round to 2^-126 .. the largest float
+    if (mag != 0 && mag - 0x3810000000000000ULL >= 0x47effffff0000000ULL - 0x3810000000000000ULL) return narrow_rare(v);
+    const unsigned long long t = (mag + 0x0fffffffULL + ((mag >> 29) & 1u)) >> 29;
+    return __uint_as_float(sign | (mag != 0 ? (unsigned)t - 0xc0000000u : 0u));
+}
+template <typename TO>
+__device__ __forceinline__ TO to_prec(float v) {
+    if constexpr (sizeof(TO) == 8) return widen(v);
+    else return v;
+}
+template <typename TO>
+__device__ __forceinline__ TO to_prec(double v) {
+    if constexpr (sizeof(TO) == 8) return v;
+    else return narrow(v);
+}
+
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);

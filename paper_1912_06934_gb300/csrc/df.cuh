@@ -20,8 +20,8 @@ struct DF {
 // is hi + lo with |lo| <= ulp(hi)/2. The _rn intrinsics keep the compiler
 // from contracting the error-free transformations into FMAs.
 __device__ __forceinline__ DF df_from(double x) {
-    float h = (float)x;
-    return DF{h, (float)(x - (double)h)};
+    const float h = narrow(x);
+    return DF{h, narrow(x - widen(h))};
 }
 __device__ __forceinline__ DF quick_two_sum(float a, float b) {  // |a| >= |b|
     const float s = __fadd_rn(a, b);

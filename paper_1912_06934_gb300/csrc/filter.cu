@@ -255,7 +255,7 @@ msrsb_status sell_structure(int n, const int32_t *rowptr, Sell *S, cudaStream_t 
     MSRSB_CUDA(cudaMemsetAsync(flag, 0, sizeof(int32_t), s));
     if (kept) {
         const msrsb_mat *A = kept->A;
-        if (kept->W != 4 && kept->W != 8) return fail(MSRSB_ESHAPE, "%d slots a row", kept->W);
+        if (kept->W != 4 && kept->W != 8) return fail(MSRSB_EINVAL, "W must be 4 or 8 (got %d)", kept->W);
         const bool vec = ((uintptr_t)kept->p_ids & 15) == 0;
         auto kernel = kept->W == 8 ? sell_kept_width_kernel<8> : sell_kept_width_kernel<4>;
         kernel<<<ceil_div((long)S->nslices * kSell, kTileRows), kTileRows, 0, s>>>(
@@ -287,7 +287,7 @@ msrsb_status sell_fill(const msrsb_mat *A, int comp, int raw, double omega, cons
     T *v = nullptr;
     MSRSB_TRY(dalloc(&v, S->entries, s));
     S->val[comp] = v;
-    if (W != 4 && W != 8) return fail(MSRSB_ESHAPE, "%d slots a row", W);
+    if (W != 4 && W != 8) return fail(MSRSB_EINVAL, "W must be 4 or 8 (got %d)", W);
     const bool vec = ((uintptr_t)p_ids & 15) == 0;
     auto kernel = W == 8 ? sell_fill_kernel<T, 8> : sell_fill_kernel<T, 4>;
     kernel<<<ceil_div((long)S->nslices * kSell, kTileRows), kTileRows, 0, s>>>(

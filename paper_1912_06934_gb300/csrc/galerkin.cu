@@ -100,20 +100,6 @@ __global__ void coarse_code_kernel(long nW, int nb0, int nb1, int dim, const int
     code[e] = (uint8_t)c;
 }
 
-// a value in FP64. FP32 to FP64 conversions share the narrow FP64 pipe with the FMAs
-// they feed, so values are widened by their bits: sign, exponent rebased by 1023 - 127,
-// fraction moved up by 29; subnormals are scaled into the normal range first (exactly,
-// by 2^32), infinities and NaN keep the largest exponent. Without a branch, in which a
-// conversion would be issued all the same.
-__device__ __forceinline__ double widen(double v) { return v; }
-__device__ __forceinline__ double widen(float v) {
-    const unsigned e = __float_as_uint(v) & 0x7f800000u;
-    const unsigned u = __float_as_uint(e == 0u ? v * 4294967296.0f : v), mag = u & 0x7fffffffu;
-    const unsigned base = e == 0u ? 0x38000000u - (32u << 20) : e == 0x7f800000u ? 0x70000000u : 0x38000000u;
-    const unsigned hi = (u & 0x80000000u) | (mag != 0u ? (mag >> 3) + base : 0u);
-    return __hiloint2double((int)hi, (int)(u << 29));
-}
-
 // Pass 1, one thread per fine (block) row i and component l (blockIdx.y):
 // AP[i][l][s][m] = sum_k A_ik[l][m] P^m_{k,L} over the coarse nodes L with
 // code s met through row i (FP64, fixed order: A's row order, then slots).
@@ -311,7 +297,7 @@ msrsb_status galerkin(const msrsb_mat *A, const msrsb_grid *g, int W, int nc, co
     int nb[3];
     coarse_extent(g, nb);
     if (nb[0] * nb[1] * nb[2] != nc) return fail(MSRSB_ESHAPE, "grid implies %d coarse nodes, got %d", nb[0] * nb[1] * nb[2], nc);
-    if (W != 4 && W != 8) return fail(MSRSB_ESHAPE, "%d slots a row", W);
+    if (W != 4 && W != 8) return fail(MSRSB_EINVAL, "W must be 4 or 8 (got %d)", W);
     uint8_t *code = nullptr;
     double *AP = nullptr;
     MSRSB_TRY(dalloc(&code, (size_t)n * W, s));

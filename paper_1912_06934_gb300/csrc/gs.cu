@@ -242,11 +242,11 @@ __global__ void __launch_bounds__(kGsThreads, sizeof(T) == 4 ? 7 : 4) gs_sweep_k
         T e = d[3 * l] * b[0] + d[3 * l + 1] * b[1] + d[3 * l + 2] * b[2];
         const long o = 3 * (long)i + l0 + l;
         if (forward) {
-            if (z) z[o] = TZ(e);
+            if (z) z[o] = to_prec<TZ>(e);
         } else {
-            const TZ zn = TZ(zo[l] + TZ(e));
+            const TZ zn = TZ(zo[l] + to_prec<TZ>(e));
             z[o] = zn;
-            e = T(zn);
+            e = to_prec<T>(zn);
         }
         x4[4 * (long)i + l0 + l] = e;
     }

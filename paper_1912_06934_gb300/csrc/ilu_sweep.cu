@@ -331,7 +331,7 @@ __global__ void __launch_bounds__(128 * WPL, 1) lines_sweep_kernel(
                         if (d || mode == 0) ys.p[v0 + c][st + x] = a[c][s];
                         if (d) {
                             TZ *zp = zs.p[v0 + c] + row[s];
-                            *zp = TZ(zv[c][s] + TZ(a[c][s]));
+                            *zp = TZ(zv[c][s] + to_prec<TZ>(a[c][s]));
                         }
                     }
                 }

@@ -35,7 +35,7 @@ __global__ void __launch_bounds__(256) restrict_multi_kernel(int nc, int k, cons
 #pragma unroll
     for (int c = 0; c < kMaxRhs; ++c) {
         if (c >= k) break;
-        const double t = warp_sum((double)acc[c]);
+        const double t = warp_sum(widen(acc[c]));
         if (lane == 0) red[c][warp] = t;
     }
     __syncthreads();
@@ -121,7 +121,7 @@ __global__ void __launch_bounds__(256) prolong_multi_kernel(int n, int k, const 
             if constexpr (sizeof(TP) == 4) sum = fmaf(pv[s], wc32.p[c][ids[s]], sum);
             else sum = fma(pv[s], wc.p[c][ids[s]], sum);
         }
-        z.p[c][i] = TZ(sum);
+        z.p[c][i] = to_prec<TZ>(sum);
         if (z32.p[c]) z32.p[c][i] = float(sum);
     }
 }
