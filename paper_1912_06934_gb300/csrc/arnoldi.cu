@@ -24,6 +24,7 @@
 
 namespace msrsb {
 
+static_assert(kArnBlocks % 4 == 0, "the step's scalars sum the chunks in four fixed quarters");
 
 // ---- pass 1: dot products ------------------------------------------------------------------
 
@@ -156,24 +157,14 @@ __global__ void __launch_bounds__(256) dcgs2_dots_kernel(long N, int nv, long ld
 // ---- the step's scalars (one CTA a right-hand side) ----------------------------------------------------------
 //
 // Sums the dot products' row-chunk partials (d = (s_0, t_0, s_1, t_1, ...,
-// rho, sigma), in a fixed order) and finishes column j-1 of
+// rho, sigma), one warp per product, fixed order) and finishes column j-1 of
 // Hu (+= s, Hu[j][j-1] = alpha), copied to H for the Givens rotation; with
 // `full` (what given) also R[:, j] = (s, alpha), the provisional column j of Hu
 // (V_j^T w_j) and the update coefficients cv = s / alpha (for v_j),
 // cp = H s / alpha + Hu[:, j] (for the next p), scal[0] = 1 / alpha.
-//
-// A chain of short FP64 steps, so each is spread wide or done once: eight lanes a
-// product with two sums each; one warp forms alpha and 1 / alpha (in every thread, the
-// square root and the division kept the FP64 pipe busy for longer than the rest) from
-// one reciprocal square root with a correction each; the finished columns of Hu come to
-// shared memory beside the partials where they fit. Up to 30 columns: 8.3 us a step, now 6.5.
-constexpr int kScalThreads = 512, kScalLanes = 8;
-constexpr int kScalStage = 48;  // columns of Hu staged
-
 template <typename T>
-__global__ void __launch_bounds__(kScalThreads) dcgs2_scalar_kernel(int m, int j,
-                                                                    const __grid_constant__ ArnBatch<T> B,
-                                                                    long pstride, const double *__restrict__ partial) {
+__global__ void __launch_bounds__(256) dcgs2_scalar_kernel(int m, int j, const __grid_constant__ ArnBatch<T> B,
+                                                           long pstride, const double *__restrict__ partial) {
     double *__restrict__ kh = B.r[blockIdx.x].kh;
     const bool full = B.r[blockIdx.x].Wh != nullptr;
     partial += blockIdx.x * pstride;
@@ -181,40 +172,23 @@ __global__ void __launch_bounds__(kScalThreads) dcgs2_scalar_kernel(int m, int j
     const KhLayout L(m);
     double *H = kh + L.H, *Hu = kh + L.Hu, *R = kh + L.R;
     double *cv = kh + L.cv, *cp = kh + L.cp, *sc = kh + L.scal;
-    __shared__ double s_d[2 * 513], s_hs[513], s_hu[kScalStage * (kScalStage + 1)];
-    __shared__ double s_st, s_alpha, s_inva;
-    const int tid = threadIdx.x, ld = j + 1;
-    const bool staged = full && j <= kScalStage;
-    if (staged)
-        for (int t = tid; t < j * ld; t += kScalThreads) {  // Hu[r][c], r <= c + 1
-            const int c = t / ld, r = t - c * ld;
-            if (r <= c + 1) cp_async8(s_hu + t, Hu + (long)c * (m + 1) + r);
-        }
-    cp_async_commit();
-    {
-        constexpr int kEach = (kArnBlocks + kScalLanes - 1) / kScalLanes;
-        const int sub = tid & (kScalLanes - 1), nrows = 2 * (j + 1);
-        for (int row0 = 0; row0 < nrows; row0 += kScalThreads / kScalLanes) {
-            const int row = row0 + tid / kScalLanes;
-            double v[kEach];
+    __shared__ double s_d[2 * 513], s_hs[513];
+    __shared__ double s_ss, s_st;
+    const int tid = threadIdx.x;
+    {  // four lanes per product, each a fixed quarter of the chunks, loads issued together
+        const int sub = tid & 3, nrows = 2 * (j + 1);
+        for (int row0 = 0; row0 < nrows; row0 += 64) {
+            const int row = row0 + (tid >> 2);
+            double a = 0.0;
+            if (row < nrows) {
 #pragma unroll
-            for (int k = 0; k < kEach; ++k)
-                v[k] = row < nrows && sub + kScalLanes * k < kArnBlocks
-                           ? partial[(long)row * kArnBlocks + sub + kScalLanes * k]
-                           : 0.0;
-            double a = v[0], b = kEach > 1 ? v[1] : 0.0;
-#pragma unroll
-            for (int k = 2; k < kEach; ++k) {
-                if (k & 1) b += v[k];
-                else a += v[k];
+                for (int k = 0; k < kArnBlocks / 4; ++k) a += partial[(long)row * kArnBlocks + sub + 4 * k];
             }
-            a += b;
-#pragma unroll
-            for (int o = kScalLanes / 2; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+            a += __shfl_xor_sync(0xffffffffu, a, 1);
+            a += __shfl_xor_sync(0xffffffffu, a, 2);
             if (sub == 0 && row < nrows) s_d[row] = a;
         }
     }
-    cp_async_wait<0>();
     __syncthreads();
     const double *s_s = s_d;  // s_q = s_d[2q], t_q = s_d[2q + 1]
     if (tid < 32) {
@@ -225,63 +199,51 @@ __global__ void __launch_bounds__(kScalThreads) dcgs2_scalar_kernel(int m, int j
         }
         a = warp_sum(a);
         b = warp_sum(b);
-        double alpha = 1.0, inva = 1.0;  // v_0 is a unit vector already
-        if (j > 0) {
-            const double a2 = s_d[2 * j] - a;
-            if (a2 > 1e-290 && a2 < 1e290) {
-                const double y = rsqrt(a2), r = a2 * y;
-                alpha = fma(fma(-r, r, a2), 0.5 * y, r);
-                inva = fma(fma(-alpha, y, 1.0), y, y);
-            } else {
-                alpha = a2 > 0.0 ? sqrt(a2) : 0.0;  // 0: breakdown, the Krylov space is invariant
-                inva = alpha > 0.0 ? 1.0 / alpha : 0.0;
-            }
-        }
         if (tid == 0) {
+            s_ss = a;
             s_st = b;
-            s_alpha = alpha;
-            s_inva = inva;
         }
     }
     __syncthreads();
-    const double alpha = s_alpha, inva = s_inva;
+    const double rho = s_d[2 * j], sig = s_d[2 * j + 1];
+    double alpha = 1.0;  // v_0 is a unit vector already
     if (j > 0) {
+        const double a2 = rho - s_ss;
+        alpha = a2 > 0.0 ? sqrt(a2) : 0.0;  // 0: breakdown, the Krylov space is invariant
         double *hu = Hu + (long)(j - 1) * (m + 1), *hc = H + (long)(j - 1) * (m + 1);
-        for (int q = tid; q <= j; q += kScalThreads) {
-            const double v = q < j ? (staged ? s_hu[(j - 1) * ld + q] : hu[q]) + s_s[2 * q] : alpha;
+        for (int q = tid; q <= j; q += blockDim.x) {
+            const double v = q < j ? hu[q] + s_s[2 * q] : alpha;
             hu[q] = v;
             hc[q] = v;
-            if (staged) s_hu[(j - 1) * ld + q] = v;
         }
     }
     if (!full) return;
+    const double inva = alpha > 0.0 ? 1.0 / alpha : 0.0;
     double *rc = R + (long)j * m;
-    for (int q = tid; q <= j; q += kScalThreads) rc[q] = q < j ? s_s[2 * q] : alpha;
+    for (int q = tid; q <= j; q += blockDim.x) rc[q] = q < j ? s_s[2 * q] : alpha;
     __syncthreads();  // column j-1 of Hu is complete
     // H s over the finished columns 0 .. j-1 (Hu[r][c] != 0 only for r <= c + 1),
-    // eight independent sums per thread
-    const double *T0 = staged ? s_hu : Hu;
-    const long ldt = staged ? ld : m + 1;
-    for (int r = tid; r <= j; r += kScalThreads) {
+    // eight independent loads in flight per thread
+    for (int r = tid; r <= j; r += blockDim.x) {
         double acc[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
         int c = r > 0 ? r - 1 : 0;
         for (; c + 8 <= j; c += 8) {
 #pragma unroll
-            for (int u = 0; u < 8; ++u) acc[u] = fma(T0[(long)(c + u) * ldt + r], s_s[2 * (c + u)], acc[u]);
+            for (int u = 0; u < 8; ++u) acc[u] = fma(Hu[(long)(c + u) * (m + 1) + r], s_s[2 * (c + u)], acc[u]);
         }
-        for (; c < j; ++c) acc[0] = fma(T0[(long)c * ldt + r], s_s[2 * c], acc[0]);
+        for (; c < j; ++c) acc[0] = fma(Hu[(long)c * (m + 1) + r], s_s[2 * c], acc[0]);
         s_hs[r] = ((acc[0] + acc[1]) + (acc[2] + acc[3])) + ((acc[4] + acc[5]) + (acc[6] + acc[7]));
     }
     __syncthreads();
     double *hn = Hu + (long)j * (m + 1);
-    for (int q = tid; q < j; q += kScalThreads) {
+    for (int q = tid; q < j; q += blockDim.x) {
         const double h = (s_d[2 * q + 1] - s_hs[q]) * inva;
         hn[q] = h;
         cp[q] = fma(s_hs[q], inva, h);
         cv[q] = s_d[2 * q] * inva;
     }
     if (tid == 0) {
-        const double h = ((s_d[2 * j + 1] - s_st) * inva - s_hs[j]) * inva;
+        const double h = ((sig - s_st) * inva - s_hs[j]) * inva;
         hn[j] = h;
         cp[j] = fma(s_hs[j], inva, h);
         sc[0] = inva;
@@ -419,7 +381,7 @@ msrsb_status arnoldi_step(long N, int j, int m, int k, const ArnBatch<float> &B,
         MSRSB_PDL((dcgs2_dots_df_kernel<4>), gd, 256, 0, s, NW, j, N, B, ps, partial);
     else
         MSRSB_PDL((dcgs2_dots_df_kernel<1>), gd, 256, 0, s, NW, j, N, B, ps, partial);
-    MSRSB_PDL((dcgs2_scalar_kernel<float>), k, kScalThreads, 0, s, m, j, B, ps, (const double *)partial);
+    MSRSB_PDL((dcgs2_scalar_kernel<float>), k, 256, 0, s, m, j, B, ps, (const double *)partial);
     bool any = false;
     for (int c = 0; c < k; ++c) any = any || B.r[c].Wh;
     if (!any) return MSRSB_OK;
@@ -436,7 +398,7 @@ msrsb_status arnoldi_step(long N, int j, int m, int k, const ArnBatch<double> &B
     const long ps = (long)arn_partial(m);
     MSRSB_PDL((dcgs2_dots_kernel), dim3(kArnBlocks, j + 1, k), 256, 0, s, N, j, N, B, ps,
               partial);
-    MSRSB_PDL((dcgs2_scalar_kernel<double>), k, kScalThreads, 0, s, m, j, B, ps, (const double *)partial);
+    MSRSB_PDL((dcgs2_scalar_kernel<double>), k, 256, 0, s, m, j, B, ps, (const double *)partial);
     bool any = false;
     for (int c = 0; c < k; ++c) any = any || B.r[c].Wh;
     if (!any) return MSRSB_OK;

@@ -337,7 +337,7 @@ template <typename T>
 struct ArnBatch {
     ArnRhs<T> r[kMaxRhs];
 };
-constexpr int kArnBlocks = 76;  // row chunks of the dot products (fixed reduction order)
+constexpr int kArnBlocks = 76;  // row chunks of the dot products (fixed reduction order; a multiple of 4)
 // partials of one right-hand side's step
 inline size_t arn_partial(int m) { return 2 * (size_t)(m + 1) * kArnBlocks; }
 
