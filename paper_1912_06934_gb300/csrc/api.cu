@@ -158,6 +158,7 @@ template <typename TP, typename TZ>
 msrsb_status prolong_op(const msrsb_handle *h, const TP *P, const double *wc, const float *wc32, TZ *z, float *z32,
                         TP *x4, int add, cudaStream_t s);
 msrsb_status norm2(long N, const double *w, double *partial, double *out, cudaStream_t s);
+msrsb_status norm2_mixed(long N, const double *w, double *partial, double *out, cudaStream_t s);
 template <typename TZ>
 msrsb_status mvadd(long N, int nvec, const TZ *Z, long ldz, const double *y, double *x, cudaStream_t s);
 msrsb_status df_scale(long N, const double *r, const double *beta, float *vh, float *vl, cudaStream_t s);
@@ -840,7 +841,7 @@ static msrsb_status gmres_t(msrsb_handle *h, const double *b, double *x, double 
     // double-float basis and work vector of the mixed form: [Vh | Vl | Wh | Wl]
     float *Vh = (float *)h->kv32, *Vl = Vh + (m + 1) * N, *Wh = Vl + (m + 1) * N, *Wl = Wh + N;
     double bnorm = 0.0;
-    MSRSB_TRY(norm2(N, b, h->partial, beta, s));
+    MSRSB_TRY((DFV ? norm2_mixed : norm2)(N, b, h->partial, beta, s));
     MSRSB_TRY(read_scalar(beta, &bnorm, s));
     int its = 0;
     if (hist) hist[0] = 1.0;
@@ -853,7 +854,7 @@ static msrsb_status gmres_t(msrsb_handle *h, const double *b, double *x, double 
     for (;;) {
         // r = b - A x (FP64), beta = |r|, V_0 = r / beta
         MSRSB_TRY(fine_spmv(h, x, b, h->tmp_d, true, s));
-        MSRSB_TRY(norm2(N, h->tmp_d, h->partial, beta, s));
+        MSRSB_TRY((DFV ? norm2_mixed : norm2)(N, h->tmp_d, h->partial, beta, s));
         double bt = 0.0;
         MSRSB_TRY(read_scalar(beta, &bt, s));
         if (!std::isfinite(bt)) return fail(MSRSB_ENAN, "non-finite residual in GMRES");
@@ -1119,7 +1120,7 @@ static msrsb_status gmres_multi_t(msrsb_handle *h, int k, const double *B, doubl
     for (int r = 0; r < k; ++r) {
         iters[r] = 0;
         relres[r] = 0.0;
-        MSRSB_TRY(norm2(N, B + r * N, h->partial, KH[r] + L.beta, s));
+        MSRSB_TRY((DFV ? norm2_mixed : norm2)(N, B + r * N, h->partial, KH[r] + L.beta, s));
         MSRSB_TRY(read_scalar(KH[r] + L.beta, &bnorm[r], s));
         if (bnorm[r] == 0.0) {
             MSRSB_CUDA(cudaMemsetAsync(X + r * N, 0, N * sizeof(double), s));
@@ -1134,7 +1135,7 @@ static msrsb_status gmres_multi_t(msrsb_handle *h, int k, const double *B, doubl
             if (done[r]) continue;
             double *beta = KH[r] + L.beta;
             MSRSB_TRY(fine_spmv(h, X + r * N, B + r * N, h->tmp_d, true, s));
-            MSRSB_TRY(norm2(N, h->tmp_d, h->partial, beta, s));
+            MSRSB_TRY((DFV ? norm2_mixed : norm2)(N, h->tmp_d, h->partial, beta, s));
             double bt = 0.0;
             MSRSB_TRY(read_scalar(beta, &bt, s));
             if (!std::isfinite(bt)) return fail(MSRSB_ENAN, "non-finite residual in GMRES (right-hand side %d)", r);
