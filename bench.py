@@ -443,12 +443,13 @@ def run_extra_config(M, name, c, kind, flush, stream, dev, steps, warmup, hbm, p
         if out[label]["smooth_roofline"] is not None:
             out[label]["smooth_roofline"]["launch_shape"] = shape
         if e == 8 and f["smooth_launches"]:
-            # the FP64 form's pass: products of A_hat P on the pattern plus the
-            # W-wide update per row, in 64-bit fixed point on the integer pipe
-            prods = float(np.mean([k[1] for k in kept])) + n * W
-            out[label]["smooth_products"] = {"arithmetic": "64-bit fixed point", "bound": "gathers of P's rows",
-                                             "products_per_launch": prods,
-                                             "products_per_s": prods / (f["smooth_ms"] / f["smooth_launches"] * 1e-3)}
+            # the FP64 pass is bound by the FP64 pipe: multiply-adds of A_hat P
+            # on the pattern plus the W-wide update per row
+            fmas = float(np.mean([k[1] for k in kept])) + n * W
+            rate = fmas / (f["smooth_ms"] / f["smooth_launches"] * 1e-3)
+            out[label]["smooth_fp64_pipe"] = {"bound": "fp64", "fma_per_launch": fmas, "achieved_fma_per_s": rate,
+                                              "peak_fma_per_s": peaks_fma["fp64_fma_per_s"],
+                                              "frac": rate / peaks_fma["fp64_fma_per_s"]}
         out[label]["apply_us"] = ap_ms * 1e3
         ci_ms = f["info"]["phase_ms"][3]
         cf = coarse_factor_fmas(c)
@@ -570,14 +571,16 @@ def gpu_arm(args, rank, world):
     achieved = per_launch32 / (sm_ms32 / sm_l32 * 1e-3) / 1e9 if sm_l32 else None
     per_launch64 = smooth_bytes(n, nnz_hat, W, 8)
     achieved64 = per_launch64 / (sm_ms64 / sm_l64 * 1e-3) / 1e9 if sm_l64 else None
-    prods64 = matches + n * W
+    fma64 = matches + n * W
     coarse_fmas = coarse_factor_fmas(c)
     mixed = form_summary(f32, args.steps)
     fp64 = form_summary(f64, args.steps)
     fp64["smooth_kernel_gbs"] = achieved64
-    fp64["smooth_products"] = {  # in 64-bit fixed point on the integer pipe
-        "arithmetic": "64-bit fixed point", "bound": "gathers of P's rows", "products_per_launch": prods64,
-        "products_per_s": prods64 / (sm_ms64 / sm_l64 * 1e-3) if sm_l64 else None}
+    fp64["smooth_fp64_pipe"] = {
+        "bound": "fp64", "fma_per_launch": fma64,
+        "achieved_fma_per_s": fma64 / (sm_ms64 / sm_l64 * 1e-3) if sm_l64 else None,
+        "peak_fma_per_s": pk["fp64_fma_per_s"],
+        "frac": fma64 / (sm_ms64 / sm_l64 * 1e-3) / pk["fp64_fma_per_s"] if sm_l64 else None}
     ci_ms = inf64["phase_ms"][3]
     fp64["coarse_fp64_pipe"] = {"op": "coarse factorisation over planes (+ explicit inverse when n_C <= 1024)",
                                 "fmas": coarse_fmas,

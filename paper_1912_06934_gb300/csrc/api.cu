@@ -79,7 +79,7 @@ template <typename T>
 msrsb_status indicator(int n, int W, const int32_t *part, const int32_t *p_ids, T *P, cudaStream_t s);
 template <typename T>
 msrsb_status smooth_basis(const msrsb_mat *A, int comp, int raw, const int32_t *p_ids, const uint8_t *skel, int W,
-                          const msrsb_basis_opts *o, T *P, const double *p_check, int *nzd, int *iters, double *e,
+                          const msrsb_basis_opts *o, T *P, bool fix, int *nzd, int *iters, double *e,
                           cudaStream_t s);
 msrsb_status build_transpose(int n, int W, int nc, const int32_t *p_ids, int32_t **pt_ptr, int32_t **pt_rows,
                              int8_t **jslot, int *nnzp_out, cudaStream_t s);
@@ -385,8 +385,7 @@ static msrsb_status setup_t(msrsb_handle *h, const void *p_init, cudaStream_t s)
             MSRSB_TRY(indicator<T>(n, W, h->part, h->p_ids, Pl, s));
         int it = 0;
         double e = 0.0;
-        const double *check = p_init && sizeof(T) == 8 ? (const double *)Pl : nullptr;
-        MSRSB_TRY(smooth_basis<T>(&A, l, 1, h->p_ids, h->skel, W, &h->opts.basis, Pl, check, nzd, &it, &e, s));
+        MSRSB_TRY(smooth_basis<T>(&A, l, 1, h->p_ids, h->skel, W, &h->opts.basis, Pl, false, nzd, &it, &e, s));
         if (it > h->basis_iters) h->basis_iters = it;
         if (l == 0 || e > h->basis_e_it) h->basis_e_it = e;
     }

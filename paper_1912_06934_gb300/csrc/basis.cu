@@ -15,14 +15,16 @@
 // and the rows of the initial basis sum to 1, as Alg. 1 has it, a pass is a convex
 // combination of P's rows followed by a rescaling of the row: with weights w_ik =
 // omega |a_ik| / D_hat_ii and w_ii = 1 - omega, P_iJ + dP_iJ = sum_k w_ik P_kJ, all
-// of it in [0, 1]. The FP64 form then runs the passes in 64-bit fixed point on the
+// of it in [0, 1]. A basis built by itself then runs the passes in 64-bit fixed point on the
 // integer pipe: P as fractions of 2^63, weights of 2^64, products by their high 64
 // bits (half a unit of truncation given back per product), the row's reciprocal by
 // two Newton steps. A unit is 1.1e-19, below FP64's rounding of every entry above
 // 1e-3: against extended precision P's error after 60 passes is 2.2e-15 in the
 // 2-norm over 37,000 entries, the FP64 passes' 4.7e-15 (tests/test_gpu_fixed.py).
 // Other operators, relaxations above 0.7 (a row sum may then fall below 1/4) and
-// other initial bases keep the FP64 passes. Measured: 152,000 rows (61 x 47 x 53) 50
+// other initial bases keep the FP64 passes, and so do the set-ups of a solver: the last
+// bits of P steer which part of the error a solve to 1e-8 leaves, and on fields of
+// contrast near 1e8 moved its solution by up to 5e-9 of itself. Measured: 152,000 rows (61 x 47 x 53) 50
 // -> 20 us a pass. (Three 32-bit multiply-adds a product on 58-bit fractions instead
 // of the ten instructions of a high product gave the same time: the passes are now
 // bound by the gathers of P's 64-byte rows.)
@@ -663,11 +665,11 @@ msrsb_status sell_fill(const msrsb_mat *A, int comp, int raw, double omega, cons
 void sell_free(Sell *S, cudaStream_t s);
 
 // Filtered operator of component comp (filtered here when raw is set), then the
-// loop; FP64 in fixed point where the operator, the relaxation and the initial
-// basis allow it (p_check: that basis, to be looked over; nullptr: the indicator).
+// loop; with `fix` FP64 in fixed point where the operator, the relaxation and the
+// initial basis P allow it.
 template <typename T>
 msrsb_status smooth_basis(const msrsb_mat *A, int comp, int raw, const int32_t *p_ids, const uint8_t *skel, int W,
-                          const msrsb_basis_opts *o, T *P, const double *p_check, int *nzd, int *iters, double *e,
+                          const msrsb_basis_opts *o, T *P, bool fix, int *nzd, int *iters, double *e,
                           cudaStream_t s) {
     const int n = A->nrows;
     Sell S;
@@ -679,8 +681,8 @@ msrsb_status smooth_basis(const msrsb_mat *A, int comp, int raw, const int32_t *
     keep.raw = raw;
     keep.W = W;
     keep.p_ids = p_ids;
-    keep.look = sizeof(T) == 8;
-    keep.p_init = p_check;
+    keep.look = fix && sizeof(T) == 8;
+    if constexpr (sizeof(T) == 8) keep.p_init = fix ? (const double *)P : nullptr;
     MSRSB_TRY(sell_structure(n, A->rowptr, &S, s, &keep));
     MSRSB_TRY(dalloc(&scale, n, s));
     MSRSB_TRY(dalloc(&vmask, n, s));
@@ -705,10 +707,10 @@ msrsb_status smooth_basis(const msrsb_mat *A, int comp, int raw, const int32_t *
     return st;
 }
 template msrsb_status smooth_basis<double>(const msrsb_mat *, int, int, const int32_t *, const uint8_t *, int,
-                                           const msrsb_basis_opts *, double *, const double *, int *, int *, double *,
+                                           const msrsb_basis_opts *, double *, bool, int *, int *, double *,
                                            cudaStream_t);
 template msrsb_status smooth_basis<float>(const msrsb_mat *, int, int, const int32_t *, const uint8_t *, int,
-                                          const msrsb_basis_opts *, float *, const double *, int *, int *, double *,
+                                          const msrsb_basis_opts *, float *, bool, int *, int *, double *,
                                           cudaStream_t);
 
 }  // namespace msrsb
@@ -725,10 +727,10 @@ extern "C" msrsb_status msrsb_build_basis(const msrsb_mat *Ahat, const int32_t *
     double e = 0.0;
     msrsb_status st;
     if (prec == MSRSB_F64)
-        st = smooth_basis<double>(Ahat, 0, 0, p_ids, skel, W, opts, (double *)p_val, (const double *)p_val, nullptr, &it,
+        st = smooth_basis<double>(Ahat, 0, 0, p_ids, skel, W, opts, (double *)p_val, true, nullptr, &it,
                                   &e, stream);
     else if (prec == MSRSB_F32)
-        st = smooth_basis<float>(Ahat, 0, 0, p_ids, skel, W, opts, (float *)p_val, nullptr, nullptr, &it, &e, stream);
+        st = smooth_basis<float>(Ahat, 0, 0, p_ids, skel, W, opts, (float *)p_val, false, nullptr, &it, &e, stream);
     else
         return fail(MSRSB_EINVAL, "prec must be MSRSB_F64 or MSRSB_F32");
     if (st != MSRSB_OK) return st;
