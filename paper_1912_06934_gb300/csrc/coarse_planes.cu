@@ -99,9 +99,6 @@ constexpr int kPlaneMaxCluster = 16;
 constexpr int kFactorThreads = kPlaneThreads + 32;  // a warp of its own for the pivot's reciprocal
 
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
-__device__ __forceinline__ void cluster_arrive_relaxed() {
-    asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory");
-}
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
 // shared-memory address of p in CTA `rank` of the cluster
 __device__ __forceinline__ unsigned map_rank(const void *p, int rank) {
@@ -371,8 +368,9 @@ __global__ void __launch_bounds__(kFactorThreads, 1) plane_factor_kernel(PlaneGe
                 }
                 publish(kk + 1, jl, v);
             }
-            if (next) cluster_arrive();
-            else if (kk + 1 < m) cluster_arrive_relaxed();  // nothing written for another CTA, reads consumed
+            // releases the owner's stores, and every thread's reads of step kk - 1 before another
+            // CTA's store into that buffer two barriers on
+            if (kk + 1 < m) cluster_arrive();
             if (!worker) {
                 if (lane == 0 && p != kk) {
                     const int t = pil[kk];
