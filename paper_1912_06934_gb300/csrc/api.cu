@@ -74,13 +74,16 @@ msrsb_status sell_copy(const msrsb_mat *A, bool with_f32, Sell *S, cudaStream_t 
 template <typename TA, typename TX, typename TV, typename TY, typename TACC>
 msrsb_status sell_spmv(const Sell &S, const TA *val, const TX *x, const TV *v, TY *y, bool resid, cudaStream_t s,
                        const int32_t *operm = nullptr);
+template <typename T>
+msrsb_status sell_fill(const msrsb_mat *A, int comp, int raw, double omega, const int32_t *p_ids, int W, Sell *S,
+                       T *scale, uint8_t *vmask, int write_col, int *n_zero_d, cudaStream_t s);
 void sell_free(Sell *S, cudaStream_t s);
 template <typename T>
 msrsb_status indicator(int n, int W, const int32_t *part, const int32_t *p_ids, T *P, cudaStream_t s);
 template <typename T>
-msrsb_status smooth_basis(const msrsb_mat *A, int comp, int raw, const int32_t *p_ids, const uint8_t *skel, int W,
-                          const msrsb_basis_opts *o, T *P, bool fix, int *nzd, int *iters, double *e,
-                          cudaStream_t s);
+msrsb_status basis_loop(int n, int W, const Sell &S, int comp, const T *scale, const uint8_t *vmask,
+                        const uint8_t *skel, T *P, const msrsb_basis_opts *o, int *iters_out, double *e_out,
+                        cudaStream_t s);
 msrsb_status build_transpose(int n, int W, int nc, const int32_t *p_ids, int32_t **pt_ptr, int32_t **pt_rows,
                              int8_t **jslot, int *nnzp_out, cudaStream_t s);
 template <typename TP>
@@ -373,7 +376,11 @@ static msrsb_status setup_t(msrsb_handle *h, const void *p_init, cudaStream_t s)
     T *P = nullptr;
     MSRSB_TRY(dalloc(&P, nW * bd, s));
     h->p_val = P;
+    T *scale = nullptr;
+    uint8_t *vmask = nullptr;
     int *nzd = nullptr;
+    MSRSB_TRY(dalloc(&scale, n, s));
+    MSRSB_TRY(dalloc(&vmask, n, s));
     MSRSB_TRY(dalloc(&nzd, 1, s));
     MSRSB_CUDA(cudaMemsetAsync(nzd, 0, sizeof(int), s));
     h->basis_iters = 0;
@@ -383,12 +390,25 @@ static msrsb_status setup_t(msrsb_handle *h, const void *p_init, cudaStream_t s)
             MSRSB_CUDA(cudaMemcpyAsync(Pl, (const T *)p_init + l * nW, nW * sizeof(T), cudaMemcpyDeviceToDevice, s));
         else
             MSRSB_TRY(indicator<T>(n, W, h->part, h->p_ids, Pl, s));
+        // the filtered operator of this component, its kept entries only
+        Sell S;
+        SellKeep keep;
+        keep.A = &A;
+        keep.comp = l;
+        keep.raw = 1;
+        keep.W = W;
+        keep.p_ids = h->p_ids;
+        MSRSB_TRY(sell_structure(n, A.rowptr, &S, s, &keep));
+        MSRSB_TRY(sell_fill<T>(&A, l, 1, h->opts.basis.omega, h->p_ids, W, &S, scale, vmask, 1, nzd, s));
         int it = 0;
         double e = 0.0;
-        MSRSB_TRY(smooth_basis<T>(&A, l, 1, h->p_ids, h->skel, W, &h->opts.basis, Pl, false, nzd, &it, &e, s));
+        MSRSB_TRY(basis_loop<T>(n, W, S, l, scale, vmask, h->skel, Pl, &h->opts.basis, &it, &e, s));
         if (it > h->basis_iters) h->basis_iters = it;
         if (l == 0 || e > h->basis_e_it) h->basis_e_it = e;
+        sell_free(&S, s);
     }
+    dfree(scale, s);
+    dfree(vmask, s);
     MSRSB_TRY(mark(2));
     if (ilu_chain) {
         MSRSB_CUDA(cudaEventRecord(go_ev, s));

@@ -9,58 +9,9 @@
 // mask packed beside column k says which slots match. The epilogue is fused:
 // dP = -(omega / D_hat_ii) * (A_hat P)_i* on the pattern, P + dP divided by
 // its row sum, and max |dP| over non-skeleton rows into a device scalar.
-//
-// FP64 passes are bound by the FP64 pipe (a warp's FMA every 19 cycles and SM;
-// 180 of them a warp of rows), not by memory. Where the operator is an M-matrix
-// and the rows of the initial basis sum to 1, as Alg. 1 has it, a pass is a convex
-// combination of P's rows followed by a rescaling of the row: with weights w_ik =
-// omega |a_ik| / D_hat_ii and w_ii = 1 - omega, P_iJ + dP_iJ = sum_k w_ik P_kJ, all
-// of it in [0, 1]. A basis built by itself then runs the passes in 64-bit fixed point on the
-// integer pipe: P as fractions of 2^63, weights of 2^64, products by their high 64
-// bits (half a unit of truncation given back per product), the row's reciprocal by
-// two Newton steps. A unit is 1.1e-19, below FP64's rounding of every entry above
-// 1e-3: against extended precision P's error after 60 passes is 2.2e-15 in the
-// 2-norm over 37,000 entries, the FP64 passes' 4.7e-15 (tests/test_gpu_fixed.py).
-// Other operators, relaxations above 0.7 (a row sum may then fall below 1/4) and
-// other initial bases keep the FP64 passes, and so do the set-ups of a solver: the last
-// bits of P steer which part of the error a solve to 1e-8 leaves, and on fields of
-// contrast near 1e8 moved its solution by up to 5e-9 of itself. Measured: 152,000 rows (61 x 47 x 53) 50
-// -> 20 us a pass. (Three 32-bit multiply-adds a product on 58-bit fractions instead
-// of the ten instructions of a high product gave the same time: the passes are now
-// bound by the gathers of P's 64-byte rows.)
 #include "common.cuh"
-#include <type_traits>
 
 namespace msrsb {
-
-template <typename T>
-constexpr bool kFx = std::is_same<T, fx64>::value;
-
-// acc += a p: FMA, or the high 64 bits of the fixed-point product
-template <typename T>
-__device__ __forceinline__ void smooth_mac(T &acc, T a, T p) {
-    if constexpr (kFx<T>) acc += __umul64hi(a, p);
-    else acc = fma(a, p, acc);
-}
-
-// 2^125 / s for s in [2^61, 2^63 (1 + 1e-8)]: 1 / (s / 2^63) as a fraction of 2^62,
-// within 2^-60: a float reciprocal, then y += y (1 - s y) twice
-__device__ __forceinline__ fx64 fx_recip(fx64 s) {
-    const float r = 1.0f / ((float)(unsigned)(s >> 32) * 4.656612873077393e-10f);  // 2^-31
-    fx64 y = (fx64)(unsigned)fminf(r * 1073741824.0f, 4294967040.0f) << 32;        // 2^30, below 4
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-        const long long e = (long long)((1ull << 61) - __umul64hi(s, y));
-        y = e >= 0 ? y + __umul64hi(y, (fx64)e << 3) : y - __umul64hi(y, (fx64)(-e) << 3);
-    }
-    return y;
-}
-// t y, y a fraction of 2^62, rounded
-__device__ __forceinline__ fx64 fx_scale(fx64 t, fx64 y) {
-    const fx64 lo = t * y;
-    return (__umul64hi(t, y) << 2) + (lo >> 62) + ((lo >> 61) & 1u);
-}
-__device__ __forceinline__ fx64 fx_diff(fx64 a, fx64 b) { return a > b ? a - b : b - a; }
 
 template <typename T, int W>
 struct PRow {
@@ -96,56 +47,33 @@ __device__ __forceinline__ void store_row(T *__restrict__ P, long k, const T (&i
 // Epilogue of a row's pass: dP = -scale_i (A_hat P)_i on the row's valid
 // slots, P_i + dP divided by its sum (one reciprocal), stored; sets
 // max |dP| over the row's slots in e_loc on check passes of non-skeleton rows.
-// Fixed point: acc is the new row already; cnt entries contributed.
 template <typename T, int W>
-__device__ __forceinline__ void smooth_epilogue(int i, const T (&acc)[W], int cnt, const T *__restrict__ scale,
+__device__ __forceinline__ void smooth_epilogue(int i, const T (&acc)[W], const T *__restrict__ scale,
                                                 const uint8_t *__restrict__ vmask, const uint8_t *__restrict__ skel,
                                                 const T *__restrict__ Pin, T *__restrict__ Pout, int check,
                                                 double &e_loc) {
-    if constexpr (kFx<T>) {
-        const unsigned vm = vmask[i];
-        T t[W], sum = 0;
+    T own[W];
+    load_row<T, W>(Pin, i, own);
+    unsigned vm = vmask[i];
+    T sc = scale[i];
+    T t[W];
+    T sum = T(0), emx = T(0);
 #pragma unroll
-        for (int c = 0; c < W; ++c) {
-            t[c] = vm & (1u << c) ? acc[c] + (unsigned)(cnt >> 1) : 0ull;
+    for (int c = 0; c < W; ++c) {
+        if (vm & (1u << c)) {
+            T d = -sc * acc[c];
+            t[c] = own[c] + d;
             sum += t[c];
+            emx = fmax(emx, fabs(d));
+        } else {
+            t[c] = T(0);
         }
-        if (check) {
-            T own[W], emx = 0;
-            load_row<T, W>(Pin, i, own);
-#pragma unroll
-            for (int c = 0; c < W; ++c)
-                if (vm & (1u << c)) emx = max(emx, fx_diff(t[c], own[c]));
-            if (!skel[i]) e_loc = (double)emx * (1.0 / kFxOne);
-        }
-        const T y = fx_recip(sum);
-#pragma unroll
-        for (int c = 0; c < W; ++c) t[c] = fx_scale(t[c], y);
-        store_row<T, W>(Pout, i, t);
-    } else {
-        T own[W];
-        load_row<T, W>(Pin, i, own);
-        unsigned vm = vmask[i];
-        T sc = scale[i];
-        T t[W];
-        T sum = T(0), emx = T(0);
-#pragma unroll
-        for (int c = 0; c < W; ++c) {
-            if (vm & (1u << c)) {
-                T d = -sc * acc[c];
-                t[c] = own[c] + d;
-                sum += t[c];
-                emx = fmax(emx, fabs(d));
-            } else {
-                t[c] = T(0);
-            }
-        }
-        const T rs = T(1) / sum;  // one division per row (FP64 issue slots are scarce)
-#pragma unroll
-        for (int c = 0; c < W; ++c) t[c] = (vm & (1u << c)) ? t[c] * rs : T(0);
-        store_row<T, W>(Pout, i, t);
-        if (check && !skel[i]) e_loc = (double)emx;
     }
+    const T rs = T(1) / sum;  // one division per row (FP64 issue slots are scarce)
+#pragma unroll
+    for (int c = 0; c < W; ++c) t[c] = (vm & (1u << c)) ? t[c] * rs : T(0);
+    store_row<T, W>(Pout, i, t);
+    if (check && !skel[i]) e_loc = (double)emx;
 }
 
 template <typename T, int W>
@@ -170,21 +98,40 @@ __global__ void __launch_bounds__(256) smooth_kernel(int n, const int32_t *__res
         for (int c = 0; c < W; ++c) acc[c] = T(0);
         const int32_t *cp = scol + beg + lane;
         const T *vp = sval + beg + lane;
-        int cnt = 0;
         for (int j = 0; j < width; ++j) {
             const unsigned pc = (unsigned)__ldg(cp + (j << 5));
             const T a = __ldg(vp + (j << 5));
             const unsigned m = pc >> kColShift;
             if (m) {
-                ++cnt;
                 T pk[W];
                 load_row<T, W>(Pin, (long)(pc & kColMask), pk);
 #pragma unroll
                 for (int c = 0; c < W; ++c)
-                    if (m & (1u << c)) smooth_mac<T>(acc[c], a, pk[c]);
+                    if (m & (1u << c)) acc[c] = fma(a, pk[c], acc[c]);
             }
         }
-        smooth_epilogue<T, W>(i, acc, cnt, scale, vmask, skel, Pin, Pout, check, e_loc);
+        T own[W];
+        load_row<T, W>(Pin, i, own);
+        unsigned vm = vmask[i];
+        T sc = scale[i];
+        T t[W];
+        T sum = T(0), emx = T(0);
+#pragma unroll
+        for (int c = 0; c < W; ++c) {
+            if (vm & (1u << c)) {
+                T d = -sc * acc[c];
+                t[c] = own[c] + d;
+                sum += t[c];
+                emx = fmax(emx, fabs(d));
+            } else {
+                t[c] = T(0);
+            }
+        }
+        const T rs = T(1) / sum;  // one division per row (FP64 issue slots are scarce)
+#pragma unroll
+        for (int c = 0; c < W; ++c) t[c] = (vm & (1u << c)) ? t[c] * rs : T(0);
+        store_row<T, W>(Pout, i, t);
+        if (check && !skel[i]) e_loc = (double)emx;
     }
     if (check) {
         e_loc = warp_max(e_loc);
@@ -222,7 +169,6 @@ __global__ void __launch_bounds__(256, CAP ? (sizeof(T) == 4 ? 8 : 4) : 1)
         // 32-bit entry indices off the kernel's base pointers (no derived
         // 64-bit pointers held across the loop: registers are the limit)
         const int e0 = beg + lane, e_end = e0 + (width << 5);
-        int cnt = 0;
         unsigned pq[D];
         T aq[D];
 #pragma unroll
@@ -248,15 +194,14 @@ __global__ void __launch_bounds__(256, CAP ? (sizeof(T) == 4 ? 8 : 4) : 1)
             }
             const unsigned m = pc >> kColShift;
             if (m) {
-                ++cnt;
                 T pk[W];
                 load_row<T, W>(Pin, (long)(pc & kColMask), pk);
 #pragma unroll
                 for (int c = 0; c < W; ++c)
-                    if (m & (1u << c)) smooth_mac<T>(acc[c], a, pk[c]);
+                    if (m & (1u << c)) acc[c] = fma(a, pk[c], acc[c]);
             }
         }
-        smooth_epilogue<T, W>(i, acc, cnt, scale, vmask, skel, Pin, Pout, check, e_loc);
+        smooth_epilogue<T, W>(i, acc, scale, vmask, skel, Pin, Pout, check, e_loc);
     }
     if (check) {
         e_loc = warp_max(e_loc);
@@ -346,79 +291,49 @@ __global__ void __launch_bounds__(256) smooth_lanes_kernel(int n, const int32_t 
         for (int c = 0; c < NC; ++c) acc[c] = T(0);
         const int32_t *cp = scol + beg + r;
         const T *vp = sval + beg + r;
-        int cnt = 0;
         for (int j = 0; j < width; ++j) {
             const unsigned pc = (unsigned)__ldg(cp + (j << 5));
             const T a = __ldg(vp + (j << 5));
             const unsigned m = (pc >> (kColShift + c0)) & ((1u << NC) - 1u);
-            cnt += pc >> kColShift ? 1 : 0;
             if (m) {
                 T pk[NC];
                 load_part<T, NC>(Pin + (long)(pc & kColMask) * W + c0, pk);
 #pragma unroll
                 for (int c = 0; c < NC; ++c)
-                    if (m & (1u << c)) smooth_mac<T>(acc[c], a, pk[c]);
+                    if (m & (1u << c)) acc[c] = fma(a, pk[c], acc[c]);
             }
         }
-        if constexpr (kFx<T>) {
-            const unsigned vm = vmask[i];
-            T tl[NC], sum = 0;
+        T own[NC];
+        load_part<T, NC>(Pin + (long)i * W + c0, own);
+        const unsigned vm = vmask[i];
+        const T sc = scale[i];
+        T tl[NC];
+        T emx = T(0);
 #pragma unroll
-            for (int c = 0; c < NC; ++c) {
-                tl[c] = vm & (1u << (c0 + c)) ? acc[c] + (unsigned)(cnt >> 1) : 0ull;
-                sum += tl[c];
+        for (int c = 0; c < NC; ++c) {
+            if (vm & (1u << (c0 + c))) {
+                const T d = -sc * acc[c];
+                tl[c] = own[c] + d;
+                emx = fmax(emx, fabs(d));
+            } else {
+                tl[c] = T(0);
             }
-            T emx = 0;
-            if (check) {
-                T own[NC];
-                load_part<T, NC>(Pin + (long)i * W + c0, own);
-#pragma unroll
-                for (int c = 0; c < NC; ++c)
-                    if (vm & (1u << (c0 + c))) emx = max(emx, fx_diff(tl[c], own[c]));
-            }
-#pragma unroll
-            for (int o = 1; o < L; o <<= 1) {
-                sum += __shfl_xor_sync(gmask, sum, o, L);
-                emx = max(emx, __shfl_xor_sync(gmask, emx, o, L));
-            }
-            const T y = fx_recip(sum);
-#pragma unroll
-            for (int c = 0; c < NC; ++c) tl[c] = fx_scale(tl[c], y);
-            store_part<T, NC>(Pout + (long)i * W + c0, tl);
-            if (check && !skel[i]) e_loc = (double)emx * (1.0 / kFxOne);
-        } else {
-            T own[NC];
-            load_part<T, NC>(Pin + (long)i * W + c0, own);
-            const unsigned vm = vmask[i];
-            const T sc = scale[i];
-            T tl[NC];
-            T emx = T(0);
-#pragma unroll
-            for (int c = 0; c < NC; ++c) {
-                if (vm & (1u << (c0 + c))) {
-                    const T d = -sc * acc[c];
-                    tl[c] = own[c] + d;
-                    emx = fmax(emx, fabs(d));
-                } else {
-                    tl[c] = T(0);
-                }
-            }
-            T sum = T(0);
-#pragma unroll
-            for (int q = 0; q < L; ++q)
-#pragma unroll
-                for (int c = 0; c < NC; ++c) {
-                    const T v = __shfl_sync(gmask, tl[c], q, L);
-                    if (vm & (1u << (q * NC + c))) sum += v;
-                }
-#pragma unroll
-            for (int o = 1; o < L; o <<= 1) emx = fmax(emx, __shfl_xor_sync(gmask, emx, o, L));
-            const T rs = T(1) / sum;
-#pragma unroll
-            for (int c = 0; c < NC; ++c) tl[c] = (vm & (1u << (c0 + c))) ? tl[c] * rs : T(0);
-            store_part<T, NC>(Pout + (long)i * W + c0, tl);
-            if (check && !skel[i]) e_loc = (double)emx;
         }
+        T sum = T(0);
+#pragma unroll
+        for (int q = 0; q < L; ++q)
+#pragma unroll
+            for (int c = 0; c < NC; ++c) {
+                const T v = __shfl_sync(gmask, tl[c], q, L);
+                if (vm & (1u << (q * NC + c))) sum += v;
+            }
+#pragma unroll
+        for (int o = 1; o < L; o <<= 1) emx = fmax(emx, __shfl_xor_sync(gmask, emx, o, L));
+        const T rs = T(1) / sum;
+#pragma unroll
+        for (int c = 0; c < NC; ++c) tl[c] = (vm & (1u << (c0 + c))) ? tl[c] * rs : T(0);
+        store_part<T, NC>(Pout + (long)i * W + c0, tl);
+        if (check && !skel[i]) e_loc = (double)emx;
     }
     if (check) {
         e_loc = warp_max(e_loc);
@@ -427,18 +342,6 @@ __global__ void __launch_bounds__(256) smooth_lanes_kernel(int n, const int32_t 
 }
 
 __global__ void set_value_kernel(double *__restrict__ p, double v) { *p = v; }
-
-// P's valid slots as fixed point in place (0 elsewhere), and back
-__global__ void to_fixed_kernel(int n, int W, const uint8_t *__restrict__ vmask, double *__restrict__ P) {
-    const long t = blockIdx.x * (long)blockDim.x + threadIdx.x;
-    if (t >= (long)n * W) return;
-    const double v = vmask[t / W] >> (t % W) & 1u ? fmin(P[t], 1.0) : 0.0;
-    reinterpret_cast<fx64 *>(P)[t] = (fx64)(v * kFxOne);
-}
-__global__ void from_fixed_kernel(long nW, const fx64 *__restrict__ F, double *__restrict__ P) {
-    const long t = blockIdx.x * (long)blockDim.x + threadIdx.x;
-    if (t < nW) P[t] = (double)F[t] * (1.0 / kFxOne);
-}
 
 __global__ void basis_check_kernel(const unsigned long long *__restrict__ emax_k, double tol, int *__restrict__ done,
                                    double *__restrict__ e_last) {
@@ -503,8 +406,7 @@ static msrsb_status launch_smooth(int variant, int n, const Sell &S, int comp, c
 }
 
 // Alg. 1 loop on one basis family. P (device, [n][W]) holds the initial
-// basis on entry and the result on return (T = fx64: fixed point on entry, FP64
-// on return).
+// basis on entry and the result on return.
 template <typename T>
 msrsb_status basis_loop(int n, int W, const Sell &S, int comp, const T *scale, const uint8_t *vmask,
                         const uint8_t *skel, T *P, const msrsb_basis_opts *o, int *iters_out, double *e_out,
@@ -638,10 +540,7 @@ msrsb_status basis_loop(int n, int W, const Sell &S, int comp, const T *scale, c
         cudaEventDestroy(tev[0]);
         cudaEventDestroy(tev[1]);
     }
-    if constexpr (kFx<T>) {
-        from_fixed_kernel<<<ceil_div((long)n * W, 256), 256, 0, s>>>((long)n * W, iters & 1 ? P2 : P, (double *)P);
-        MSRSB_LAUNCHED("from_fixed_kernel");
-    } else if (iters & 1) MSRSB_CUDA(cudaMemcpyAsync(P, P2, (size_t)n * W * sizeof(T), cudaMemcpyDeviceToDevice, s));
+    if (iters & 1) MSRSB_CUDA(cudaMemcpyAsync(P, P2, (size_t)n * W * sizeof(T), cudaMemcpyDeviceToDevice, s));
     if (iters_out) *iters_out = iters;
     if (e_out) *e_out = h_e;
     dfree(P2, s);
@@ -654,8 +553,6 @@ template msrsb_status basis_loop<double>(int, int, const Sell &, int, const doub
                                          double *, const msrsb_basis_opts *, int *, double *, cudaStream_t);
 template msrsb_status basis_loop<float>(int, int, const Sell &, int, const float *, const uint8_t *, const uint8_t *,
                                         float *, const msrsb_basis_opts *, int *, double *, cudaStream_t);
-template msrsb_status basis_loop<fx64>(int, int, const Sell &, int, const fx64 *, const uint8_t *, const uint8_t *,
-                                       fx64 *, const msrsb_basis_opts *, int *, double *, cudaStream_t);
 
 msrsb_status check_mat(const msrsb_mat *A);
 msrsb_status sell_structure(int n, const int32_t *rowptr, Sell *S, cudaStream_t s, const SellKeep *kept);
@@ -664,54 +561,29 @@ msrsb_status sell_fill(const msrsb_mat *A, int comp, int raw, double omega, cons
                        T *scale, uint8_t *vmask, int write_col, int *n_zero_d, cudaStream_t s);
 void sell_free(Sell *S, cudaStream_t s);
 
-// Filtered operator of component comp (filtered here when raw is set), then the
-// loop; with `fix` FP64 in fixed point where the operator, the relaxation and the
-// initial basis P allow it.
 template <typename T>
-msrsb_status smooth_basis(const msrsb_mat *A, int comp, int raw, const int32_t *p_ids, const uint8_t *skel, int W,
-                          const msrsb_basis_opts *o, T *P, bool fix, int *nzd, int *iters, double *e,
-                          cudaStream_t s) {
-    const int n = A->nrows;
+static msrsb_status build_basis_t(const msrsb_mat *Ahat, const int32_t *p_ids, const uint8_t *skel, int W,
+                                  const msrsb_basis_opts *o, T *P, int *iters, double *e, cudaStream_t s) {
+    int n = Ahat->nrows;
     Sell S;
     T *scale = nullptr;
     uint8_t *vmask = nullptr;
-    SellKeep keep;
-    keep.A = A;
-    keep.comp = comp;
-    keep.raw = raw;
+    SellKeep keep;  // Ahat is given filtered: keep its nonzero entries that share a slot
+    keep.A = Ahat;
+    keep.comp = 0;
+    keep.raw = 0;
     keep.W = W;
     keep.p_ids = p_ids;
-    keep.look = fix && sizeof(T) == 8;
-    if constexpr (sizeof(T) == 8) keep.p_init = fix ? (const double *)P : nullptr;
-    MSRSB_TRY(sell_structure(n, A->rowptr, &S, s, &keep));
+    MSRSB_TRY(sell_structure(n, Ahat->rowptr, &S, s, &keep));
     MSRSB_TRY(dalloc(&scale, n, s));
     MSRSB_TRY(dalloc(&vmask, n, s));
-    msrsb_status st = MSRSB_OK;
-    bool fixed = false;
-    if constexpr (sizeof(T) == 8) {
-        fixed = S.convex && o->omega > 0.0 && o->omega <= kFxMaxOmega && o->max_iter > 0 && (W == 4 || W == 8);
-        if (fixed) {
-            MSRSB_TRY(sell_fill<fx64>(A, comp, raw, o->omega, p_ids, W, &S, (fx64 *)nullptr, vmask, 1, nzd, s));
-            to_fixed_kernel<<<ceil_div((long)n * W, 256), 256, 0, s>>>(n, W, vmask, P);
-            MSRSB_LAUNCHED("to_fixed_kernel");
-            st = basis_loop<fx64>(n, W, S, comp, nullptr, vmask, skel, (fx64 *)P, o, iters, e, s);
-        }
-    }
-    if (!fixed) {
-        MSRSB_TRY(sell_fill<T>(A, comp, raw, o->omega, p_ids, W, &S, scale, vmask, 1, nzd, s));
-        st = basis_loop<T>(n, W, S, comp, scale, vmask, skel, P, o, iters, e, s);
-    }
+    MSRSB_TRY(sell_fill<T>(Ahat, 0, 0, o->omega, p_ids, W, &S, scale, vmask, 1, nullptr, s));
+    msrsb_status st = basis_loop<T>(n, W, S, 0, scale, vmask, skel, P, o, iters, e, s);
     sell_free(&S, s);
     dfree(scale, s);
     dfree(vmask, s);
     return st;
 }
-template msrsb_status smooth_basis<double>(const msrsb_mat *, int, int, const int32_t *, const uint8_t *, int,
-                                           const msrsb_basis_opts *, double *, bool, int *, int *, double *,
-                                           cudaStream_t);
-template msrsb_status smooth_basis<float>(const msrsb_mat *, int, int, const int32_t *, const uint8_t *, int,
-                                          const msrsb_basis_opts *, float *, bool, int *, int *, double *,
-                                          cudaStream_t);
 
 }  // namespace msrsb
 
@@ -727,10 +599,9 @@ extern "C" msrsb_status msrsb_build_basis(const msrsb_mat *Ahat, const int32_t *
     double e = 0.0;
     msrsb_status st;
     if (prec == MSRSB_F64)
-        st = smooth_basis<double>(Ahat, 0, 0, p_ids, skel, W, opts, (double *)p_val, true, nullptr, &it,
-                                  &e, stream);
+        st = build_basis_t<double>(Ahat, p_ids, skel, W, opts, (double *)p_val, &it, &e, stream);
     else if (prec == MSRSB_F32)
-        st = smooth_basis<float>(Ahat, 0, 0, p_ids, skel, W, opts, (float *)p_val, false, nullptr, &it, &e, stream);
+        st = build_basis_t<float>(Ahat, p_ids, skel, W, opts, (float *)p_val, &it, &e, stream);
     else
         return fail(MSRSB_EINVAL, "prec must be MSRSB_F64 or MSRSB_F32");
     if (st != MSRSB_OK) return st;

@@ -173,7 +173,6 @@ struct Sell {
     int n = 0, nslices = 0;
     long entries = 0;
     int32_t *slice_ptr = nullptr;  // [nslices+1] offsets (entries)
-    bool convex = false;           // kept entries of an M-matrix (see sell_kept_width_kernel)
     int32_t *col = nullptr;        // [entries] packed col | mask << 24 (mask unused outside the basis)
     void *val[3] = {nullptr, nullptr, nullptr};
 };
@@ -184,15 +183,7 @@ struct SellKeep {
     const msrsb_mat *A = nullptr;
     int comp = 0, raw = 1, W = 8;
     const int32_t *p_ids = nullptr;
-    bool look = false;               // whether Sell::convex is wanted
-    const double *p_init = nullptr;  // initial basis to look over as well (nullable)
 };
-
-// 64-bit fixed-point values of the restricted smoothing (basis.cu): fractions
-// of 2^63 (P) and 2^64 (weights)
-using fx64 = unsigned long long;
-constexpr double kFxOne = 9223372036854775808.0;   // 1 as a fraction of 2^63
-constexpr double kFxMaxOmega = 0.7;                // relaxation up to which row sums stay above 1/4
 
 // work arrays of the coarse inverse while it runs (see coarse.cu)
 struct CoarseInverseWork {

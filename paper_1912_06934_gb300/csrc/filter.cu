@@ -2,7 +2,6 @@
 // separate-displacement-component (Eq. 20, Remark 2), and the sliced-ELL
 // copy of the filtered operator that the smoothing kernel streams.
 #include "common.cuh"
-#include <type_traits>
 #include <cub/device/device_scan.cuh>
 
 namespace msrsb {
@@ -117,55 +116,23 @@ __device__ __forceinline__ CsrTile csr_tile(int n, int i0, const int32_t *__rest
 // (about half of a rotated anisotropic MPFA stencil), so this halves the
 // operator bytes of every smoothing pass. Width of every 32-row slice (times
 // 32) in kept entries.
-// flag (nullable) is raised unless the smoothing pass is a convex combination of
-// P's rows followed by a rescaling, for which P's entries stay in [0, 1]: every
-// off-diagonal of A_hat <= 0, its diagonal at least the sum of their
-// magnitudes, and the rows of the initial basis (where given) non-negative with
-// sum 1, all within 1e-9.
 template <int W>
 __global__ void __launch_bounds__(kTileRows) sell_kept_width_kernel(
     int n, const int32_t *__restrict__ rowptr, const int32_t *__restrict__ colidx, const double *__restrict__ val,
-    int bdim, int comp, int raw, const int32_t *__restrict__ p_ids, bool vec, int32_t *__restrict__ sizes,
-    const double *__restrict__ p_init, int32_t *__restrict__ flag) {
+    int bdim, int comp, int raw, const int32_t *__restrict__ p_ids, bool vec, int32_t *__restrict__ sizes) {
     __shared__ double s_val[kTileCap];
     __shared__ int32_t s_col[kTileCap];
     const int i0 = blockIdx.x * kTileRows, i = i0 + threadIdx.x;
     const CsrTile A = csr_tile(n, i0, rowptr, colidx, val, bdim, comp, raw, s_col, s_val);
     int len = 0;
-    bool bad = false;
     if (i < n) {
         int32_t my[W];
         load_ids<W>(p_ids, vec, i, my);
-        double off = 0.0, top = 0.0, dia = 0.0;
-        bool has = false;
         for (int e = rowptr[i]; e < rowptr[i + 1]; ++e) {
             const int k = A.col(e);
-            const double a = k == i ? 0.0 : A.offdiag(e);
-            if (flag) {
-                if (k == i) {
-                    dia = raw ? 0.0 : A.value(e);
-                    has = true;
-                }
-                off += a;
-                top = fmax(top, a);
-            }
-            if (k == i || (a != 0.0 && slot_mask<W>(my, p_ids, vec, k) != 0)) ++len;
-        }
-        if (flag) {  // written so that NaN and infinities raise it too
-            const double d = raw ? -off : dia;
-            bad = !(has && top <= 0.0 && d >= 0.0 && d * (1.0 + 1e-9) >= -off && d <= 1e300);
-            if (p_init) {
-                double sum = 0.0, lo = 0.0;
-                for (int c = 0; c < W; ++c)
-                    if (my[c] >= 0) {
-                        sum += p_init[(long)i * W + c];
-                        lo = fmin(lo, p_init[(long)i * W + c]);
-                    }
-                bad = bad || !(lo >= 0.0 && fabs(sum - 1.0) <= 1e-9);
-            }
+            if (k == i || (A.offdiag(e) != 0.0 && slot_mask<W>(my, p_ids, vec, k) != 0)) ++len;
         }
     }
-    if (flag && __any_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) *flag = 1;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) len = max(len, __shfl_xor_sync(0xffffffffu, len, o));
     if ((threadIdx.x & 31) == 0 && i < ((n + 31) & ~31)) sizes[i >> 5] = len * kSell;
@@ -176,8 +143,7 @@ __global__ void __launch_bounds__(kTileRows) sell_kept_width_kernel(
 // holds k and its slot mask. Values: the filtered operator A_hat (component
 // comp); when `raw` is set the filter is applied here, else val already holds
 // A_hat. scale[i] = omega / D_hat_ii, or 0 where D_hat_ii = 0 (row left
-// unchanged). T = fx64: the weights of the pass instead, as fractions of 2^64:
-// omega |a_ik| / D_hat_ii, and 1 - omega on the diagonal (1 where D_hat_ii = 0).
+// unchanged).
 template <typename T, int W>
 __global__ void __launch_bounds__(kTileRows) sell_fill_kernel(
     int n, const int32_t *__restrict__ rowptr, const int32_t *__restrict__ colidx, const double *__restrict__ val,
@@ -218,12 +184,7 @@ __global__ void __launch_bounds__(kTileRows) sell_fill_kernel(
         if (k != i && m == 0) continue;
         const long e = base + (long)j * kSell + lane;
         if (write_col) scol[e] = (int32_t)((unsigned)k | (m << kColShift));
-        if constexpr (std::is_same<T, fx64>::value) {
-            const double w = dh == 0.0 ? (k == i ? 1.0 : 0.0) : (k == i ? 1.0 - omega : -(omega * a) / dh);
-            sval[e] = w >= 1.0 ? ~0ull : (fx64)(w * (2.0 * kFxOne));
-        } else {
-            sval[e] = T(a);
-        }
+        sval[e] = T(a);
         ++j;
     }
     for (; j < width; ++j) {
@@ -231,7 +192,7 @@ __global__ void __launch_bounds__(kTileRows) sell_fill_kernel(
         if (write_col) scol[e] = i;  // mask 0: contributes nothing
         sval[e] = T(0);
     }
-    if constexpr (!std::is_same<T, fx64>::value) scale[i] = dh != 0.0 ? T(omega / dh) : T(0);
+    scale[i] = dh != 0.0 ? T(omega / dh) : T(0);
     if (vmask) {
         unsigned v = 0;
         for (int c = 0; c < W; ++c)
@@ -245,22 +206,19 @@ __global__ void __launch_bounds__(kTileRows) sell_fill_kernel(
 // (kept == nullptr), or of the entries the smoothing kernel keeps for
 // component kept->comp (see sell_kept_width_kernel).
 msrsb_status sell_structure(int n, const int32_t *rowptr, Sell *S, cudaStream_t s, const SellKeep *kept) {
+    if (kept && kept->W != 4 && kept->W != 8) return fail(MSRSB_EINVAL, "W must be 4 or 8 (got %d)", kept->W);
     S->n = n;
     S->nslices = ceil_div(n, kSell);
     int32_t *sizes = nullptr;
     MSRSB_TRY(dalloc(&sizes, S->nslices + 1, s));
-    MSRSB_TRY(dalloc(&S->slice_ptr, S->nslices + 2, s));  // offsets, then the flag
+    MSRSB_TRY(dalloc(&S->slice_ptr, S->nslices + 1, s));
     MSRSB_CUDA(cudaMemsetAsync(sizes, 0, (S->nslices + 1) * sizeof(int32_t), s));
-    int32_t *flag = S->slice_ptr + S->nslices + 1;
-    MSRSB_CUDA(cudaMemsetAsync(flag, 0, sizeof(int32_t), s));
     if (kept) {
         const msrsb_mat *A = kept->A;
-        if (kept->W != 4 && kept->W != 8) return fail(MSRSB_EINVAL, "W must be 4 or 8 (got %d)", kept->W);
         const bool vec = ((uintptr_t)kept->p_ids & 15) == 0;
         auto kernel = kept->W == 8 ? sell_kept_width_kernel<8> : sell_kept_width_kernel<4>;
         kernel<<<ceil_div((long)S->nslices * kSell, kTileRows), kTileRows, 0, s>>>(
-            n, A->rowptr, A->colidx, A->val, A->bdim, kept->comp, kept->raw, kept->p_ids, vec, sizes, kept->p_init,
-            kept->look ? flag : nullptr);
+            n, A->rowptr, A->colidx, A->val, A->bdim, kept->comp, kept->raw, kept->p_ids, vec, sizes);
         MSRSB_LAUNCHED("sell_kept_width_kernel");
     } else {
         sell_width_kernel<<<ceil_div((long)S->nslices * kSell, 256), 256, 0, s>>>(n, rowptr, sizes);
@@ -271,10 +229,9 @@ msrsb_status sell_structure(int n, const int32_t *rowptr, Sell *S, cudaStream_t 
     void *tbuf = nullptr;
     MSRSB_TRY(dalloc((char **)&tbuf, tmp, s));
     MSRSB_CUDA(cub::DeviceScan::ExclusiveSum(tbuf, tmp, sizes, S->slice_ptr, S->nslices + 1, s));
-    int32_t total[2] = {0, 0};
-    MSRSB_TRY(read_back(total, S->slice_ptr + S->nslices, 2 * sizeof(int32_t), s));
-    S->entries = total[0];
-    S->convex = kept && kept->look && total[1] == 0;
+    int32_t total = 0;
+    MSRSB_TRY(read_back(&total, S->slice_ptr + S->nslices, sizeof(int32_t), s));
+    S->entries = total;
     dfree(tbuf, s);
     dfree(sizes, s);
     MSRSB_TRY(dalloc(&S->col, S->entries, s));
@@ -284,10 +241,10 @@ msrsb_status sell_structure(int n, const int32_t *rowptr, Sell *S, cudaStream_t 
 template <typename T>
 msrsb_status sell_fill(const msrsb_mat *A, int comp, int raw, double omega, const int32_t *p_ids, int W, Sell *S,
                        T *scale, uint8_t *vmask, int write_col, int *n_zero_d, cudaStream_t s) {
+    if (W != 4 && W != 8) return fail(MSRSB_EINVAL, "W must be 4 or 8 (got %d)", W);
     T *v = nullptr;
     MSRSB_TRY(dalloc(&v, S->entries, s));
     S->val[comp] = v;
-    if (W != 4 && W != 8) return fail(MSRSB_EINVAL, "W must be 4 or 8 (got %d)", W);
     const bool vec = ((uintptr_t)p_ids & 15) == 0;
     auto kernel = W == 8 ? sell_fill_kernel<T, 8> : sell_fill_kernel<T, 4>;
     kernel<<<ceil_div((long)S->nslices * kSell, kTileRows), kTileRows, 0, s>>>(
@@ -300,8 +257,6 @@ template msrsb_status sell_fill<double>(const msrsb_mat *, int, int, double, con
                                         uint8_t *, int, int *, cudaStream_t);
 template msrsb_status sell_fill<float>(const msrsb_mat *, int, int, double, const int32_t *, int, Sell *, float *,
                                        uint8_t *, int, int *, cudaStream_t);
-template msrsb_status sell_fill<fx64>(const msrsb_mat *, int, int, double, const int32_t *, int, Sell *, fx64 *,
-                                      uint8_t *, int, int *, cudaStream_t);
 
 void sell_free(Sell *S, cudaStream_t s) {
     dfree(S->slice_ptr, s);
