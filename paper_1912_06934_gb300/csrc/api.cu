@@ -742,7 +742,7 @@ __global__ void givens_kernel(int m, int j, double *__restrict__ kh) {
 // unknown is known, thread i < c removes its column's entry from row i. A block a
 // right-hand side. The 2k columns are a chain: what a column costs is an unknown
 // (a multiplication by its reciprocal diagonal, formed for all unknowns beforehand, and
-// the correction by the remainder that rounds the quotient), one barrier and a row's
+// the correction by the remainder that rounds the quotient, Markstein's), one barrier and a row's
 // update; the columns are loaded four ahead. (With a division and the column's load on
 // the chain 70 us for k = 32, 34 now with the launch.)
 constexpr int kHessThreads = 256;
