@@ -164,7 +164,9 @@ __device__ __forceinline__ unsigned plane_top(long long key, int row) {
 //    other CTAs are independent of one another.
 // Three pivot-column buffers: a CTA arrives for column kk + 1 when it has done
 // with step kk - 1, so the column that a passed barrier lets the next owner
-// overwrite is two steps old. The arithmetic and its order are those of the
+// overwrite is two steps old. Every arrive releases, the readers' too: what orders
+// their reads before that store is the barrier (a relaxed arrive of the CTAs that
+// only read gave the same times). The arithmetic and its order are those of the
 // plain elimination. Measured, both factorisation launches: 128^3 (9 dependent
 // planes of 256) 11.2 -> 4.9 ms, 48^3 elasticity (5 of 243) 5.6 -> 2.7 ms, 64^3 (5
 // of 64, with the explicit inverse) 0.79 -> 0.61 ms; of a step's 4,200 cycles at

@@ -21,9 +21,10 @@
 // lines still to come take each finished line's contributions at once instead
 // of all of them at their turn.
 // Measured against one thread per point with column indices beside the values
-// and every warp of the CTA in every scan: solves of 64^3 in FP64 10.6 -> 6.9
-// ms, of 128^3 in FP32 33.3 -> 27.2, 8 lockstep right-hand sides of 80^3 in FP32
-// 46.2 -> 36.3. A launch inside a solve now takes 4.9 us at 64^3 (FP32), 8.2
+// and every warp of the CTA in every scan, the rest of the solve as it was then
+// (whole calls): solves of 64^3 in FP64 10.6 -> 6.9 ms, of 128^3 in FP32 33.3 ->
+// 27.2, 8 lockstep right-hand sides of 80^3 in FP32 46.2 -> 36.3. A launch inside a
+// solve now takes 4.9 us at 64^3 (FP32), 8.2
 // (FP64), 19.4 at 128^3 (FP32; 36 MB of coefficients, 5.4 us at the copy rate).
 #include "common.cuh"
 #include "lines.cuh"
@@ -407,8 +408,8 @@ static msrsb_status lines_sweeps(const msrsb_handle *h, int k, const Cols<T> &ry
         // Up to two CTAs per SM the off-block part is staged ahead of the
         // wait. Beyond, a launch has several waves, only the first of which
         // gains by that, and the shared memory costs CTAs in flight: read
-        // where it is used (128^3 FP32 solve 24.4 ms with it staged, 22.6
-        // without; 64^3 FP32, one wave: 7.86 and 7.94). So it is on FP64
+        // where it is used (128^3 FP32 solve, whole call: 24.5 ms with it staged,
+        // 22.5 without; 64^3 FP32, one wave: 1 % less with it). So it is on FP64
         // lines too wide for the shared memory.
         C.stage = nb * ceil_div(k, NV) <= kSweepStageCtas && (size_t)(nlin * (C.ng[dir] > back ? C.ng[dir] : back) + gin) * L.nx * 16 + vals <= kSweepSmemMax;
         C.room = C.stage && C.ng[dir] > back ? C.ng[dir] : back;
